@@ -106,6 +106,23 @@ __device__ __forceinline__ float translate_x(uint64_t w, const Norm &nm) {
     return __double2float_rn(__dmul_rn(__dsub_rn(k, nm.lo_val), nm.scale));
 }
 
+// translate_x of a key held in W: the same value. A 32-bit key whose normaliser fits 32 bits takes
+// its difference and its one rounding in 32-bit arithmetic (the 64-bit conversion is several
+// instructions on a slow pipe; the difference is the same integer, so the rounding is the same).
+template <typename W> __device__ __forceinline__ float translate_key(W w, const Norm &nm) {
+    if constexpr (sizeof(W) == 4) {
+        const bool ob = nm.translate == NNSORT_TRANSLATE_ORDBITS || nm.dtype == NNSORT_U32;
+        if (ob && (nm.lo_bits >> 32) == 0) {
+            const uint32_t lo = (uint32_t)nm.lo_bits;
+            uint32_t u = w;
+            if (nm.dtype == NNSORT_F32) u = (w & 0x80000000u) ? ~w : (w | 0x80000000u);
+            const float d = (u >= lo) ? __uint2float_rn(u - lo) : -__uint2float_rn(lo - u);
+            return __fmul_rn(d, nm.scale_f);
+        }
+    }
+    return translate_x(word64(w), nm);
+}
+
 __device__ __forceinline__ float relu_f(float v) { return v > 0.0f ? v : 0.0f; }
 
 // Two binary32 lanes per instruction (packed FP32 on sm_100 and later): each lane is rounded exactly
@@ -189,7 +206,9 @@ __device__ __forceinline__ uint32_t slot_of(float y, float nm_hi, float nm_lo, u
     const float f = floorf(p);
     const float r = __fadd_rn(__fsub_rn(p, f), e);
     const float g = floorf(__fadd_rn(r, 0.5f));
-    long long s = (long long)f + (long long)g;
+    // positions stay below 2^32 - 512 (whole buckets of at least 2^9 positions below 2^32), so both
+    // parts convert exactly in 32 bits; only their sum needs the 33rd
+    long long s = (long long)__float2uint_rz(f) + (long long)__float2int_rz(g);
     if (s < 0) s = 0;
     if ((unsigned long long)s > L - 1) s = (long long)(L - 1);
     return (uint32_t)s;

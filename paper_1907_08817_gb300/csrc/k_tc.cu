@@ -445,7 +445,7 @@ __global__ void __launch_bounds__(NG * TC_THREADS, 1) k_predict_bf16_mg(PredictA
                 pre_st = st2;
             }
         }
-        const float x = valid ? translate_x(wv, sg.norm) : 0.0f;
+        const float x = valid ? translate_key<W>((W)wv, sg.norm) : 0.0f;
         const unsigned long long xx = pk2(x, x);
 #pragma unroll
         for (int j0 = 0; j0 < H; j0 += 8) {
