@@ -161,6 +161,37 @@ struct Carve {
 
 void nns::note_launch(int kernels) { g_launches.fetch_add((unsigned long long)kernels); }
 
+namespace {
+std::map<int, cudaMemPool_t> g_pools;  // one per device, made on first use (guarded by g_mu)
+}
+cudaError_t nns::pool_alloc(void **p, size_t bytes, cudaStream_t s) {
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    cudaMemPool_t pool;
+    {
+        std::lock_guard<std::mutex> lk(g_mu);
+        auto it = g_pools.find(dev);
+        if (it == g_pools.end()) {
+            cudaMemPoolProps pp;
+            std::memset(&pp, 0, sizeof(pp));
+            pp.allocType = cudaMemAllocationTypePinned;
+            pp.location.type = cudaMemLocationTypeDevice;
+            pp.location.id = dev;
+            cudaMemPool_t np;
+            if ((e = cudaMemPoolCreate(&np, &pp)) != cudaSuccess) return e;
+            uint64_t keep = POOL_KEEP;
+            if ((e = cudaMemPoolSetAttribute(np, cudaMemPoolAttrReleaseThreshold, &keep)) != cudaSuccess) {
+                cudaMemPoolDestroy(np);
+                return e;
+            }
+            it = g_pools.emplace(dev, np).first;
+        }
+        pool = it->second;
+    }
+    return cudaMallocFromPoolAsync(p, bytes, pool, s);
+}
+
 // ---------------------------------------------------------------------------------------------
 // models
 namespace nns {
@@ -325,6 +356,12 @@ int nnsort_release(void) {
         delete w;
     }
     g_ws.clear();
+    // free memory of the pools goes back to the device; blocks in use (a call in another thread) stay
+    for (auto &kv : g_pools) {
+        cudaSetDevice(kv.first);
+        cudaDeviceSynchronize();
+        cudaMemPoolTrimTo(kv.second, 0);
+    }
     cudaSetDevice(cur);
     return NNSORT_OK;
 }
@@ -1389,7 +1426,7 @@ int nnsort_train_batch(void *const *d_keys, const uint64_t *ns, int32_t count, i
         std::memcpy(host.data() + off_c + (size_t)(steps + t) * 4, &c2, 4);
     }
     unsigned char *dev = nullptr;
-    CK(cudaMallocAsync((void **)&dev, total, s));
+    CK(pool_alloc((void **)&dev, total, s));
     // the trained parameters stay where the kernel writes them: one device block that the models
     // share (each model's padded parameters are a slice; the block is freed with the last model)
     float *dpar = nullptr;
@@ -1483,117 +1520,47 @@ int nnsort_train(const void *d_keys, uint64_t n, int32_t dtype, const nnsort_tra
     if (op) o = *op; else nnsort_default_train_opts(&o);
     if (!out || !d_keys || n == 0 || !dtype_ok(dtype) || !arch_ok(o.layers, o.h1, o.h2)) return NNSORT_E_INVALID_ARG;
     if (o.sample_n == 0 || o.loss < 0 || o.loss > 1) return NNSORT_E_INVALID_ARG;
-    const uint64_t S = o.sample_n;
-    const uint64_t B = o.batch ? o.batch : S;
-    const PadArch pa = pad_arch(o.layers, o.h1, o.h2);
-    const size_t Pp = padded_param_count(pa), P = param_count(o.layers, o.h1, o.h2);
-    const int blocks = train_grad_blocks(pa, B);
-    uint32_t *terr = train_err_word();
-    if (!terr) return NNSORT_E_CUDA;
-    // device buffers for this call (separate from the per-stream arena used by sampling)
-    float *dx = nullptr;
-    const uint32_t nst = std::max<uint32_t>(o.steps, 1);
-    const size_t fl = S * 2 + Pp * 5 + (size_t)blocks * Pp + blocks + nst + 2 * (size_t)nst + 64;
-    CK(cudaMallocAsync((void **)&dx, fl * sizeof(float), s));
-    float *dlab = dx + S, *dp = dlab + S, *dm = dp + Pp, *dv = dm + Pp, *dg = dv + Pp;
-    float *dmask = dg + Pp;
-    float *dpart = dmask + Pp, *dlp = dpart + (size_t)blocks * Pp, *dloss = dlp + blocks;
-    float *dc12 = dloss + nst;                                           // [2 * steps]
-    unsigned int *dcount = reinterpret_cast<unsigned int *>(dc12 + 2 * (size_t)nst);  // [1]
-    nnsort_model_desc d;
-    int rc = nnsort_sample_labels(d_keys, n, dtype, S, o.seed, o.translate, &d, dx, dlab, nullptr, s);
-    if (rc) { cudaFreeAsync(dx, s); return rc; }
-    d.layers = o.layers; d.h1 = o.h1; d.h2 = o.h2;
-    std::vector<float> p0(P);
-    init_params_host(o.layers, o.h1, o.h2, o.seed, p0.data());
-    std::vector<float> mask;
-    if (o.monotone) {
-        // sign structure: layer-1 unit j keeps sign s_j of W1_j; with two hidden layers output
-        // unit k keeps sign q_k of W3_k and W2_kj carries s_j q_k; with one, W3_j carries s_j
-        std::vector<float> sg(P, 0.0f);
-        for (int j = 0; j < o.h1; ++j) sg[j] = p0[j] >= 0.0f ? 1.0f : -1.0f;
-        if (o.layers == 1) {
-            for (int j = 0; j < o.h1; ++j) sg[2 * o.h1 + j] = sg[j];
-        } else {
-            const size_t w2 = 2 * (size_t)o.h1, w3 = w2 + (size_t)o.h2 * o.h1 + o.h2;
-            for (int k = 0; k < o.h2; ++k) {
-                const float q = p0[w3 + k] >= 0.0f ? 1.0f : -1.0f;
-                sg[w3 + k] = q;
-                for (int j = 0; j < o.h1; ++j) sg[w2 + (size_t)k * o.h1 + j] = sg[j] * q;
-            }
-        }
-        for (size_t u = 0; u < P; ++u)
-            if (sg[u] != 0.0f) p0[u] = sg[u] * std::fabs(p0[u]);
-        mask = to_padded(d, pa, sg.data());
-        CK(cudaMemcpyAsync(dmask, mask.data(), Pp * sizeof(float), cudaMemcpyHostToDevice, s));
-    }
-    const std::vector<float> pp = to_padded(d, pa, p0.data());
-    CK(cudaMemcpyAsync(dp, pp.data(), Pp * sizeof(float), cudaMemcpyHostToDevice, s));
-    CK(cudaMemsetAsync(dm, 0, 2 * Pp * sizeof(float), s));
-    TrainStepArgs t{};
-    t.params = dp; t.m = dm; t.v = dv; t.grad = dg; t.partials = dpart; t.loss_partials = dlp;
-    t.loss_out = dloss; t.x = dx; t.label = dlab; t.S = S; t.batch = o.batch;
-    t.batch_seed = rng_h(o.seed, TAG_BATCH); t.loss = o.loss; t.delta = o.huber_delta;
-    t.lr = o.lr; t.b1 = o.beta1; t.b2 = o.beta2; t.eps = o.adam_eps; t.P = Pp;
-    t.mask = o.monotone ? dmask : nullptr;
-    CK(cudaMemsetAsync(terr, 0, sizeof(uint32_t), s));
-    if (pa.layers == 2 && pa.h1 == 64) {
-        // every step in one cooperative launch (its blocks meet twice per step)
-        std::vector<float> c12(2 * (size_t)nst);
-        for (uint32_t k = 0; k < o.steps; ++k) {
-            c12[k] = (float)(1.0 - std::pow((double)o.beta1, (double)(k + 1)));
-            c12[o.steps + k] = (float)(1.0 - std::pow((double)o.beta2, (double)(k + 1)));
-        }
-        CK(cudaMemcpyAsync(dc12, c12.data(), c12.size() * sizeof(float), cudaMemcpyHostToDevice, s));
-        CK(cudaMemsetAsync(dcount, 0, sizeof(unsigned int), s));
-        CK(launch_train_tc64(t, o.steps, dc12, dcount, s));
-    } else {
-        for (uint32_t k = 0; k < o.steps; ++k) {
-            t.step = (int)k;
-            CK(launch_train_step(pa, t, s));
-        }
-    }
-    std::vector<float> hpp(Pp);
-    CK(cudaMemcpyAsync(hpp.data(), dp, Pp * sizeof(float), cudaMemcpyDeviceToHost, s));
-    std::vector<float> hl(std::max<uint32_t>(o.steps, 1));
-    if (o.steps) CK(cudaMemcpyAsync(hl.data(), dloss, o.steps * sizeof(float), cudaMemcpyDeviceToHost, s));
-    uint32_t herr = 0;
-    CK(cudaMemcpyAsync(&herr, terr, sizeof(uint32_t), cudaMemcpyDeviceToHost, s));
-    CK(cudaStreamSynchronize(s));
-    cudaFreeAsync(dx, s);
-    if (herr & ERR_TIMEOUT) return NNSORT_E_TIMEOUT;
-    if (h_loss) std::memcpy(h_loss, hl.data(), o.steps * sizeof(float));
-    std::vector<float> up(P);
-    for (size_t u = 0; u < P; ++u) up[u] = hpp[pad_index(o.layers, o.h1, o.h2, pa, u)];
-    return nnsort_model_create(&d, up.data(), out);
+    nnsort_model *f = nullptr;
+    int one = NNSORT_OK;
+    const int rc = nnsort_train_models(&d_keys, &n, 1, dtype, o, &o.sample_n, &o.seed, &f, &one, h_loss, s);
+    if (rc || one) return rc ? rc : one;
+    *out = f;
+    return NNSORT_OK;
 }
 
 // ---- explicit forward / backward (autograd)
-static int with_padded(const float *d_params, int layers, int h1, int h2, cudaStream_t s,
-                       float **dpad, PadArch *pa, size_t extra_floats, float **extra) {
+// Scratch of one call and, for widths that the kernels pad, the padded parameters at its start
+// (*pp; parameters that need no padding are used where they are, and without scratch *buf stays null)
+static int with_padded(const float *d_params, int layers, int h1, int h2, cudaStream_t s, float **buf,
+                       const float **pp, PadArch *pa, size_t extra_floats, float **extra) {
     if (!arch_ok(layers, h1, h2) || !d_params) return NNSORT_E_INVALID_ARG;
     *pa = pad_arch(layers, h1, h2);
     const size_t Pp = padded_param_count(*pa), P = param_count(layers, h1, h2);
-    float *buf = nullptr;
-    CK(cudaMallocAsync((void **)&buf, (Pp + extra_floats) * sizeof(float), s));
-    CK(cudaMemsetAsync(buf, 0, Pp * sizeof(float), s));
-    k_pad<<<(unsigned)((P + 255) / 256), 256, 0, s>>>(d_params, buf, layers, h1, h2, pa->h1, pa->h2, P);
-    CK(cudaGetLastError());
-    note_launch(1);
-    *dpad = buf;
-    *extra = buf + Pp;
+    const size_t pad = Pp == P ? 0 : Pp;
+    *buf = nullptr;
+    if (pad + extra_floats) CK(pool_alloc((void **)buf, (pad + extra_floats) * sizeof(float), s));
+    *pp = d_params;
+    if (pad) {
+        CK(cudaMemsetAsync(*buf, 0, Pp * sizeof(float), s));
+        k_pad<<<(unsigned)((P + 255) / 256), 256, 0, s>>>(d_params, *buf, layers, h1, h2, pa->h1, pa->h2, P);
+        CK(cudaGetLastError());
+        note_launch(1);
+        *pp = *buf;
+    }
+    *extra = *buf + pad;
     return NNSORT_OK;
 }
 
 int nnsort_mlp_forward(const float *d_params, int32_t layers, int32_t h1, int32_t h2, const float *d_x,
                        uint64_t n, float *d_y, cudaStream_t s) {
     if ((n && (!d_x || !d_y))) return NNSORT_E_INVALID_ARG;
-    float *pp = nullptr, *ex = nullptr;
+    float *buf = nullptr, *ex = nullptr;
+    const float *pp = nullptr;
     PadArch pa;
-    int rc = with_padded(d_params, layers, h1, h2, s, &pp, &pa, 0, &ex);
+    int rc = with_padded(d_params, layers, h1, h2, s, &buf, &pp, &pa, 0, &ex);
     if (rc) return rc;
     CK(launch_mlp_forward(pa, pp, d_x, n, d_y, s));
-    CK(cudaFreeAsync(pp, s));
+    if (buf) CK(cudaFreeAsync(buf, s));
     return NNSORT_OK;
 }
 
@@ -1604,23 +1571,28 @@ static int backward_common(const float *d_params, int layers, int h1, int h2, co
     PadArch pa = pad_arch(layers, h1, h2);
     const size_t Pp = padded_param_count(pa), P = param_count(layers, h1, h2);
     const int blocks = train_grad_blocks(pa, n);
-    float *pp = nullptr, *ex = nullptr;
-    int rc = with_padded(d_params, layers, h1, h2, s, &pp, &pa, (size_t)blocks * Pp + blocks + Pp + 4, &ex);
+    float *buf = nullptr, *ex = nullptr;
+    const float *pp = nullptr;
+    int rc = with_padded(d_params, layers, h1, h2, s, &buf, &pp, &pa,
+                         (size_t)blocks * Pp + blocks + (Pp == P ? 0 : Pp), &ex);
     if (rc) return rc;
-    float *part = ex, *lp = part + (size_t)blocks * Pp, *gpad = lp + blocks;
+    float *part = ex, *lp = part + (size_t)blocks * Pp;
+    float *gpad = Pp == P ? d_gparams : lp + blocks;
     if (n == 0) {
         CK(cudaMemsetAsync(d_gparams, 0, P * sizeof(float), s));
         if (d_loss) CK(cudaMemsetAsync(d_loss, 0, sizeof(float), s));
-        CK(cudaFreeAsync(pp, s));
+        CK(cudaFreeAsync(buf, s));
         return NNSORT_OK;
     }
     int nb = 0;
     CK(launch_mlp_backward(pa, pp, d_x, d_gy, d_label, n, mode, loss, delta, part, lp, d_gx, s, &nb));
     CK(launch_reduce_partials(part, nb, Pp, gpad, lp, d_loss, 1.0f / (float)n, s));
-    k_unpad<<<(unsigned)((P + 255) / 256), 256, 0, s>>>(gpad, d_gparams, layers, h1, h2, pa.h1, pa.h2, P);
-    CK(cudaGetLastError());
-    note_launch(1);
-    CK(cudaFreeAsync(pp, s));
+    if (Pp != P) {
+        k_unpad<<<(unsigned)((P + 255) / 256), 256, 0, s>>>(gpad, d_gparams, layers, h1, h2, pa.h1, pa.h2, P);
+        CK(cudaGetLastError());
+        note_launch(1);
+    }
+    CK(cudaFreeAsync(buf, s));
     return NNSORT_OK;
 }
 
@@ -1640,3 +1612,200 @@ int nnsort_mlp_loss_grad(const float *d_params, int32_t layers, int32_t h1, int3
 }
 
 }  // extern "C"
+
+// sign structure of the monotone option: layer-1 unit j keeps sign s_j of W1_j; with two hidden layers
+// output unit k keeps sign q_k of W3_k and W2_kj carries s_j q_k; with one, W3_j carries s_j. Applied to
+// the initial parameters p0; returns the signs.
+static std::vector<float> monotone_signs(const nnsort_train_opts &o, std::vector<float> &p0) {
+    std::vector<float> sg(p0.size(), 0.0f);
+    for (int j = 0; j < o.h1; ++j) sg[j] = p0[j] >= 0.0f ? 1.0f : -1.0f;
+    if (o.layers == 1) {
+        for (int j = 0; j < o.h1; ++j) sg[2 * o.h1 + j] = sg[j];
+    } else {
+        const size_t w2 = 2 * (size_t)o.h1, w3 = w2 + (size_t)o.h2 * o.h1 + o.h2;
+        for (int k = 0; k < o.h2; ++k) {
+            const float q = p0[w3 + k] >= 0.0f ? 1.0f : -1.0f;
+            sg[w3 + k] = q;
+            for (int j = 0; j < o.h1; ++j) sg[w2 + (size_t)k * o.h1 + j] = sg[j] * q;
+        }
+    }
+    for (size_t u = 0; u < p0.size(); ++u)
+        if (sg[u] != 0.0f) p0[u] = sg[u] * std::fabs(p0[u]);
+    return sg;
+}
+
+int nnsort_train_models(const void *const *d_keys, const uint64_t *ns, uint32_t count, int32_t dtype,
+                        const nnsort_train_opts &o, const uint64_t *S, const uint64_t *seeds,
+                        nnsort_model **out, int *rcs, float *h_loss, cudaStream_t s) {
+    if (count == 0) return NNSORT_OK;
+    if (count > 65535u || !dtype_ok(dtype) || !arch_ok(o.layers, o.h1, o.h2) || o.loss < 0 || o.loss > 1)
+        return NNSORT_E_INVALID_ARG;
+    const PadArch pa = pad_arch(o.layers, o.h1, o.h2);
+    const size_t Pp = padded_param_count(pa), P = param_count(o.layers, o.h1, o.h2);
+    const int kb = key_bytes_of(dtype);
+    uint64_t total = 0, max_S = 0, max_B = 0;
+    for (uint32_t j = 0; j < count; ++j) {
+        out[j] = nullptr;
+        rcs[j] = NNSORT_OK;
+        if (S[j] >= 0xFFFFFFFFull) return NNSORT_E_INVALID_ARG;
+        total += S[j];
+        max_S = std::max(max_S, S[j]);
+        max_B = std::max<uint64_t>(max_B, o.batch ? o.batch : S[j]);
+    }
+    if (total >= 0xFFFFFFFFull) return NNSORT_E_INVALID_ARG;
+    const bool tc64 = pa.layers == 2 && pa.h1 == 64;
+    const bool cluster = train_cluster_ok(pa, max_B);
+    uint32_t *terr = train_err_word();
+    if (!terr) return NNSORT_E_CUDA;
+    Workspace *w = nullptr;
+    int rc = get_ws(s, &w);
+    if (rc) return rc;
+    if ((rc = ensure_part(w, total, s))) return rc;
+    // one device block: tables and parameters (uploaded together), then what the kernels make; the
+    // parameters, normalisers, losses and the error word lie together and come back in one copy
+    std::vector<uint32_t> blocks(count);
+    size_t rows = 0;
+    for (uint32_t j = 0; j < count; ++j) {
+        blocks[j] = (uint32_t)train_grad_blocks(pa, o.batch ? o.batch : S[j]);
+        rows += blocks[j];
+    }
+    const size_t steps = o.steps;
+    Carve c;
+    struct {
+        TrainJob *jobs; float *c12, *mask, *params; Norm *norms; float *loss; uint32_t *err; float *mv;
+        unsigned int *meet; void *key[2]; uint32_t *grp[2]; float *x, *label, *part, *lpart;
+    } L;
+    size_t up_end = 0, back_end = 0;
+    auto lay = [&](unsigned char *base) {
+        c = Carve();
+        c.base = base;
+        L.jobs = c.take<TrainJob>(count);
+        L.c12 = c.take<float>(2 * steps);
+        L.mask = c.take<float>(o.monotone ? count * Pp : 0);
+        L.params = c.take<float>(count * Pp);
+        up_end = c.off;
+        L.norms = c.take<Norm>(count);
+        L.loss = c.take<float>(count * steps);
+        L.err = c.take<uint32_t>(count);  // a word per model: a NaN fails its own model only
+        back_end = c.off;
+        L.mv = c.take<float>(2 * count * Pp);
+        L.meet = c.take<unsigned int>(1);
+        for (int i = 0; i < 2; ++i) {
+            L.key[i] = c.take<unsigned char>(total * kb);
+            L.grp[i] = count > 1 ? c.take<uint32_t>(total) : nullptr;
+        }
+        L.x = c.take<float>(total);
+        L.label = c.take<float>(total);
+        L.part = cluster ? nullptr : c.take<float>(rows * Pp);
+        L.lpart = cluster ? nullptr : c.take<float>(rows);
+    };
+    lay(nullptr);
+    unsigned char *dev = nullptr;
+    cudaError_t e = pool_alloc((void **)&dev, c.off, s);
+    if (e != cudaSuccess) {
+        g_last_cuda = (int)e;
+        cudaGetLastError();
+        return e == cudaErrorMemoryAllocation ? NNSORT_E_OOM : NNSORT_E_CUDA;
+    }
+    struct Free {
+        void *p; cudaStream_t s;
+        ~Free() { cudaFreeAsync(p, s); }
+    } guard{dev, s};
+    lay(dev);
+    const size_t off_par = (size_t)((unsigned char *)L.params - dev);
+    std::vector<unsigned char> host(back_end, 0);
+    auto hp = [&](const void *d) { return host.data() + ((const unsigned char *)d - dev); };
+    float *hc = reinterpret_cast<float *>(hp(L.c12));
+    for (uint32_t k = 0; k < steps; ++k) {
+        hc[k] = (float)(1.0 - std::pow((double)o.beta1, (double)(k + 1)));
+        hc[steps + k] = (float)(1.0 - std::pow((double)o.beta2, (double)(k + 1)));
+    }
+    nnsort_model_desc d;
+    std::memset(&d, 0, sizeof(d));
+    d.dtype = dtype;
+    d.translate = o.translate;
+    d.layers = o.layers; d.h1 = o.h1; d.h2 = o.h2;
+    TrainJob *hj = reinterpret_cast<TrainJob *>(hp(L.jobs));
+    std::vector<float> p0(P);
+    uint64_t off = 0;
+    size_t row = 0;
+    for (uint32_t j = 0; j < count; ++j) {
+        init_params_host(o.layers, o.h1, o.h2, seeds[j], p0.data());
+        if (o.monotone) {
+            const std::vector<float> m = to_padded(d, pa, monotone_signs(o, p0).data());
+            std::memcpy(hp(L.mask + j * Pp), m.data(), Pp * sizeof(float));
+        }
+        const std::vector<float> pp = to_padded(d, pa, p0.data());
+        std::memcpy(hp(L.params + j * Pp), pp.data(), Pp * sizeof(float));
+        TrainJob q{};
+        q.keys = d_keys[j]; q.n = ns[j]; q.S = S[j]; q.off = off;
+        q.sseed = rng_h(seeds[j], TAG_SAMPLE);
+        q.bseed = rng_h(seeds[j], TAG_BATCH);
+        q.B = o.batch ? o.batch : S[j];
+        q.inv_n = 1.0f / (float)q.B;
+        q.blocks = blocks[j];
+        q.params = L.params + j * Pp;
+        q.m = L.mv + 2 * j * Pp; q.v = q.m + Pp;
+        q.mask = o.monotone ? L.mask + j * Pp : nullptr;
+        q.x = L.x + off; q.label = L.label + off;
+        q.partials = cluster ? nullptr : L.part + row * Pp;
+        q.loss_partials = cluster ? nullptr : L.lpart + row;
+        q.loss_out = L.loss + j * steps;
+        hj[j] = q;
+        off += S[j];
+        row += blocks[j];
+    }
+    CK(cudaMemcpyAsync(dev, host.data(), up_end, cudaMemcpyHostToDevice, s));
+    CK(cudaMemsetAsync(L.err, 0, (size_t)((unsigned char *)(L.meet + 1) - (unsigned char *)L.err), s));
+    CK(cudaMemsetAsync(terr, 0, sizeof(uint32_t), s));
+    // samples, sorted by key and then by model; inputs, labels and normalisers
+    CK(launch_sample_jobs(L.jobs, count, max_S, kb, dtype, L.key[0], L.grp[0], L.err, s));
+    void *const K[2] = {L.key[0], L.key[1]};
+    uint32_t *const none[2] = {nullptr, nullptr};
+    uint32_t *const G[2] = {L.grp[0], L.grp[1]};
+    int fin = 0;
+    if ((rc = sort_packed(w, total, kb, dtype, K, none, G, count - 1, &fin, s))) return rc;
+    CK(launch_norm_xy(L.jobs, count, max_S, kb, dtype, o.translate, L.key[fin], L.norms, s));
+    TrainHyper h{};
+    h.steps = (int)o.steps; h.batch = o.batch; h.loss = o.loss; h.delta = o.huber_delta;
+    h.lr = o.lr; h.b1 = o.beta1; h.b2 = o.beta2; h.eps = o.adam_eps; h.c12 = L.c12;
+    if (cluster) {
+        CK(launch_train_cluster(pa, L.jobs, count, h, max_B, s));
+    } else if (tc64) {
+        for (uint32_t j = 0; j < count; ++j) {
+            TrainStepArgs t{};
+            t.params = hj[j].params; t.m = hj[j].m; t.v = hj[j].v;
+            t.partials = hj[j].partials; t.loss_partials = hj[j].loss_partials; t.loss_out = hj[j].loss_out;
+            t.x = hj[j].x; t.label = hj[j].label; t.S = S[j]; t.batch = o.batch; t.batch_seed = hj[j].bseed;
+            t.loss = o.loss; t.delta = o.huber_delta;
+            t.lr = o.lr; t.b1 = o.beta1; t.b2 = o.beta2; t.eps = o.adam_eps; t.mask = hj[j].mask;
+            // every step in one cooperative launch, whose blocks meet on a count that starts at zero
+            if (j) CK(cudaMemsetAsync(L.meet, 0, sizeof(unsigned int), s));
+            CK(launch_train_tc64(t, o.steps, L.c12, L.meet, s));
+        }
+    } else {
+        const uint32_t mb = *std::max_element(blocks.begin(), blocks.end());
+        for (uint32_t k = 0; k < o.steps; ++k)
+            CK(launch_train_step(pa, L.jobs, count, mb, h, Pp, (int)k, hc[k], hc[steps + k], s));
+    }
+    uint32_t te = 0;
+    if (tc64) CK(cudaMemcpyAsync(&te, terr, sizeof(uint32_t), cudaMemcpyDeviceToHost, s));
+    CK(cudaMemcpyAsync(host.data() + off_par, dev + off_par, back_end - off_par, cudaMemcpyDeviceToHost, s));
+    CK(cudaStreamSynchronize(s));
+    if (te & ERR_TIMEOUT) return NNSORT_E_TIMEOUT;
+    if (h_loss && steps) std::memcpy(h_loss, hp(L.loss), count * steps * sizeof(float));
+    std::vector<float> up(P);
+    for (uint32_t j = 0; j < count; ++j) {
+        const float *pp = reinterpret_cast<const float *>(hp(L.params + j * Pp));
+        for (size_t u = 0; u < P; ++u) up[u] = pp[pad_index(o.layers, o.h1, o.h2, pa, u)];
+        const Norm &q = *reinterpret_cast<const Norm *>(hp(L.norms + j));
+        d.lo_bits = q.lo_bits;
+        d.lo_val = q.lo_val;
+        d.scale = q.scale;
+        uint32_t err = 0;
+        std::memcpy(&err, hp(L.err + j), 4);
+        if (err & ERR_NAN) { rcs[j] = NNSORT_E_NAN_KEY; continue; }
+        rcs[j] = nnsort_model_create(&d, up.data(), &out[j]);
+    }
+    return NNSORT_OK;
+}

@@ -14,6 +14,7 @@ namespace nns {
 void note_launch(int kernels);
 
 struct Seg;
+struct Norm;
 struct SegStats;
 struct OKey;
 
@@ -206,10 +207,10 @@ cudaError_t launch_minmax_norm(const void *sorted_keys, uint64_t S, int key_byte
                                unsigned long long *lobits_out, cudaStream_t s);
 cudaError_t launch_make_xy(const void *sorted_keys, uint64_t S, int key_bytes, const Norm *nm_dev,
                            float *x, float *label, cudaStream_t s);
+// a training run of the two-layer model of width 64 (k_train_tc.cu)
 struct TrainStepArgs {
     float *params;        // padded layout, updated in place
     float *m, *v;         // Adam moments (padded layout)
-    float *grad;          // padded layout
     float *partials;      // [blocks * P]
     float *loss_partials; // [blocks]
     float *loss_out;      // [steps]
@@ -217,13 +218,45 @@ struct TrainStepArgs {
     uint64_t S;
     uint32_t batch;       // 0 = full
     uint64_t batch_seed;
-    int step;             // 0-based
     int loss; float delta;
     float lr, b1, b2, eps;
-    size_t P;
-    const float *mask;    // 1 for real parameters, 0 for padding
+    const float *mask;    // nullable: +1/-1 sign a parameter must keep, 0 free
 };
-cudaError_t launch_train_step(const PadArch &a, const TrainStepArgs &t, cudaStream_t s);
+// One model of a training call (models of one architecture trained side by side): its sample, its
+// batch and its parameters. Sample arrays of all models are packed; `off` is the model's first entry.
+struct TrainJob {
+    const void *keys;        // device keys to sample
+    uint64_t n, S, off;      // keys, sample size, offset in the packed sample arrays
+    uint64_t sseed, bseed;   // sample and mini-batch streams
+    uint64_t B;              // samples per step
+    float inv_n;             // 1 / B
+    uint32_t blocks;         // partial gradient rows of a step
+    float *params, *m, *v;   // padded layout
+    const float *mask;       // nullable: signs to keep
+    const float *x, *label;  // [S]
+    float *partials, *loss_partials;  // [blocks * P], [blocks] (null where no kernel uses them)
+    float *loss_out;         // [steps]
+};
+struct TrainHyper {
+    int steps;
+    uint32_t batch;          // 0: full batch
+    int loss;
+    float delta, lr, b1, b2, eps;
+    const float *c12;        // device [2 * steps]: 1 - beta1^(t+1), then 1 - beta2^(t+1)
+};
+// sample keys of every job (packed; `group` nullable: the job index of each), their inputs, labels and
+// normalisers once sorted
+cudaError_t launch_sample_jobs(const TrainJob *jobs, uint32_t models, uint64_t max_S, int key_bytes, int dtype,
+                               void *sample_keys, uint32_t *group, uint32_t *err, cudaStream_t s);
+cudaError_t launch_norm_xy(const TrainJob *jobs, uint32_t models, uint64_t max_S, int key_bytes, int dtype,
+                           int translate, const void *sorted_keys, Norm *norms, cudaStream_t s);
+// one Adam step of every job (per-step kernels), all steps of one-hidden-layer jobs in one launch
+// (k_train_cluster.cu)
+cudaError_t launch_train_step(const PadArch &a, const TrainJob *jobs, uint32_t models, uint32_t max_blocks,
+                              const TrainHyper &hp, size_t P, int step, float c1, float c2, cudaStream_t s);
+bool train_cluster_ok(const PadArch &a, uint64_t max_batch);
+cudaError_t launch_train_cluster(const PadArch &a, const TrainJob *jobs, uint32_t models, const TrainHyper &hp,
+                                 uint64_t max_batch, cudaStream_t s);
 // many small models at once, one block per model (k_train_block.cu): one hidden layer of padded
 // width 8, 16 or 32, samples of at most TB_MAX_S keys; the sort buffer holds `cap` keys (a power of
 // two >= every S of the launch)
@@ -263,6 +296,8 @@ struct GradArgs {
     float *partials;     // [rows * P]
     float *loss_partials;  // [rows], nullable
     float *gx;           // nullable (mode 0)
+    const TrainJob *jobs;  // nullable: block row y computes the step of job y (mode 1 or 2)
+    int step;              // with jobs: the step
 };
 int train_grad_blocks(const PadArch &a, uint64_t nsamples);
 // two hidden layers of width 64 on the tensor cores (k_train_tc.cu): blocks of the launch (each
@@ -287,7 +322,21 @@ cudaError_t launch_reduce_partials(const float *partials, int blocks, size_t P, 
                                    const float *loss_partials, float *loss_out, float scale,
                                    cudaStream_t s);
 
+// Device memory from the library's own pool (api.cu), ordered on the stream like cudaMallocAsync. The
+// device's default pool gives its memory back at every synchronisation, so that each call after one
+// maps its buffers again; this one keeps up to POOL_KEEP bytes until nnsort_release.
+constexpr size_t POOL_KEEP = (size_t)256 << 20;
+cudaError_t pool_alloc(void **p, size_t bytes, cudaStream_t s);
+
 }  // namespace nns
+
+// Trains `count` models of one architecture side by side (the recipe of nnsort_train; api.cu): model j
+// on d_keys[j] with sample size S[j] and seed seeds[j]. rc[j] receives each model's status and out[j]
+// its model (null unless NNSORT_OK); h_loss (nullable): count x steps. Synchronous. Returns an error
+// that concerns the whole call.
+int nnsort_train_models(const void *const *d_keys, const uint64_t *ns, uint32_t count, int32_t dtype,
+                        const nnsort_train_opts &o, const uint64_t *S, const uint64_t *seeds,
+                        struct nnsort_model **out, int *rc, float *h_loss, cudaStream_t s);
 
 // The model handle behind the opaque nnsort_model of the C ABI: one definition for every
 // translation unit that reads it.

@@ -12,6 +12,7 @@
 
 #include "common.cuh"
 #include "internal.h"
+#include "train_math.cuh"
 
 namespace nns {
 static inline cudaError_t nns_launched(cudaError_t e, int k = 1) {
@@ -76,6 +77,84 @@ cudaError_t launch_make_xy(const void *sorted_keys, uint64_t S, int key_bytes, c
     return nns_launched(cudaGetLastError());
 }
 
+// ---- the samples of a training call: row y of the grid serves job y
+template <typename W>
+__global__ void k_sample_jobs(const TrainJob *jobs, int dtype, W *out, uint32_t *group, uint32_t *err) {
+    const TrainJob &J = jobs[blockIdx.y];
+    const W *keys = reinterpret_cast<const W *>(J.keys);
+    const uint64_t n = J.n, S = J.S, off = J.off, seed = J.sseed;
+    for (uint64_t j = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; j < S;
+         j += (uint64_t)gridDim.x * blockDim.x) {
+        const W k = keys[__umul64hi(rng_draw(seed, j), n)];
+        if (key_is_nan(word64(k), dtype)) atomicOr(&err[blockIdx.y], ERR_NAN);
+        out[off + j] = k;
+        if (group) group[off + j] = blockIdx.y;
+    }
+}
+
+cudaError_t launch_sample_jobs(const TrainJob *jobs, uint32_t models, uint64_t max_S, int key_bytes, int dtype,
+                               void *sample_keys, uint32_t *group, uint32_t *err, cudaStream_t s) {
+    const dim3 grid((unsigned)std::min<uint64_t>((max_S + 255) / 256, 4096), models);
+    if (key_bytes == 4)
+        k_sample_jobs<uint32_t><<<grid, 256, 0, s>>>(jobs, dtype, reinterpret_cast<uint32_t *>(sample_keys), group, err);
+    else
+        k_sample_jobs<uint64_t><<<grid, 256, 0, s>>>(jobs, dtype, reinterpret_cast<uint64_t *>(sample_keys), group, err);
+    return nns_launched(cudaGetLastError());
+}
+
+// the normaliser of a job from the ends of its sorted sample (the host's arithmetic in
+// nnsort_sample_labels: every operation is a correctly rounded binary64 one), then inputs and labels
+__device__ __forceinline__ double key_value(uint64_t w, int dtype) {
+    if (dtype == NNSORT_F32) return (double)__uint_as_float((uint32_t)w);
+    if (dtype == NNSORT_F64) return __longlong_as_double((long long)w);
+    return __ull2double_rn(w);
+}
+template <typename W>
+__global__ void k_norm_xy(const TrainJob *jobs, int dtype, int translate, const W *sorted, Norm *norms) {
+    __shared__ Norm sn;
+    const TrainJob &J = jobs[blockIdx.y];
+    const uint64_t S = J.S;
+    const W *key = sorted + J.off;
+    if (threadIdx.x == 0) {
+        const uint64_t wlo = word64(key[0]), whi = word64(key[S - 1]);
+        const uint64_t lo = ordbits(wlo, dtype), hi = ordbits(whi, dtype);
+        Norm q;
+        q.dtype = dtype;
+        q.translate = translate;
+        q.lo_bits = lo;
+        q.lo_val = key_value(wlo, dtype);
+        const bool ob = translate == NNSORT_TRANSLATE_ORDBITS || dtype == NNSORT_U32 || dtype == NNSORT_U64;
+        if (ob) {
+            q.scale = (hi > lo) ? __ddiv_rn(1.0, __ull2double_rn(hi - lo)) : 1.0;
+        } else {
+            const double hv = key_value(whi, dtype);
+            q.scale = (hv > q.lo_val) ? __ddiv_rn(1.0, __dsub_rn(hv, q.lo_val)) : 1.0;
+        }
+        q.lo_f = __double2float_rn(q.lo_val);
+        q.scale_f = __double2float_rn(q.scale);
+        sn = q;
+        if (blockIdx.x == 0) norms[blockIdx.y] = q;
+    }
+    __syncthreads();
+    const Norm N = sn;
+    float *x = const_cast<float *>(J.x), *label = const_cast<float *>(J.label);
+    for (uint64_t j = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; j < S;
+         j += (uint64_t)gridDim.x * blockDim.x) {
+        x[j] = translate_key<W>(key[j], N);
+        label[j] = __double2float_rn(__ddiv_rn((double)j, (double)S));
+    }
+}
+
+cudaError_t launch_norm_xy(const TrainJob *jobs, uint32_t models, uint64_t max_S, int key_bytes, int dtype,
+                           int translate, const void *sorted_keys, Norm *norms, cudaStream_t s) {
+    const dim3 grid((unsigned)std::min<uint64_t>((max_S + 255) / 256, 4096), models);
+    if (key_bytes == 4)
+        k_norm_xy<uint32_t><<<grid, 256, 0, s>>>(jobs, dtype, translate, reinterpret_cast<const uint32_t *>(sorted_keys), norms);
+    else
+        k_norm_xy<uint64_t><<<grid, 256, 0, s>>>(jobs, dtype, translate, reinterpret_cast<const uint64_t *>(sorted_keys), norms);
+    return nns_launched(cudaGetLastError());
+}
+
 // ---- forward pass for explicit inputs
 template <int H1, int H2>
 __global__ void k_mlp_forward(const float *params, const float *x, uint64_t n, float *y) {
@@ -89,8 +168,19 @@ __global__ void k_mlp_forward(const float *params, const float *x, uint64_t n, f
 }
 
 // ---- gradient of a sum over samples (GradArgs: internal.h)
+// a training step of several jobs: block row y takes job y's arrays; returns the job's block count
+__device__ __forceinline__ uint32_t grad_job(GradArgs &g) {
+    if (!g.jobs) return gridDim.x;
+    const TrainJob &J = g.jobs[blockIdx.y];
+    g.params = J.params; g.x = J.x; g.label = J.label;
+    g.n = J.B; g.S = J.S; g.bseed = J.bseed; g.bofs = (uint64_t)g.step * J.B; g.inv_n = J.inv_n;
+    g.partials = J.partials; g.loss_partials = J.loss_partials;
+    return J.blocks;
+}
 template <int H1, int H2>
 __global__ void __launch_bounds__(TR_THREADS) k_grad(GradArgs g) {
+    const uint32_t nblk = grad_job(g);
+    if (blockIdx.x >= nblk) return;
     constexpr int HL = (H2 == 0) ? H1 : H2;
     constexpr int P = (H2 == 0) ? (3 * H1 + 1) : (2 * H1 + H2 * H1 + 2 * H2 + 1);
     extern __shared__ __align__(16) float sm[];
@@ -109,7 +199,7 @@ __global__ void __launch_bounds__(TR_THREADS) k_grad(GradArgs g) {
     const float *W2 = sp + 2 * H1, *b2 = W2 + H2 * H1;
     const float *W3 = (H2 == 0) ? sp + 2 * H1 : b2 + H2;
     // each block owns a contiguous range of the batch
-    const uint64_t per = (g.n + gridDim.x - 1) / gridDim.x;
+    const uint64_t per = (g.n + nblk - 1) / nblk;
     const uint64_t i0 = std::min<uint64_t>(g.n, (uint64_t)blockIdx.x * per);
     const uint64_t i1 = std::min<uint64_t>(g.n, i0 + per);
     float acc[(P + TR_THREADS - 1) / TR_THREADS];
@@ -148,16 +238,7 @@ __global__ void __launch_bounds__(TR_THREADS) k_grad(GradArgs g) {
             if (g.mode == 0) {
                 gy = g.gy[i];
             } else {
-                const float r = y - g.label[src];
-                if (g.loss == NNSORT_LOSS_HUBER) {
-                    const float ar = fabsf(r);
-                    lv = (ar <= g.delta) ? 0.5f * r * r : g.delta * ar - 0.5f * g.delta * g.delta;
-                    gy = (r > g.delta) ? g.delta : ((r < -g.delta) ? -g.delta : r);
-                } else {
-                    lv = r * r;
-                    gy = 2.0f * r;
-                }
-                gy *= g.inv_n;
+                loss_term(y - g.label[src], g.loss, g.delta, g.inv_n, gy, lv);
             }
             sx[tid] = x;
             sgy[tid] = gy;
@@ -271,6 +352,8 @@ __device__ __forceinline__ void load_pairs(const float *p, unsigned long long *b
 
 template <int H>
 __global__ void __launch_bounds__(TR_THREADS, 2) k_grad_gemm(GradArgs g) {
+    const uint32_t nblk = grad_job(g);
+    if (blockIdx.x >= nblk) return;
     using S = GemmSmem<H>;
     constexpr int LD = S::LD, LDT = S::LDT, P = S::P;
     constexpr int TN = H / 16;  // outputs per thread along the width (4 for H = 64, 2 for H = 32)
@@ -310,7 +393,7 @@ __global__ void __launch_bounds__(TR_THREADS, 2) k_grad_gemm(GradArgs g) {
     float pb1[TN], pw1[TN];
 #pragma unroll
     for (int q = 0; q < TN; ++q) { pb1[q] = 0.0f; pw1[q] = 0.0f; }
-    const uint64_t per = (g.n + gridDim.x - 1) / gridDim.x;
+    const uint64_t per = (g.n + nblk - 1) / nblk;
     const uint64_t i0 = std::min<uint64_t>(g.n, (uint64_t)blockIdx.x * per);
     const uint64_t i1 = std::min<uint64_t>(g.n, i0 + per);
     __syncthreads();
@@ -372,16 +455,7 @@ __global__ void __launch_bounds__(TR_THREADS, 2) k_grad_gemm(GradArgs g) {
                 if (g.mode == 0) {
                     gy = g.gy[c0 + tid];
                 } else {
-                    const float r = y - g.label[src];
-                    if (g.loss == NNSORT_LOSS_HUBER) {
-                        const float ar = fabsf(r);
-                        lv = (ar <= g.delta) ? 0.5f * r * r : g.delta * ar - 0.5f * g.delta * g.delta;
-                        gy = (r > g.delta) ? g.delta : ((r < -g.delta) ? -g.delta : r);
-                    } else {
-                        lv = r * r;
-                        gy = 2.0f * r;
-                    }
-                    gy *= g.inv_n;
+                    loss_term(y - g.label[src], g.loss, g.delta, g.inv_n, gy, lv);
                 }
             }
             sGY[tid] = gy;
@@ -532,7 +606,7 @@ int train_grad_blocks(const PadArch &a, uint64_t nsamples) {
 }
 
 template <int H1, int H2>
-static cudaError_t grad_go(const GradArgs &g, int blocks, cudaStream_t s) {
+static cudaError_t grad_go(const GradArgs &g, dim3 blocks, cudaStream_t s) {
     const size_t smem = grad_smem<H1, H2>();
     cudaError_t e = cudaFuncSetAttribute(k_grad<H1, H2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
@@ -541,7 +615,7 @@ static cudaError_t grad_go(const GradArgs &g, int blocks, cudaStream_t s) {
 }
 
 template <int H>
-static cudaError_t grad_gemm_go(const GradArgs &g, int blocks, cudaStream_t s) {
+static cudaError_t grad_gemm_go(const GradArgs &g, dim3 blocks, cudaStream_t s) {
     const size_t smem = sizeof(float) * GemmSmem<H>::FLOATS;
     cudaError_t e = cudaFuncSetAttribute(k_grad_gemm<H>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
@@ -549,7 +623,7 @@ static cudaError_t grad_gemm_go(const GradArgs &g, int blocks, cudaStream_t s) {
     return nns_launched(cudaGetLastError());
 }
 
-static cudaError_t grad_dispatch(const PadArch &a, const GradArgs &g, int blocks, cudaStream_t s) {
+static cudaError_t grad_dispatch(const PadArch &a, const GradArgs &g, dim3 blocks, cudaStream_t s) {
     if (a.layers == 1) {
         switch (a.h1) {
         case 8: return grad_go<8, 0>(g, blocks, s);
@@ -581,6 +655,8 @@ struct ReduceArgs {
     float *params, *m, *v;
     const float *mask;  // nullable: +1/-1 sign a parameter must keep, 0 free
     float lr, b1, b2, eps, c1, c2;
+    const TrainJob *jobs;  // nullable: block row y reduces and updates job y
+    int step;
 };
 
 // A block takes 32 parameters (lane l: parameter 32 b + l) and its warp w adds partial rows w, w + 16,
@@ -608,6 +684,12 @@ __global__ void __launch_bounds__(RD_WARPS * 32) k_reduce(ReduceArgs r) {
     __shared__ float sh[RD_WARPS][33];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const size_t nb = (r.P + 31) / 32;
+    if (r.jobs) {
+        const TrainJob &J = r.jobs[blockIdx.y];
+        r.partials = J.partials; r.blocks = (int)J.blocks; r.loss_partials = J.loss_partials;
+        r.loss_out = J.loss_out + r.step; r.loss_scale = J.inv_n;
+        r.params = J.params; r.m = J.m; r.v = J.v; r.mask = J.mask;
+    }
     if (blockIdx.x == nb) {  // the loss
         const bool on = r.loss_partials && r.loss_out && lane == 0;
         sh[w][lane] = rows_sum(r.loss_partials, 1, r.blocks, w, on);
@@ -627,14 +709,11 @@ __global__ void __launch_bounds__(RD_WARPS * 32) k_reduce(ReduceArgs r) {
     for (int q = 0; q < RD_WARPS; ++q) g = __fadd_rn(g, sh[q][lane]);
     if (r.out) r.out[p] = g;
     if (r.params) {
-        const float m = r.b1 * r.m[p] + (1.0f - r.b1) * g;
-        const float v = r.b2 * r.v[p] + (1.0f - r.b2) * g * g;
+        float m = r.m[p], v = r.v[p];
+        r.params[p] = adam_step(r.params[p], g, m, v, r.lr, r.b1, r.b2, r.eps, r.c1, r.c2,
+                                r.mask ? r.mask[p] : 0.0f);
         r.m[p] = m;
         r.v[p] = v;
-        const float mh = m / r.c1, vh = v / r.c2;
-        float np = r.params[p] - r.lr * mh / (sqrtf(vh) + r.eps);
-        if (r.mask && r.mask[p] * np < 0.0f) np = 0.0f;  // monotone projection
-        r.params[p] = np;
     }
 }
 static unsigned reduce_grid(size_t P) { return (unsigned)((P + 31) / 32 + 1); }
@@ -649,25 +728,17 @@ cudaError_t launch_reduce_partials(const float *partials, int blocks, size_t P, 
     return nns_launched(cudaGetLastError());
 }
 
-cudaError_t launch_train_step(const PadArch &a, const TrainStepArgs &t, cudaStream_t s) {
-    const uint64_t B = t.batch ? t.batch : t.S;
-    const int blocks = train_grad_blocks(a, B);
+cudaError_t launch_train_step(const PadArch &a, const TrainJob *jobs, uint32_t models, uint32_t max_blocks,
+                              const TrainHyper &hp, size_t P, int step, float c1, float c2, cudaStream_t s) {
     GradArgs g{};
-    g.params = t.params; g.x = t.x; g.label = t.label; g.n = B; g.S = t.S;
-    g.bseed = t.batch_seed; g.bofs = (uint64_t)t.step * B;
-    g.mode = t.batch ? 2 : 1; g.loss = t.loss; g.delta = t.delta; g.inv_n = 1.0f / (float)B;
-    g.partials = t.partials; g.loss_partials = t.loss_partials; g.gx = nullptr;
-    cudaError_t e = grad_dispatch(a, g, blocks, s);
+    g.jobs = jobs; g.step = step;
+    g.mode = hp.batch ? 2 : 1; g.loss = hp.loss; g.delta = hp.delta;
+    cudaError_t e = grad_dispatch(a, g, dim3(max_blocks, models), s);
     if (e != cudaSuccess) return e;
     ReduceArgs r{};
-    r.partials = t.partials; r.blocks = blocks; r.P = t.P; r.out = t.grad;
-    r.loss_partials = t.loss_partials; r.loss_out = t.loss_out + t.step; r.loss_scale = 1.0f / (float)B;
-    r.params = t.params; r.m = t.m; r.v = t.v; r.lr = t.lr; r.b1 = t.b1; r.b2 = t.b2; r.eps = t.eps;
-    r.mask = t.mask;
-    const double c1 = 1.0 - std::pow((double)t.b1, (double)(t.step + 1));
-    const double c2 = 1.0 - std::pow((double)t.b2, (double)(t.step + 1));
-    r.c1 = (float)c1; r.c2 = (float)c2;
-    k_reduce<<<reduce_grid(t.P), RD_WARPS * 32, 0, s>>>(r);
+    r.jobs = jobs; r.step = step; r.P = P;
+    r.lr = hp.lr; r.b1 = hp.b1; r.b2 = hp.b2; r.eps = hp.eps; r.c1 = c1; r.c2 = c2;
+    k_reduce<<<dim3(reduce_grid(P), models), RD_WARPS * 32, 0, s>>>(r);
     return nns_launched(cudaGetLastError());
 }
 
@@ -710,7 +781,7 @@ cudaError_t launch_mlp_backward(const PadArch &a, const float *params, const flo
     g.params = params; g.x = x; g.gy = gy; g.label = label; g.n = n; g.S = n;
     g.mode = mode; g.loss = loss; g.delta = delta; g.inv_n = n ? 1.0f / (float)n : 0.0f;
     g.partials = partials; g.loss_partials = loss_partials; g.gx = gx;
-    return grad_dispatch(a, g, blocks, s);
+    return grad_dispatch(a, g, dim3((unsigned)blocks), s);
 }
 
 }  // namespace nns

@@ -14,7 +14,7 @@
 
 #include <cuda_runtime.h>
 
-#include "nnsort.h"
+#include "internal.h"
 
 namespace {
 
@@ -109,8 +109,8 @@ void worker_main(nnsort_server *s) {
         std::vector<int> rc(cnt, NNSORT_OK);
         for (int i = 0; i < cnt; ++i) {
             const Req &r = batch[i];
-            if (cudaMallocAsync(&dk[i], r.n * kb, st) != cudaSuccess ||
-                (r.h_pay && cudaMallocAsync((void **)&dp[i], r.n * 4, st) != cudaSuccess)) {
+            if (nns::pool_alloc(&dk[i], r.n * kb, st) != cudaSuccess ||
+                (r.h_pay && nns::pool_alloc((void **)&dp[i], r.n * 4, st) != cudaSuccess)) {
                 cudaGetLastError();
                 rc[i] = NNSORT_E_OOM;
                 continue;
@@ -118,12 +118,36 @@ void worker_main(nnsort_server *s) {
             cudaMemcpyAsync(dk[i], r.h_keys, r.n * kb, cudaMemcpyHostToDevice, st);
             if (r.h_pay) cudaMemcpyAsync(dp[i], r.h_pay, r.n * 4, cudaMemcpyHostToDevice, st);
         }
-        for (int i = 0; i < cnt; ++i) {
-            if (rc[i]) continue;
-            nnsort_train_opts to = s->o.train;
-            to.seed = batch[i].seed;
-            to.sample_n = std::max<uint64_t>(1, std::min<uint64_t>(to.sample_n, batch[i].n));
-            rc[i] = nnsort_train(dk[i], batch[i].n, dt, &to, &models[i], nullptr, st);
+        // the requests' models side by side: a step of one small model leaves most of the GPU idle
+        {
+            std::vector<const void *> tk;
+            std::vector<uint64_t> tn, ts, tseed;
+            std::vector<int> ti;
+            for (int i = 0; i < cnt; ++i) {
+                if (rc[i]) continue;
+                tk.push_back(dk[i]);
+                tn.push_back(batch[i].n);
+                ts.push_back(std::max<uint64_t>(1, std::min<uint64_t>(s->o.train.sample_n, batch[i].n)));
+                tseed.push_back(batch[i].seed);
+                ti.push_back(i);
+            }
+            const uint32_t m = (uint32_t)ti.size();
+            std::vector<nnsort_model *> tf(m, nullptr);
+            std::vector<int> trc(m, NNSORT_OK);
+            const int all = nnsort_train_models(tk.data(), tn.data(), m, dt, s->o.train, ts.data(), tseed.data(),
+                                                tf.data(), trc.data(), nullptr, st);
+            for (uint32_t q = 0; q < m; ++q) {
+                const int i = ti[q];
+                if (all == NNSORT_OK) {
+                    models[i] = tf[q];
+                    rc[i] = trc[q];
+                } else {  // the joint call failed (no memory for all of them, say): one by one
+                    nnsort_train_opts to = s->o.train;
+                    to.seed = tseed[q];
+                    to.sample_n = ts[q];
+                    rc[i] = nnsort_train(tk[q], tn[q], dt, &to, &models[i], nullptr, st);
+                }
+            }
         }
         // one pass of the pipeline over every request that trained
         std::vector<void *> sk;
