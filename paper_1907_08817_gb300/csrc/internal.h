@@ -87,10 +87,8 @@ void pwl_key_table(const nnsort_model_desc &d, const std::vector<double> &brk, c
 // chunks and digits, then the scatter of every tile to its chunk's base + its in-chunk prefix.
 // The pass finds its own digit offsets, so no histogram is needed beforehand; tile_hist, chunk and
 // bin_total are scratch.
-constexpr int SC_THREADS = 512;
-constexpr int SC_ITEMS = 8;
-constexpr int SC_TILE = SC_THREADS * SC_ITEMS;  // 4096
-constexpr int SC_CHUNK = 16;                    // tiles per chunk (in-chunk prefix < 2^16)
+constexpr int SC_TILE = 4096;
+constexpr int SC_CHUNK = 65536 / SC_TILE;  // tiles per chunk (in-chunk prefix < 2^16)
 struct PartitionArgs {
     uint64_t N;
     const uint32_t *gs_in;  uint32_t *gs_out;   // null when sorting by key bits
