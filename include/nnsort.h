@@ -154,11 +154,13 @@ typedef struct {
     double e[NNSORT_MAX_ROUNDS];               /* out-of-order rate of o_i */
     double trad_rate;                          /* traditional sorting rate: |w_t| / n */
     uint64_t buckets;                          /* on-chip buckets the positions were cut into */
-    uint64_t oversized_buckets;                /* buckets processed from global memory */
+    uint64_t oversized_buckets;                /* buckets above the on-chip capacity of a polish that
+                                                  runs polish_blocks blocks per SM */
     uint64_t repaired;                         /* elements re-sorted across bucket seams */
     /* stage durations (CUDA events on the call's stream), filled when nnsort_sort_opts.timing = 1:
-     * [0] predict, [1] partition (all passes), [2] bucket bounds, [3] rounds, [4] finalize,
-     * [5] polish, [6] seam/repair, [7] whole call. Batched sorts report them in entry 0. */
+     * [0] predict, [1] partition (all passes), [2] bucket bounds, [3] rounds (and, where one pass
+     * serves a bucket, its runs and sorted output), [4] finalize, [5] polish (what the carries decide,
+     * and buckets that no block holds), [6] seam/repair, [7] whole call. Batched sorts report them in entry 0. */
     float ms_stage[8];
     uint32_t partition_passes;                 /* stable partition passes run */
     uint32_t bucket_log2;                      /* log2 of the positions per bucket */

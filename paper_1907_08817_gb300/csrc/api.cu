@@ -525,7 +525,7 @@ struct Layout {
     uint8_t *rank; uint8_t *g_flag; uint32_t *g_x, *g_y; uint32_t *bstart;
     OKey *bmax, *carry, *blo, *bhi;
     SeamRange *ranges; uint32_t *seam_cnt;
-    uint32_t *order, *order_cnt;
+    uint32_t *order, *order_cnt, *rend;
     BigRange *big; uint32_t *big_cnt;
     BigRange *giant; uint32_t *giant_cnt; unsigned int *g_cnt, *g_tbmax; unsigned long long *g_kmax;
 };
@@ -558,11 +558,12 @@ Layout carve(unsigned char *base, int nseg, uint64_t N, uint32_t NB, int kb, boo
     L.seam_cnt = c.take<uint32_t>(4);
     L.order = c.take<uint32_t>(NB);
     L.order_cnt = c.take<uint32_t>(4);
+    L.rend = rows ? nullptr : c.take<uint32_t>((size_t)NB * MAXR);
     L.big = c.take<BigRange>(N / POLISH_BIG + 1);
     L.big_cnt = c.take<uint32_t>(4);
-    L.giant = c.take<BigRange>(N / POLISH_BIG + 1);
+    L.giant = c.take<BigRange>(N / GIANT_LEAST + 1);
     L.giant_cnt = c.take<uint32_t>(4);
-    L.g_cnt = c.take<unsigned int>((N / POLISH_BIG + 1) * MAXR);
+    L.g_cnt = c.take<unsigned int>((N / GIANT_LEAST + 1) * MAXR);
     L.g_tbmax = c.take<unsigned int>((N / POLISH_BIG + 1) * MAXR);
     L.g_kmax = c.take<unsigned long long>((N / POLISH_BIG + 1) * MAXR);
     *total = align_up(c.off, 256);
@@ -749,30 +750,23 @@ int repair_long_ranges(Workspace *w, Layout &L, SeamRange *hr, uint32_t nr, int 
     return NNSORT_OK;  // the next call on this stream waits before it rewrites the staging area
 }
 
-// buckets too large for one block's polish (listed by k_polish, host copy hb[0..nb)): their
-// elements, packed from the partition buffers (pair `src`), sorted by key and then by bucket, and
-// written to their output positions; then their first/last elements for the seam
-int sort_big_buckets(Workspace *w, Layout &L, BigRange *hb, uint32_t nb, int src, int kb, int dtype,
-                     bool anypay, cudaStream_t s) {
-    std::sort(hb, hb + nb, [](const BigRange &x, const BigRange &y) { return x.lo < y.lo; });
-    uint64_t total = 0;
-    for (uint32_t j = 0; j < nb; ++j) {
-        hb[j].off = (uint32_t)total;
-        total += hb[j].hi - hb[j].lo;
-    }
-    CK(cudaMemcpyAsync(L.big, hb, sizeof(BigRange) * nb, cudaMemcpyHostToDevice, s));
+// buckets too large for one block (listed on the device with their packed offsets, `total` elements):
+// packed from the partition buffers (pair `src`), sorted by key and then by bucket, and written to
+// their output positions; then their first/last elements for the seam
+int sort_big_buckets(Workspace *w, Layout &L, const BigRange *list, uint32_t nb, uint64_t total, int src, int kb,
+                     int dtype, bool anypay, cudaStream_t s) {
     const int sms = sm_count(), o = src ^ 1;
     // pack into the free pair, then ping-pong between it and the (now dead) source pair
     void *const K[2] = {L.key[o], L.key[src]};
     uint32_t *const P[2] = {anypay ? L.pay[o] : nullptr, anypay ? L.pay[src] : nullptr};
     uint32_t *const J[2] = {L.gs[o], L.gs[src]};
-    CK(launch_big_pack(L.big, nb, L.segs, total, kb, L.key[src], anypay ? L.pay[src] : nullptr, K[0], P[0],
+    CK(launch_big_pack(list, nb, L.segs, total, kb, L.key[src], anypay ? L.pay[src] : nullptr, K[0], P[0],
                        nb > 1 ? J[0] : nullptr, 0, sms, s));
     int fin = 0, rc;
     if ((rc = sort_packed(w, total, kb, dtype, K, P, J, nb > 1 ? nb - 1 : 0u, &fin, s)))
         return rc;
-    CK(launch_big_pack(L.big, nb, L.segs, total, kb, nullptr, nullptr, K[fin], P[fin], nullptr, 1, sms, s));
-    CK(launch_big_bounds(L.big, nb, L.segs, kb, dtype, L.blo, L.bhi, s));
+    CK(launch_big_pack(list, nb, L.segs, total, kb, nullptr, nullptr, K[fin], P[fin], nullptr, 1, sms, s));
+    CK(launch_big_bounds(list, nb, L.segs, kb, dtype, L.blo, L.bhi, s));
     return NNSORT_OK;
 }
 
@@ -940,11 +934,26 @@ int run_sort(const std::vector<SegIn> &in, const nnsort_sort_opts *op, int dtype
     sa.seam_suf = L.bmax;  // free once the polish has run
     sa.seam_pre = L.bmax + P.NB;
     sa.seam_cut = reinterpret_cast<unsigned long long *>(L.carry);
-    // buckets above POLISH_BIG elements (possible only when N exceeds it) run their rounds on the
-    // whole GPU; their claim tables reuse the g_x scratch ((N / POLISH_BIG + 1) W entries of 8 bytes
-    // fit in 4 N bytes for N > POLISH_BIG, W <= 2^14), which the polish needs only later
+    const int sms = sm_count();
+    const bool onepass = buckets_ok(P.wlog, rows);
+    uint64_t heavy = (uint64_t)sa.polish_cap;  // elements of a bucket that the front of the order exceeds
+    sa.giant_min = POLISH_BIG;
+    if (onepass) {
+        sa.bucket_cap[0] = bucket_capacity(kb, anypay, 2);
+        sa.bucket_cap[1] = bucket_capacity(kb, anypay, 1);
+        heavy = (uint64_t)sa.bucket_cap[0];
+        sa.giant_min = (uint32_t)sa.bucket_cap[1];
+        // the other pair of partition buffers holds the runs until their carries are known
+        sa.rk = L.key[oi];
+        sa.rt = L.gs[oi];
+        sa.rend = L.rend;
+    }
+    // giant buckets (possible only when N exceeds their least size) run their rounds on the whole GPU;
+    // their claim tables reuse the g_x scratch, which the polish needs only later: at most N / giant_min
+    // entries of W 8-byte words fit in 4 N bytes for W <= giant_min / 2
+    const bool giants = P.N > sa.giant_min;
     GiantRounds gr{};
-    if (P.N > POLISH_BIG) {
+    if (giants) {
         sa.giant = L.giant;
         sa.giant_cnt = L.giant_cnt;
         gr.list = L.giant;
@@ -953,39 +962,59 @@ int run_sort(const std::vector<SegIn> &in, const nnsort_sort_opts *op, int dtype
         gr.cnt = L.g_cnt;
         gr.kmax = L.g_kmax;
         gr.tbmax = L.g_tbmax;
-        gr.cap = (uint32_t)(P.N / POLISH_BIG + 1);
+        gr.cap = (uint32_t)(P.N / sa.giant_min + 1);
     }
-    CK(launch_bucket_order(sa, (uint32_t)sa.polish_cap, L.order, L.order_cnt, s));
-    sa.order = L.order;
-    if (!rows) {
-        sa.big = L.big;
-        sa.big_cnt = L.big_cnt;
-        CK(cudaMemsetAsync(L.big_cnt, 0, sizeof(uint32_t), s));
+    if (P.N > heavy || !onepass) {  // no bucket can exceed it otherwise
+        CK(launch_bucket_order(sa, (uint32_t)heavy, L.order, L.order_cnt, s));
+        sa.order = L.order;
+        if (onepass) sa.heavy_cnt = L.order_cnt;
     }
-    CK(launch_rounds(sa, s));
-    if (sa.giant) CK(launch_giant_rounds(sa, gr, o.eps, sm_count(), s));
+    if (onepass) {
+        CK(launch_buckets(sa, sms, s));
+        if (giants) CK(launch_giant_buckets(sa, gr, o.eps, sms, s));
+    } else {
+        if (!rows) {
+            sa.big = L.big;
+            sa.big_cnt = L.big_cnt;
+            CK(cudaMemsetAsync(L.big_cnt, 0, sizeof(uint32_t), s));
+        }
+        CK(launch_rounds(sa, s));
+        if (giants) CK(launch_giant_rounds(sa, gr, o.eps, sms, s));
+    }
     CK(mark(4));
     CK(launch_finalize(sa, s));
     CK(mark(5));
-    CK(launch_polish(sa, s));
-    if (sa.big) {
+    if (onepass) CK(launch_carried(sa, s));
+    else CK(launch_polish(sa, s));
+    if (giants && !rows) {
         // buckets too large for one block: one wait, then one multi-block sort of all of them
         uint32_t *hc = reinterpret_cast<uint32_t *>(w->pinned + pin_cnt);
-        CK(cudaMemcpyAsync(hc, L.big_cnt, sizeof(uint32_t), cudaMemcpyDeviceToHost, s));
+        CK(cudaMemcpyAsync(hc, onepass ? L.giant_cnt : L.big_cnt, 2 * sizeof(uint32_t), cudaMemcpyDeviceToHost, s));
         CK(cudaStreamSynchronize(s));
         const uint32_t nbig = hc[0];
         if (nbig) {
-            if (nbig > P.N / POLISH_BIG + 1) return NNSORT_E_STATE;
-            BigRange *hb = reinterpret_cast<BigRange *>(w->pinned + pin_big);
-            CK(cudaMemcpyAsync(hb, L.big, sizeof(BigRange) * nbig, cudaMemcpyDeviceToHost, s));
-            CK(cudaStreamSynchronize(s));
-            for (uint32_t j = 0; j < nbig; ++j)
-                if (hb[j].seg >= (uint32_t)nseg || hb[j].lo >= hb[j].hi || hb[j].hi > P.N) return NNSORT_E_STATE;
-            if ((rc = sort_big_buckets(w, L, hb, nbig, fi, kb, dtype, anypay, s))) return rc;
+            if (nbig > P.N / sa.giant_min + 1) return NNSORT_E_STATE;
+            uint64_t total = hc[1];
+            if (!onepass) {
+                // k_polish's list: the packed offsets are made here
+                BigRange *hb = reinterpret_cast<BigRange *>(w->pinned + pin_big);
+                CK(cudaMemcpyAsync(hb, L.big, sizeof(BigRange) * nbig, cudaMemcpyDeviceToHost, s));
+                CK(cudaStreamSynchronize(s));
+                total = 0;
+                for (uint32_t j = 0; j < nbig; ++j) {
+                    if (hb[j].seg >= (uint32_t)nseg || hb[j].lo >= hb[j].hi || hb[j].hi > P.N) return NNSORT_E_STATE;
+                    hb[j].off = (uint32_t)total;
+                    total += hb[j].hi - hb[j].lo;
+                }
+                CK(cudaMemcpyAsync(L.big, hb, sizeof(BigRange) * nbig, cudaMemcpyHostToDevice, s));
+            }
+            if (total > P.N) return NNSORT_E_STATE;
+            if ((rc = sort_big_buckets(w, L, onepass ? L.giant : L.big, nbig, total, fi, kb, dtype, anypay, s)))
+                return rc;
         }
     }
     CK(mark(6));
-    CK(launch_seam_repair(sa, sm_count(), s));
+    CK(launch_seam_repair(sa, sms, s));
     if (sa.allow_defer) {
         // one wait at the end of the pipeline: long seam ranges run as one multi-block sort
         uint32_t *hc = reinterpret_cast<uint32_t *>(w->pinned + pin_cnt);

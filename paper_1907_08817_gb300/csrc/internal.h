@@ -123,6 +123,7 @@ struct BigRange {
     uint32_t seg, off, b, pad;
 };
 constexpr uint32_t POLISH_BIG = 1u << 16;  // buckets above this many elements sort multi-block
+constexpr uint32_t GIANT_LEAST = 8192;     // no listed bucket is smaller (sizes the lists)
 
 struct SolveArgs {
     const Seg *segs;
@@ -159,6 +160,14 @@ struct SolveArgs {
     OKey *seam_suf;           // [NB] scratch: smallest element of the later buckets
     OKey *seam_pre;           // [NB] scratch: largest element of the earlier buckets
     unsigned long long *seam_cut;  // [2 NB] scratch: first and last sorted-boundary cut per bucket
+    // one-pass buckets (launch_buckets; null rk: not used): the in-order runs that await their carries,
+    // as order images and tie-breaks in partitioned element order, and where each round's run ends
+    void *rk;                 // [N] keys' width
+    uint32_t *rt;             // [N]
+    uint32_t *rend;           // [NB * MAXR]
+    int bucket_cap[2];        // elements that a one-pass block holds with two and with one block per SM
+    const uint32_t *heavy_cnt;  // with rk: the order's first *heavy_cnt buckets exceed bucket_cap[0]
+    uint32_t giant_min;       // buckets above this many elements are listed in giant
     const uint32_t *order;    // [NB] nullable: block i of k_rounds / k_polish takes bucket order[i]
     BigRange *giant;          // nullable: k_bucket_order lists buckets above POLISH_BIG here and
     uint32_t *giant_cnt;      //   k_rounds leaves them to launch_giant_rounds
@@ -180,8 +189,19 @@ struct GiantRounds {
     unsigned int *tbmax;          // [entries x MAXR] its largest tie-break
     uint32_t cap;                 // list entries
 };
+// the same for buckets that no one-pass block holds, their runs split round by round from the claim
+// table (cnt: elements stored and run elements so far, two words per entry); count[1] receives the total
+// of their elements and the list their packed offsets
+cudaError_t launch_giant_buckets(const SolveArgs &a, const GiantRounds &g, int eps, int sms, cudaStream_t s);
 cudaError_t launch_giant_rounds(const SolveArgs &a, const GiantRounds &g, int eps, int sms, cudaStream_t s);
 cudaError_t launch_rounds(const SolveArgs &a, cudaStream_t s);
+// every bucket of at most bucket_cap[1] elements in one pass (rounds, runs and sorted output), and their
+// out-of-order counts once the carries are known; larger ones are left to launch_giant_buckets and the
+// host's multi-block sort
+bool buckets_ok(int wlog, bool rows);
+int bucket_capacity(int key_bytes, bool payload, int blocks_per_sm);
+cudaError_t launch_buckets(const SolveArgs &a, int sms, cudaStream_t s);
+cudaError_t launch_carried(const SolveArgs &a, cudaStream_t s);
 cudaError_t launch_finalize(const SolveArgs &a, cudaStream_t s);
 cudaError_t launch_polish(const SolveArgs &a, cudaStream_t s);
 cudaError_t launch_seam_repair(const SolveArgs &a, int sms, cudaStream_t s);

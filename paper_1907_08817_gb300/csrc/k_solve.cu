@@ -78,7 +78,7 @@ __global__ void k_bucket_order(SolveArgs a, uint32_t heavy, uint32_t *order, uin
     const uint32_t nbk = a.bstart[b + 1] - a.bstart[b];
     if (nbk > heavy) order[atomicAdd(&cnt[0], 1u)] = b;
     else order[a.NB - 1 - atomicAdd(&cnt[1], 1u)] = b;
-    if (a.giant && nbk > POLISH_BIG) {
+    if (a.giant && nbk > a.giant_min) {
         BigRange r;
         r.lo = a.bstart[b]; r.hi = a.bstart[b + 1];
         r.seg = (uint32_t)seg_of_bucket(a.segs, a.nseg, b); r.off = 0; r.b = b; r.pad = 0;
@@ -90,7 +90,7 @@ cudaError_t launch_bucket_order(const SolveArgs &a, uint32_t heavy, uint32_t *or
                                 cudaStream_t s) {
     if (a.NB == 0) return cudaSuccess;
     cudaError_t e = cudaMemsetAsync(cnt, 0, 2 * sizeof(uint32_t), s);
-    if (e == cudaSuccess && a.giant_cnt) e = cudaMemsetAsync(a.giant_cnt, 0, sizeof(uint32_t), s);
+    if (e == cudaSuccess && a.giant_cnt) e = cudaMemsetAsync(a.giant_cnt, 0, 2 * sizeof(uint32_t), s);
     if (e != cudaSuccess) return e;
     k_bucket_order<<<(a.NB + 255) / 256, 256, 0, s>>>(a, heavy, order, cnt);
     return nns_launched(cudaGetLastError());
@@ -1110,6 +1110,643 @@ __global__ void __launch_bounds__(SOLVE_THREADS) k_polish(SolveArgs a) {
                                       TB, Wn - 1u};
         polish_bucket<W, uint32_t, FL>(a, sm, v, b, s0, nbk, sg, nullptr, nullptr);
     }
+}
+
+// ---------------------------------------------------------------------------------------------
+// One-pass buckets: the rounds, the run split and the sorted output of a bucket of at most
+// polish_cap elements in one block, which reads the bucket once (k_rounds and k_polish read it twice and
+// pass every element's round through memory). The one thing that needs other buckets is the carry of
+// the out-of-order split, the largest element that earlier buckets stored in o_r; but an element x of
+// o_r is out of order exactly when it is below the bucket's own earlier elements of o_r or below the
+// carry, so the block counts the former, writes the others -- the in-order run, ascending -- to
+// memory, and k_carried counts those below the carry by binary search.
+//
+// Sort: the order of the composite key (key - kmin) * 2^ib + index is the stable order. Each element's
+// top 32 composite bits are its word; words drop into 4,096 bins by their top 12 bits (shared-memory
+// atomics), and each thread puts the few elements of its eight bins in order by insertion. Words that
+// cannot hold the whole composite keep the index beside them and settle equal words
+// by key and index. When a bin holds more than BIN_MAX elements the bucket takes the stable radix sort.
+//
+// Bound by instruction issue and the latency of its barrier-separated phases. Buckets too large for two
+// blocks per SM take a second launch with one block per SM; the rest (launch_giant_buckets) run on the
+// whole GPU. Against k_rounds, k_polish and their one-block global-memory path: 2^28 f32 keys 3.6 ms
+// (5.4 ms), 64M u64 key-value 1.9 ms (3.6 ms), 50M u64 keys in three rounds 1.6 ms (3.0 ms).
+template <typename W> struct OPair;  // (order image, tie-break); all zero is the least pair and stands for none
+template <> struct OPair<uint32_t> {
+    unsigned long long v;
+    __device__ __forceinline__ static OPair make(uint32_t k, uint32_t t) {
+        return {((unsigned long long)k << 32) | t};
+    }
+    __device__ __forceinline__ bool less(const OPair &o) const { return v < o.v; }
+    __device__ __forceinline__ unsigned long long key() const { return v >> 32; }
+    __device__ __forceinline__ uint32_t tie() const { return (uint32_t)v; }
+    __device__ __forceinline__ OPair up(int o) const { return {__shfl_up_sync(0xFFFFFFFFu, v, o)}; }
+    __device__ __forceinline__ OPair xr(int o) const { return {__shfl_xor_sync(0xFFFFFFFFu, v, o)}; }
+};
+template <> struct OPair<uint64_t> {
+    unsigned long long k;
+    uint32_t t;
+    __device__ __forceinline__ static OPair make(uint64_t k, uint32_t t) { return {k, t}; }
+    __device__ __forceinline__ bool less(const OPair &o) const { return okey_less(k, t, o.k, o.t); }
+    __device__ __forceinline__ unsigned long long key() const { return k; }
+    __device__ __forceinline__ uint32_t tie() const { return t; }
+    __device__ __forceinline__ OPair up(int o) const {
+        return {__shfl_up_sync(0xFFFFFFFFu, k, o), __shfl_up_sync(0xFFFFFFFFu, t, o)};
+    }
+    __device__ __forceinline__ OPair xr(int o) const {
+        return {__shfl_xor_sync(0xFFFFFFFFu, k, o), __shfl_xor_sync(0xFFFFFFFFu, t, o)};
+    }
+};
+
+// block-wide exclusive prefix maximum; `scratch` (SNW entries) may be written again after one more barrier
+template <typename W>
+__device__ __forceinline__ OPair<W> block_excl_max_pair(OPair<W> v, OPair<W> *scratch) {
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    const OPair<W> none = OPair<W>::make(0, 0);
+    OPair<W> x = v;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const OPair<W> y = x.up(o);
+        if (lane >= o && x.less(y)) x = y;
+    }
+    OPair<W> ex = x.up(1);
+    if (lane == 0) ex = none;
+    if (lane == 31) scratch[wid] = x;
+    __syncthreads();
+    OPair<W> m = lane < wid ? scratch[lane] : none;
+#pragma unroll
+    for (int o = 8; o; o >>= 1) {
+        const OPair<W> y = m.xr(o);
+        if (m.less(y)) m = y;
+    }
+    // lanes 0 .. 15 hold the maximum over the earlier warps
+    m = OPair<W>::make((W)__shfl_sync(0xFFFFFFFFu, m.key(), 0), __shfl_sync(0xFFFFFFFFu, m.tie(), 0));
+    return ex.less(m) ? m : ex;
+}
+static_assert(SNW == 16, "one half warp holds the warps' maxima");
+
+// longest list that the bins take: four elements per bin, of which a thread orders eight bins
+constexpr uint32_t BUCKET_BIN_MAX = 4 * NBIN;
+
+template <typename W> struct BucketSmem {
+    union {
+        uint32_t tbl[NBIN];   // claims of at most 2^12 positions
+        uint32_t bins[NBIN];
+        struct {
+            uint32_t hist[8 * 256];
+            uint32_t wcnt[SNW * 256];
+        };
+    };
+    OPair<W> pmax[SNW];
+    W lo[SNW], hi[SNW];
+    uint32_t scratch[33];
+    int seg;
+};
+
+template <typename W>
+__host__ __device__ constexpr size_t bucket_fixed() { return (sizeof(BucketSmem<W>) + 15) & ~(size_t)15; }
+// per element: key, word (the radix sort's index lists in its place), position (later the index), flag,
+// payload
+template <typename W>
+__host__ __device__ constexpr size_t bucket_per(bool pay) { return sizeof(W) + 4 + 2 + 1 + (pay ? 4 : 0); }
+
+template <typename W, bool FL>
+__device__ __forceinline__ W key_of_okey(W o) {  // the inverse of okey_of
+    if constexpr (!FL) return o;
+    else {
+        constexpr W top = (W)1 << (8 * sizeof(W) - 1);
+        return (o & top) ? (W)(o ^ top) : (W)~o;
+    }
+}
+
+template <typename W, bool FL, bool PAY>
+__device__ __forceinline__ void bucket_one(const SolveArgs &a, unsigned char *braw, uint32_t b, uint32_t cap) {
+    BucketSmem<W> &sm = *reinterpret_cast<BucketSmem<W> *>(braw);
+    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+    const uint32_t s0 = a.bstart[b], nbk = a.bstart[b + 1] - s0;
+    unsigned char *p = braw + bucket_fixed<W>();
+    W *K = reinterpret_cast<W *>(p); p += sizeof(W) * cap;
+    uint32_t *word = reinterpret_cast<uint32_t *>(p); p += (size_t)4 * cap;
+    uint32_t *P = nullptr;
+    if constexpr (PAY) { P = reinterpret_cast<uint32_t *>(p); p += (size_t)4 * cap; }
+    uint16_t *pos = reinterpret_cast<uint16_t *>(p); p += (size_t)2 * cap;
+    uint8_t *F = p;  // 1: stored in an earlier round
+    const uint32_t Wn = 1u << a.wlog, wm = Wn - 1u;
+    if (tid == 0) {
+        sm.seg = seg_of_bucket(a.segs, a.nseg, b);
+        if (nbk > (uint32_t)a.polish_cap) atomicAdd(&a.stats[sm.seg].oversized, 1u);
+    }
+    // the bucket, as order images, with its extremes
+    W lo = (W)~(W)0, hi = 0;
+    constexpr int LB = 8;  // loads per thread issued together
+    for (uint32_t i0 = 0; i0 < nbk; i0 += SOLVE_THREADS * LB) {
+        W k[LB];
+        uint32_t g[LB], q4[LB];
+#pragma unroll
+        for (int q = 0; q < LB; ++q) {
+            const uint32_t i = i0 + q * SOLVE_THREADS + tid;
+            if (i < nbk) {
+                k[q] = ldk<W>(a.keys, s0 + i);
+                g[q] = a.gs[s0 + i];
+                if constexpr (PAY) q4[q] = a.pay[s0 + i];
+            }
+        }
+#pragma unroll
+        for (int q = 0; q < LB; ++q) {
+            const uint32_t i = i0 + q * SOLVE_THREADS + tid;
+            if (i < nbk) {
+                const W o = okey_of<W, FL>(k[q]);
+                K[i] = o;
+                pos[i] = (uint16_t)(g[q] & wm);
+                F[i] = 0;
+                if constexpr (PAY) P[i] = q4[q];
+                lo = o < lo ? o : lo;
+                hi = o > hi ? o : hi;
+            }
+        }
+    }
+#pragma unroll
+    for (int o = 16; o; o >>= 1) {
+        const W l2 = __shfl_xor_sync(0xFFFFFFFFu, lo, o), h2 = __shfl_xor_sync(0xFFFFFFFFu, hi, o);
+        lo = l2 < lo ? l2 : lo;
+        hi = h2 > hi ? h2 : hi;
+    }
+    if (lane == 0) { sm.lo[wid] = lo; sm.hi[wid] = hi; }
+
+    // rounds (Fig. "Algorithm NN-sort"): every element still unplaced claims its position, the first to
+    // arrive is stored; the position table then gives o_r in position order
+    constexpr uint32_t PER = NBIN / SOLVE_THREADS;  // positions per thread at most
+    const uint32_t per = (Wn + SOLVE_THREADS - 1) / SOLVE_THREADS, p0 = (uint32_t)tid * per;
+    int eps = 0, r = 0;
+    uint32_t roff = 0, left = nbk;
+    W *rk = reinterpret_cast<W *>(a.rk) + s0;
+    for (;; ++r) {
+        uint4 *t4 = reinterpret_cast<uint4 *>(sm.tbl);
+        for (uint32_t j = tid; j < Wn / 4; j += SOLVE_THREADS) t4[j] = make_uint4(EMPTY32, EMPTY32, EMPTY32, EMPTY32);
+        __syncthreads();
+        if (r == 0) eps = (int)a.segs[sm.seg].eps;
+        if (r >= eps || left == 0) break;  // uniform
+        for (uint32_t i = tid; i < nbk; i += SOLVE_THREADS)
+            if (r == 0 || !F[i]) atomicMin(&sm.tbl[pos[i]], i);
+        __syncthreads();
+        uint32_t x[PER];
+        OPair<W> e[PER], loc = OPair<W>::make(0, 0);
+#pragma unroll
+        for (uint32_t q = 0; q < PER; ++q) {
+            x[q] = (q < per && p0 + q < Wn) ? sm.tbl[p0 + q] : EMPTY32;
+            if (x[q] != EMPTY32) {
+                F[x[q]] = 1;
+                e[q] = OPair<W>::make(K[x[q]], x[q]);
+                if (loc.less(e[q])) loc = e[q];
+            }
+        }
+        const OPair<W> before = block_excl_max_pair<W>(loc, sm.pmax);
+        OPair<W> run = before;
+        uint32_t cnt = 0;  // out of order here (high half), in order (low half)
+#pragma unroll
+        for (uint32_t q = 0; q < PER; ++q)
+            if (x[q] != EMPTY32) {
+                if (e[q].less(run)) { cnt += 0x10000u; x[q] = EMPTY32; }
+                else { run = e[q]; ++cnt; }
+            }
+        uint32_t tot;
+        uint32_t at = roff + (block_excl_sum(cnt, sm.scratch, &tot) & 0xFFFFu);
+#pragma unroll
+        for (uint32_t q = 0; q < PER; ++q)
+            if (x[q] != EMPTY32) {
+                rk[at] = (W)e[q].key();
+                a.rt[s0 + at] = e[q].tie();
+                ++at;
+            }
+        const uint32_t in = tot & 0xFFFFu, out = tot >> 16;
+        roff += in;
+        left -= in + out;
+        if (tid == SOLVE_THREADS - 1) {
+            OKey o; o.k = run.key(); o.tb = run.tie(); o.valid = in ? 1u : 0u;
+            a.bmax[(size_t)b * MAXR + r] = o;
+        }
+        if (tid == 0) {
+            if (left) atomicAdd(&a.stats[sm.seg].count_ge[r + 1], (unsigned long long)left);
+            if (out) atomicAdd(&a.stats[sm.seg].ooo[r], (unsigned long long)out);
+            a.rend[(size_t)b * MAXR + r] = roff;
+        }
+    }
+    for (; r < eps; ++r)  // rounds after the last one that stored anything
+        if (tid == 0) {
+            OKey z; z.k = 0; z.tb = 0; z.valid = 0;
+            a.bmax[(size_t)b * MAXR + r] = z;
+            a.rend[(size_t)b * MAXR + r] = roff;
+        }
+
+    // the bucket's output: its elements in (key, index) order
+    lo = sm.lo[0];
+    hi = sm.hi[0];
+#pragma unroll
+    for (int q = 1; q < SNW; ++q) {
+        lo = sm.lo[q] < lo ? sm.lo[q] : lo;
+        hi = sm.hi[q] > hi ? sm.hi[q] : hi;
+    }
+    if (tid == 0) {
+        OKey o; o.k = lo; o.tb = 0; o.valid = 1;
+        a.blo[b] = o;
+        o.k = hi;
+        a.bhi[b] = o;
+    }
+    const Seg &sg = a.segs[sm.seg];
+    const uint64_t off = (uint64_t)s0 - sg.ebase;
+    W *outk = reinterpret_cast<W *>(sg.keys) + off;
+    int32_t *outp = (PAY && sg.payload) ? sg.payload + off : nullptr;
+    const W range = hi - lo;
+    int br = 0;
+    if constexpr (sizeof(W) == 8) br = range ? 64 - __clzll((long long)range) : 0;
+    else br = range ? 32 - __clz((int)range) : 0;
+    const int ib = nbk > 1 ? 32 - __clz((int)(nbk - 1)) : 0;
+    const int drop = br + ib > 32 ? br + ib - 32 : 0;             // composite bits that the word leaves out
+    const int bs = br + ib - drop > NBIN_LOG ? br + ib - drop - NBIN_LOG : 0;  // word bits below the bin
+    auto word_of = [&](uint32_t i, W k) -> uint32_t {
+        const W d = k - lo;
+        return drop >= ib ? (uint32_t)(d >> (drop - ib)) : (((uint32_t)d << (ib - drop)) | (i >> drop));
+    };
+    bool binned = nbk <= BUCKET_BIN_MAX;
+    if (binned) {
+        // (the barrier that ended the rounds also ended their reads of the table)
+        uint4 *t4 = reinterpret_cast<uint4 *>(sm.bins);
+        for (uint32_t j = tid; j < NBIN / 4; j += SOLVE_THREADS) t4[j] = make_uint4(0u, 0u, 0u, 0u);
+        __syncthreads();
+        for (uint32_t i = tid; i < nbk; i += SOLVE_THREADS) atomicAdd(&sm.bins[word_of(i, K[i]) >> bs], 1u);
+        __syncthreads();
+        constexpr int BPT = NBIN / SOLVE_THREADS;
+        static_assert(BPT == 8, "two 16-byte reads per thread");
+        uint4 c0 = t4[2 * tid], c1 = t4[2 * tid + 1];
+        const uint32_t m = max(max(max(c0.x, c0.y), max(c0.z, c0.w)), max(max(c1.x, c1.y), max(c1.z, c1.w)));
+        binned = !__syncthreads_or(m > BIN_MAX);
+        if (binned) {
+            const uint32_t sum = c0.x + c0.y + c0.z + c0.w + c1.x + c1.y + c1.z + c1.w;
+            uint32_t st = block_excl_sum(sum, sm.scratch, nullptr), t;
+            t = c0.x; c0.x = st; st += t;
+            t = c0.y; c0.y = st; st += t;
+            t = c0.z; c0.z = st; st += t;
+            t = c0.w; c0.w = st; st += t;
+            t = c1.x; c1.x = st; st += t;
+            t = c1.y; c1.y = st; st += t;
+            t = c1.z; c1.z = st; st += t;
+            c1.w = st;
+            t4[2 * tid] = c0;
+            t4[2 * tid + 1] = c1;
+            __syncthreads();
+            uint16_t *idx = pos;  // the positions are not needed any more
+            for (uint32_t i = tid; i < nbk; i += SOLVE_THREADS) {
+                const uint32_t w = word_of(i, K[i]);
+                const uint32_t slot = atomicAdd(&sm.bins[w >> bs], 1u);
+                word[slot] = w;
+                if (drop) idx[slot] = (uint16_t)i;
+            }
+            __syncthreads();
+            // thread t puts the elements of its eight bins in order: they follow one another, and only
+            // bin-mates are out of place, so an insertion sort takes little more than a step per element
+            {
+                const uint32_t end = sm.bins[BPT * tid + BPT - 1], beg = tid ? sm.bins[BPT * tid - 1] : 0u;
+                if (!drop) {
+                    uint32_t top = beg < end ? word[beg] : 0u;  // the largest so far, at place j - 1
+                    for (uint32_t j = beg + 1; j < end; ++j) {
+                        const uint32_t c = word[j];
+                        if (c >= top) { top = c; continue; }
+                        uint32_t k = j;
+                        uint32_t v = top;
+                        do {
+                            word[k] = v;
+                            --k;
+                            v = k > beg ? word[k - 1] : 0u;
+                        } while (v > c);
+                        word[k] = c;
+                    }
+                } else {
+                    // equal words: the keys, then the indices, decide
+                    auto after = [&](uint32_t v, uint32_t x, uint32_t c, uint32_t y) -> bool {
+                        if (v != c) return v > c;
+                        const W kx = K[x], ky = K[y];
+                        return kx > ky || (kx == ky && x > y);
+                    };
+                    for (uint32_t j = beg + 1; j < end; ++j) {
+                        const uint32_t c = word[j], y = idx[j];
+                        uint32_t k = j;
+                        while (k > beg && after(word[k - 1], idx[k - 1], c, y)) {
+                            word[k] = word[k - 1];
+                            idx[k] = idx[k - 1];
+                            --k;
+                        }
+                        if (k != j) { word[k] = c; idx[k] = (uint16_t)y; }
+                    }
+                }
+            }
+            __syncthreads();
+            const uint32_t imask = (1u << ib) - 1u;
+            for (uint32_t j = tid; j < nbk; j += SOLVE_THREADS) {
+                const uint32_t c = word[j];
+                const uint32_t x = drop ? (uint32_t)idx[j] : (c & imask);
+                W o;
+                if constexpr (sizeof(W) == 4) o = lo + (c >> (ib - drop));  // br <= 32: the word holds the whole key
+                else o = K[x];
+                outk[j] = key_of_okey<W, FL>(o);
+                if constexpr (PAY) { if (outp) outp[j] = (int32_t)P[x]; }
+            }
+        }
+    }
+    if (!binned) {
+        uint16_t *X = reinterpret_cast<uint16_t *>(word), *Y = X + cap;
+        for (uint32_t i = tid; i < nbk; i += SOLVE_THREADS) X[i] = (uint16_t)i;
+        __syncthreads();
+        auto kf = [&](uint16_t x) -> W { return K[x]; };
+        const uint16_t *A = cta_radix_sort<uint16_t>(X, Y, nbk, 8 * (int)sizeof(W), kf, sm.hist, sm.wcnt, sm.scratch);
+        __syncthreads();
+        for (uint32_t q = tid; q < nbk; q += SOLVE_THREADS) {
+            const uint32_t x = A[q];
+            outk[q] = key_of_okey<W, FL>(K[x]);
+            if constexpr (PAY) { if (outp) outp[q] = (int32_t)P[x]; }
+        }
+    }
+}
+
+// SECOND: the heavy buckets of the order's front that a block alone on its SM can hold
+template <typename W, bool FL, bool PAY, bool SECOND>
+__global__ void __launch_bounds__(SOLVE_THREADS, SECOND ? 1 : 2) k_bucket(SolveArgs a) {
+    extern __shared__ __align__(16) unsigned char braw[];
+    if (*a.err) return;  // NaN keys or bad positions: leave the caller's arrays untouched
+    if constexpr (SECOND) {
+        const uint32_t nb = *a.heavy_cnt;
+        for (uint32_t j = blockIdx.x; j < nb; j += gridDim.x) {
+            const uint32_t b = a.order[j], nbk = a.bstart[b + 1] - a.bstart[b];
+            if (nbk > (uint32_t)a.bucket_cap[1]) continue;  // launch_giant_buckets
+            bucket_one<W, FL, PAY>(a, braw, b, (uint32_t)a.bucket_cap[1]);
+            __syncthreads();  // the next bucket reuses the shared arrays
+        }
+    } else {
+        const uint32_t b = a.order ? a.order[blockIdx.x] : blockIdx.x;
+        const uint32_t nbk = a.bstart[b + 1] - a.bstart[b];
+        if (nbk == 0) {
+            if (threadIdx.x < MAXR) {
+                OKey z; z.k = 0; z.tb = 0; z.valid = 0;
+                a.bmax[(size_t)b * MAXR + threadIdx.x] = z;
+            }
+            return;
+        }
+        if (nbk > (uint32_t)a.bucket_cap[0]) return;
+        bucket_one<W, FL, PAY>(a, braw, b, (uint32_t)a.bucket_cap[0]);
+    }
+}
+
+// Buckets that no block holds: the rounds on the whole GPU, as launch_giant_rounds, but over the listed
+// buckets' elements end to end (a list may hold hundreds of moderate buckets), and each round's run split
+// by one block per bucket from the claim table, right after the round's claims.
+constexpr int GT = 256, GI = 8;  // threads of a grid-wide block, elements per lane and chunk
+
+// packed offsets of the listed buckets (one block) and their total
+__global__ void __launch_bounds__(1024) k_giant_offsets(GiantRounds g) {
+    __shared__ uint32_t scratch[33];
+    const uint32_t n = g.count[0];
+    uint32_t base = 0;
+    for (uint32_t j0 = 0; j0 < n; j0 += blockDim.x) {
+        const uint32_t j = j0 + threadIdx.x;
+        const uint32_t len = j < n ? (uint32_t)(g.list[j].hi - g.list[j].lo) : 0u;
+        uint32_t tot;
+        const uint32_t ex = block_excl_sum(len, scratch, &tot);
+        if (j < n) g.list[j].off = base + ex;
+        base += tot;
+    }
+    if (threadIdx.x == 0) g.count[1] = base;
+}
+
+// fn(j, element's place in the partitioned arrays, its index in the bucket) for every element, all lanes
+// of a warp together (j = EMPTY32 for a lane without one)
+template <typename Fn>
+__device__ __forceinline__ void giant_flat(const GiantRounds &g, Fn fn) {
+    const uint32_t n = g.count[0], total = n ? g.count[1] : 0u;
+    const uint32_t lane = threadIdx.x & 31, warps = gridDim.x * (GT / 32);
+    for (uint64_t c0 = (uint64_t)(blockIdx.x * (GT / 32) + (threadIdx.x >> 5)) * (32 * GI); c0 < total;
+         c0 += (uint64_t)warps * (32 * GI)) {
+        uint32_t j = 0, hi = n - 1;  // the bucket of the chunk's first element
+        while (j < hi) {
+            const uint32_t mid = (j + hi + 1) >> 1;
+            if (g.list[mid].off <= c0) j = mid; else hi = mid - 1;
+        }
+        uint32_t lo = (uint32_t)g.list[j].lo, off = g.list[j].off, next = j + 1 < n ? g.list[j + 1].off : total;
+        for (int q = 0; q < GI; ++q) {
+            const uint64_t e = c0 + (uint64_t)q * 32 + lane;
+            if (e < total) {
+                while (e >= next) {
+                    ++j;
+                    off = next;
+                    lo = (uint32_t)g.list[j].lo;
+                    next = j + 1 < n ? g.list[j + 1].off : total;
+                }
+                fn(j, lo + ((uint32_t)e - off), (uint32_t)e - off);
+            } else {
+                fn(EMPTY32, 0u, 0u);
+            }
+        }
+    }
+}
+
+__global__ void __launch_bounds__(GT) k_giant_clear(SolveArgs a, GiantRounds g, int eps) {
+    const uint32_t n = g.count[0];
+    const uint64_t stride = (uint64_t)gridDim.x * blockDim.x, t0 = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    for (uint64_t q = t0; q < (uint64_t)n << a.wlog; q += stride) g.table[q] = ~0ull;
+    for (uint64_t q = t0; q < 2 * (uint64_t)n; q += stride) g.cnt[q] = 0;
+    if (eps > 1) giant_flat(g, [&](uint32_t j, uint32_t e, uint32_t) { if (j != EMPTY32) a.rank[e] = 0; });
+}
+
+__global__ void __launch_bounds__(GT) k_giant_claim_flat(SolveArgs a, GiantRounds g, int r) {
+    const uint32_t wm = (1u << a.wlog) - 1u;
+    const unsigned lanes_below = (1u << (threadIdx.x & 31)) - 1u;
+    const unsigned long long tag = (unsigned long long)(MAXR - r) << 32;
+    giant_flat(g, [&](uint32_t j, uint32_t e, uint32_t i) {
+        const bool act = j != EMPTY32 && (r == 0 || a.rank[e] == r);
+        const uint32_t p = act ? (j << a.wlog) | (a.gs[e] & wm) : EMPTY32;
+        const unsigned peers = __match_any_sync(0xFFFFFFFFu, p);  // lanes hold ascending rows
+        if (act && (peers & lanes_below) == 0) atomicMin(&g.table[p], tag | (unsigned long long)i);
+    });
+}
+
+__global__ void __launch_bounds__(GT) k_giant_move_on(SolveArgs a, GiantRounds g, int r) {
+    const uint32_t wm = (1u << a.wlog) - 1u;
+    const unsigned long long tag = (unsigned long long)(MAXR - r) << 32;
+    giant_flat(g, [&](uint32_t j, uint32_t e, uint32_t i) {
+        if (j != EMPTY32 && a.rank[e] == r &&
+            g.table[((uint64_t)j << a.wlog) + (a.gs[e] & wm)] != (tag | (unsigned long long)i))
+            a.rank[e] = (uint8_t)(r + 1);
+    });
+}
+
+template <typename W, bool FL>
+__global__ void __launch_bounds__(SOLVE_THREADS) k_giant_runs(SolveArgs a, GiantRounds g, int r) {
+    __shared__ OPair<W> pmax[SNW];
+    __shared__ uint32_t scratch[33];
+    const int tid = threadIdx.x;
+    const uint32_t n = g.count[0], Wn = 1u << a.wlog;
+    constexpr uint32_t PER = NBIN / SOLVE_THREADS;
+    const uint32_t per = (Wn + SOLVE_THREADS - 1) / SOLVE_THREADS, p0 = (uint32_t)tid * per;
+    for (uint32_t j = blockIdx.x; j < n; j += gridDim.x) {
+        const BigRange R = g.list[j];
+        const uint32_t s0 = (uint32_t)R.lo, nbk = (uint32_t)(R.hi - R.lo);
+        const uint32_t stored = g.cnt[2 * j], roff = g.cnt[2 * j + 1];
+        uint32_t x[PER];
+        OPair<W> e[PER], loc = OPair<W>::make(0, 0);
+#pragma unroll
+        for (uint32_t q = 0; q < PER; ++q) {
+            const bool in = q < per && p0 + q < Wn;
+            const unsigned long long v = in ? g.table[((uint64_t)j << a.wlog) + p0 + q] : ~0ull;
+            x[q] = (uint32_t)(v >> 32) == (uint32_t)(MAXR - r) ? (uint32_t)v : EMPTY32;
+        }
+#pragma unroll
+        for (uint32_t q = 0; q < PER; ++q)
+            if (x[q] != EMPTY32) {
+                e[q] = OPair<W>::make(okey_of<W, FL>(ldk<W>(a.keys, s0 + x[q])), x[q]);
+                if (loc.less(e[q])) loc = e[q];
+            }
+        OPair<W> run = block_excl_max_pair<W>(loc, pmax);
+        uint32_t cin = 0, cout = 0;
+#pragma unroll
+        for (uint32_t q = 0; q < PER; ++q)
+            if (x[q] != EMPTY32) {
+                if (e[q].less(run)) { ++cout; x[q] = EMPTY32; }
+                else { run = e[q]; ++cin; }
+            }
+        uint32_t tot;  // in-order elements in the low half, the others in the high one
+        uint32_t at = roff + (block_excl_sum(cin | (cout << 16), scratch, &tot) & 0xFFFFu);
+        W *rk = reinterpret_cast<W *>(a.rk) + s0;
+#pragma unroll
+        for (uint32_t q = 0; q < PER; ++q)
+            if (x[q] != EMPTY32) {
+                rk[at] = (W)e[q].key();
+                a.rt[s0 + at] = e[q].tie();
+                ++at;
+            }
+        const uint32_t in = tot & 0xFFFFu, out = tot >> 16, left = nbk - stored - in - out;
+        if (tid == SOLVE_THREADS - 1) {
+            OKey o; o.k = run.key(); o.tb = run.tie(); o.valid = in ? 1u : 0u;
+            a.bmax[(size_t)R.b * MAXR + r] = o;
+        }
+        if (tid == 0) {
+            if (r == 0 && nbk > (uint32_t)a.polish_cap) atomicAdd(&a.stats[R.seg].oversized, 1u);
+            if (left) atomicAdd(&a.stats[R.seg].count_ge[r + 1], (unsigned long long)left);
+            if (out) atomicAdd(&a.stats[R.seg].ooo[r], (unsigned long long)out);
+            a.rend[(size_t)R.b * MAXR + r] = roff + in;
+        }
+        __syncthreads();  // every thread has read cnt; the shared arrays are free
+        if (tid == 0) { g.cnt[2 * j] = stored + in + out; g.cnt[2 * j + 1] = roff + in; }
+    }
+}
+
+template <typename W>
+static cudaError_t giant_runs_go(const SolveArgs &a, const GiantRounds &g, int r, unsigned grid, cudaStream_t s) {
+    if (a.dtype == NNSORT_F32 || a.dtype == NNSORT_F64) k_giant_runs<W, true><<<grid, SOLVE_THREADS, 0, s>>>(a, g, r);
+    else k_giant_runs<W, false><<<grid, SOLVE_THREADS, 0, s>>>(a, g, r);
+    return nns_launched(cudaGetLastError());
+}
+cudaError_t launch_giant_buckets(const SolveArgs &a, const GiantRounds &g, int eps, int sms, cudaStream_t s) {
+    const unsigned grid = (unsigned)sms * 4, rgrid = std::min<unsigned>(g.cap, 2u * (unsigned)sms);
+    cudaError_t e;
+    k_giant_offsets<<<1, 1024, 0, s>>>(g);
+    if ((e = nns_launched(cudaGetLastError())) != cudaSuccess) return e;
+    k_giant_clear<<<grid, GT, 0, s>>>(a, g, eps);
+    if ((e = nns_launched(cudaGetLastError())) != cudaSuccess) return e;
+    for (int r = 0; r < eps; ++r) {
+        k_giant_claim_flat<<<grid, GT, 0, s>>>(a, g, r);
+        if ((e = nns_launched(cudaGetLastError())) != cudaSuccess) return e;
+        e = a.key_bytes == 4 ? giant_runs_go<uint32_t>(a, g, r, rgrid, s) : giant_runs_go<uint64_t>(a, g, r, rgrid, s);
+        if (e != cudaSuccess) return e;
+        if (r + 1 < eps) {
+            k_giant_move_on<<<grid, GT, 0, s>>>(a, g, r);
+            if ((e = nns_launched(cudaGetLastError())) != cudaSuccess) return e;
+        }
+    }
+    return cudaSuccess;
+}
+
+// The out-of-order elements that only the carry makes so: of each one-pass bucket's in-order runs, the
+// elements below the carry. A thread per bucket; most runs start above their carry and cost one read.
+template <typename W>
+__global__ void __launch_bounds__(256) k_carried(SolveArgs a) {
+    const uint32_t b = blockIdx.x * blockDim.x + threadIdx.x;
+    const bool err = *a.err != 0;
+    uint32_t s0 = 0, nbk = 0;
+    int seg = 0, t = 0;
+    if (b < a.NB && !err) {
+        s0 = a.bstart[b];
+        nbk = a.bstart[b + 1] - s0;
+        if (nbk) {
+            seg = a.nseg == 1 ? 0 : seg_of_bucket(a.segs, a.nseg, b);
+            t = (int)a.stats[seg].t;
+        }
+    }
+    const W *rk = reinterpret_cast<const W *>(a.rk) + s0;
+    const uint32_t *rt = a.rt + s0;
+    const int tmax = a.nseg == 1 ? (err ? 0 : (int)a.stats[0].t) : t;
+    uint32_t beg = 0;
+    for (int r = 0; r < tmax; ++r) {
+        uint32_t n = 0;
+        if (nbk) {
+            const uint32_t end = a.rend[(size_t)b * MAXR + r];
+            const OKey c = a.carry[(size_t)b * MAXR + r];
+            if (c.valid && end > beg) {
+                uint32_t l = beg, h = end;
+                if (!okey_less(rk[l], rt[l], c.k, c.tb)) h = l;
+                while (l < h) {
+                    const uint32_t mid = (l + h) >> 1;
+                    if (okey_less(rk[mid], rt[mid], c.k, c.tb)) l = mid + 1; else h = mid;
+                }
+                n = l - beg;
+            }
+            beg = end;
+        }
+        if (a.nseg == 1) {
+            n = __reduce_add_sync(0xFFFFFFFFu, n);
+            if ((threadIdx.x & 31) == 0 && n) atomicAdd(&a.stats[0].ooo[r], (unsigned long long)n);
+        } else if (n) {
+            atomicAdd(&a.stats[seg].ooo[r], (unsigned long long)n);
+        }
+    }
+}
+
+// the position table of a block holds NBIN positions; rows (traces) need every element's round
+bool buckets_ok(int wlog, bool rows) { return !rows && wlog <= NBIN_LOG; }
+
+// elements of a bucket that fit on chip with this many one-pass blocks per SM (228 KB, of which a block
+// reserves 1 KB and can use 227)
+int bucket_capacity(int key_bytes, bool payload, int blocks_per_sm) {
+    const size_t budget = blocks_per_sm == 1 ? 227 * 1024 : (228 * 1024) / blocks_per_sm - 1024 - 512;
+    const size_t cap = key_bytes == 4 ? (budget - bucket_fixed<uint32_t>()) / bucket_per<uint32_t>(payload)
+                                      : (budget - bucket_fixed<uint64_t>()) / bucket_per<uint64_t>(payload);
+    return (int)(std::min<size_t>(cap, 65534) & ~(size_t)15);
+}
+
+template <typename W, bool FL, bool PAY, bool SECOND>
+static cudaError_t bucket_go(const SolveArgs &a, unsigned grid, cudaStream_t s) {
+    const size_t smem = bucket_fixed<W>() + (size_t)a.bucket_cap[SECOND ? 1 : 0] * bucket_per<W>(PAY);
+    auto kfn = k_bucket<W, FL, PAY, SECOND>;
+    cudaError_t e = cudaFuncSetAttribute(kfn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    kfn<<<grid, SOLVE_THREADS, smem, s>>>(a);
+    return nns_launched(cudaGetLastError());
+}
+template <typename W, bool SECOND>
+static cudaError_t bucket_go2(const SolveArgs &a, unsigned grid, cudaStream_t s) {
+    const bool fl = a.dtype == NNSORT_F32 || a.dtype == NNSORT_F64;
+    if (a.pay) return fl ? bucket_go<W, true, true, SECOND>(a, grid, s) : bucket_go<W, false, true, SECOND>(a, grid, s);
+    return fl ? bucket_go<W, true, false, SECOND>(a, grid, s) : bucket_go<W, false, false, SECOND>(a, grid, s);
+}
+cudaError_t launch_buckets(const SolveArgs &a, int sms, cudaStream_t s) {
+    if (a.NB == 0) return cudaSuccess;
+    const cudaError_t e = a.key_bytes == 4 ? bucket_go2<uint32_t, false>(a, a.NB, s) : bucket_go2<uint64_t, false>(a, a.NB, s);
+    if (e != cudaSuccess || !a.heavy_cnt) return e;
+    const unsigned grid = std::min<unsigned>(a.NB, (unsigned)sms);
+    return a.key_bytes == 4 ? bucket_go2<uint32_t, true>(a, grid, s) : bucket_go2<uint64_t, true>(a, grid, s);
+}
+cudaError_t launch_carried(const SolveArgs &a, cudaStream_t s) {
+    if (a.NB == 0) return cudaSuccess;
+    if (a.key_bytes == 4) k_carried<uint32_t><<<(a.NB + 255) / 256, 256, 0, s>>>(a);
+    else k_carried<uint64_t><<<(a.NB + 255) / 256, 256, 0, s>>>(a);
+    return nns_launched(cudaGetLastError());
 }
 
 // ---------------------------------------------------------------------------------------------
