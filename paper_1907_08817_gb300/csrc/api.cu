@@ -863,6 +863,7 @@ int run_sort(const std::vector<SegIn> &in, const nnsort_sort_opts *op, int dtype
     pa.dtype = dtype;
     pa.pwl = pwl_dev;
     pa.single_model = (single && f0 && !o.d_slots) ? 1 : 0;
+    pa.host_seg = &P.segs[0];
     pa.host_pad = f0 ? f0->hpad.data() : nullptr;
     const PadArch arch = f0 ? f0->pad : pad_arch(1, 8, 0);
     const int prec = f0 ? o.precision : NNSORT_PREC_FP32;
@@ -1272,6 +1273,7 @@ int nnsort_predict(const void *d_keys, uint64_t n, int32_t dtype, const nnsort_m
     pa.dtype = dtype;
     pa.pwl = pwl_dev;
     pa.single_model = 1;
+    pa.host_seg = &P.segs[0];
     pa.host_pad = f->hpad.data();
     w->last_err = err;
     cudaError_t e = launch_predict(f->pad, precision, pa, sm_count(), stream);

@@ -68,6 +68,7 @@ struct PredictArgs {
     int dtype;
     PwlDev pwl;              // NNSORT_PREC_PWL (single array)
     int single_model;        // 1: one array whose positions come from its model (no injected slots)
+    const Seg *host_seg;     // single_model: the array's segment in host memory
     const float *host_pad;   // single_model: that model's padded parameters in host memory
 };
 cudaError_t launch_predict(const PadArch &a, int precision, const PredictArgs &p, int sms,

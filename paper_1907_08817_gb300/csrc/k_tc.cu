@@ -341,53 +341,50 @@ __global__ void __launch_bounds__(TC_THREADS) k_predict_bf16(PredictArgs a) {
 
 // ---------------------------------------------------------------------------------------------
 // One array, one model: NG independent groups of 4 warps per block and one block per SM. Group g
-// has its own A tile(s), accumulator columns [g H, (g + 1) H), mbarrier and named barrier (1 + g)
-// and walks its own sub-tiles of 128 keys; the B tile(s) and the parameters are staged once per
-// block and shared. The A tiles are then the only per-group shared memory, so NG = 6 groups fit
-// on an SM (24 warps, against 16 for blocks that each hold a W2 copy), and no block-wide barrier
-// separates one sub-tile from the next.
-constexpr int TC_NG = 6;
+// has its own A tiles (KPT keys per thread), accumulator columns, mbarrier and named barrier (1 + g) and
+// walks its own sub-tiles of KPT x 128 keys; the B tile(s) and the bias slabs are staged once per block
+// and shared. No block-wide barrier separates one sub-tile from the next.
+//
+// Bound by the CUDA-core work around the tensor layer, the ALU pipe (conversions, masks, maxima at two
+// cycles each) above all. 2^28 keys of 1-64-64-1, split form: 6.94 ms with the ALU pipe 67% busy and 630
+// instructions per key; ReLU as z + |z| on the FMA pipe 5.96 ms; the truncated part's low half shifted out
+// of the packed word instead of masked 5.82 ms; two keys per thread, which share the reads of the
+// launch constants (492 instructions per key), with three groups instead of six 5.64 ms; the epilogue's
+// columns loaded ahead 5.43 ms. 1-32-32-1 on 67M u64 keys: 1.26 ms, now 0.88 ms (six groups fit).
 
 __device__ __forceinline__ void grp_sync(int id) {
     asm volatile("bar.sync %0, %1;" ::"r"(id), "n"(TC_THREADS) : "memory");
 }
-// OR of v over the 128 threads of named barrier id (a barrier as well)
-__device__ __forceinline__ bool grp_or(int id, bool v) {
-    uint32_t r;
-    asm volatile(
-        "{\n\t.reg .pred p, q;\n\t"
-        "setp.ne.u32 p, %1, 0;\n\t"
-        "bar.red.or.pred q, %2, %3, p;\n\t"
-        "selp.u32 %0, 1, 0, q;\n\t}"
-        : "=r"(r)
-        : "r"((uint32_t)v), "r"(id), "n"(TC_THREADS)
-        : "memory");
-    return r != 0;
-}
-
 // the first and last layers' parameters as launch constants: every thread reads them through the
 // constant cache (one broadcast per warp instruction, no shared-memory traffic)
 struct TcConst {
-    float w1[64], b1[64], w3[64], b3;
+    float w1[64], b1[64], w3h[64], b3;  // w3h: W3 / 2
+    float xlim;  // inputs up to this magnitude keep every z far from overflow (negative: none does)
+    float nm_hi, nm_lo;
+    uint32_t gs_base;
+    uint64_t n, ebase, L;
+    const void *keys;
+    const int32_t *payload;
+    Norm norm;
 };
 
-template <int H, bool SPLIT, int NG>
+template <int H, bool SPLIT, int NG, int KPT>
 __host__ __device__ constexpr size_t tcmg_smem_bytes() {
-    return (size_t)NG * (SPLIT ? 2 : 1) * TC_M * H * 2 + (size_t)(SPLIT ? 2 : 1) * H * H * 2 +
-           (size_t)TC_M * 16 * 2 + (size_t)H * 16 * 2 + (size_t)(4 * H + 4) * 4;
+    return (size_t)NG * KPT * (SPLIT ? 2 : 1) * TC_M * H * 2 + (size_t)(SPLIT ? 2 : 1) * H * H * 2 +
+           (size_t)TC_M * 16 * 2 + (size_t)H * 16 * 2;
 }
 
-template <int H, typename W, bool SPLIT, int NG>
+template <int H, typename W, bool SPLIT, int NG, int KPT>
 __global__ void __launch_bounds__(NG * TC_THREADS, 1) k_predict_bf16_mg(PredictArgs a, const TcConst cst) {
     static_assert(H == 16 || H == 32 || H == 64, "tensor path widths");
-    static_assert(NG * H <= 512, "accumulators fit in tensor memory");
+    static_assert(NG * KPT * H <= 512, "accumulators fit in tensor memory");
     constexpr int NT = SPLIT ? 2 : 1;
     constexpr uint32_t TILE_B = TC_M * H * 2;
     constexpr uint32_t LBO = 128;
     constexpr uint32_t SBO = (H / 8) * 128;
-    constexpr int NCOL = NG * H <= 128 ? 128 : (NG * H <= 256 ? 256 : 512);
+    constexpr int NCOL = NG * KPT * H <= 128 ? 128 : (NG * KPT * H <= 256 ? 256 : 512);
     extern __shared__ __align__(1024) unsigned char sm[];
-    unsigned char *sB = sm + NG * NT * TILE_B;
+    unsigned char *sB = sm + NG * KPT * NT * TILE_B;
     unsigned char *sB16 = sB + H * H * 2;
     unsigned char *sOnes = sB + NT * H * H * 2;                       // TC_M x 16 bf16
     unsigned char *sBias = sOnes + TC_M * 16 * 2;                     // H x 16 bf16
@@ -401,136 +398,197 @@ __global__ void __launch_bounds__(NG * TC_THREADS, 1) k_predict_bf16_mg(PredictA
         for (int g = 0; g < NG; ++g) mbar_init(smem_u32(&bar[g]), 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
-    const Seg &sg = a.segs[0];
     {   // W2 (row = output unit, K = input unit) -> canonical K-major layout; bias slabs
-        const float *W2 = sg.params + 2 * H;
+        const float *params = a.segs[0].params, *W2 = params + 2 * H;
         for (int e = tid; e < H * H; e += NG * TC_THREADS) {
             const int nrow = e / H, k = e % H;
             const uint32_t off = (nrow / 8) * SBO + (k / 8) * LBO + (nrow % 8) * 16 + (k % 8) * 2;
             *reinterpret_cast<__nv_bfloat16 *>(sB + off) = __float2bfloat16_rn(W2[e]);
             if (SPLIT) *reinterpret_cast<__half *>(sB16 + off) = __float2half_rn(W2[e]);
         }
-        fill_bias_slabs<H>(sOnes, sBias, sg.params + 2 * H + H * H, tid, NG * TC_THREADS);
+        fill_bias_slabs<H>(sOnes, sBias, params + 2 * H + H * H, tid, NG * TC_THREADS);
     }
     fence_async_smem();
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    const uint32_t tbase = tmem_base;
-    const uint32_t dcol = tbase + (uint32_t)(grp * H);
+    const uint32_t dcol = tmem_base + (uint32_t)(grp * KPT * H);
     const uint32_t lane_addr = dcol + ((uint32_t)((warp & 3) * 32) << 16);
     const uint32_t aoff = (gt / 8) * SBO + (gt % 8) * 16;
-    unsigned char *myA = sm + grp * NT * TILE_B;
+    unsigned char *myA = sm + grp * KPT * NT * TILE_B;  // KPT x (hi tile, lo tile)
     const uint32_t mybar = smem_u32(&bar[grp]);
     const int bid = 1 + grp;
     const uint32_t idesc = idesc_bf16(TC_M, H);
     const uint32_t idesc_lo = idesc_f16(TC_M, H);
+    // descriptors of the first K step; later steps add a constant to the start address field
+    const uint64_t dA = mdesc(smem_u32(myA), LBO, SBO), dB = mdesc(smem_u32(sB), LBO, SBO);
+    const uint64_t dOnes = mdesc(smem_u32(sOnes), SLAB_LBO, SLAB_SBO), dBias = mdesc(smem_u32(sBias), SLAB_LBO, SLAB_SBO);
+    constexpr uint64_t KSTEP = (2 * LBO) >> 4;
     uint32_t phase = 0, err = 0, dead_parity = 0;
     bool dead = false;
-    const uint64_t n = sg.n;
-    const uint64_t total = (n + TC_M - 1) / TC_M;
-    const uint64_t stride = (uint64_t)gridDim.x * NG;
-    const W *keys = reinterpret_cast<const W *>(sg.keys);
-    uint64_t pre = 0, pre_st = ~0ull;
-    for (uint64_t st = (uint64_t)blockIdx.x * NG + grp; st < total; st += stride) {
-        const uint64_t i = st * TC_M + gt;
-        const bool valid = i < n;
-        const uint64_t wv = !valid ? 0ull : (pre_st == st ? pre : word64(keys[i]));
-        if (valid && key_is_nan(wv, a.dtype)) err |= ERR_NAN;
-        {   // the group's next sub-tile's keys, loaded while this one is computed
-            const uint64_t st2 = st + stride;
-            if (st2 < total) {
-                const uint64_t i2 = st2 * TC_M + gt;
-                pre = i2 < n ? word64(keys[i2]) : 0ull;
-                pre_st = st2;
-            }
+    const uint64_t n = cst.n;
+    const uint32_t total = (uint32_t)((n + KPT * TC_M - 1) / (KPT * TC_M));
+    const uint32_t stride = gridDim.x * NG;
+    const W *keys = reinterpret_cast<const W *>(cst.keys);
+    uint32_t st = grp * gridDim.x + blockIdx.x;  // few sub-tiles spread over the SMs
+    W pre[KPT];
+    auto fetch = [&](uint64_t i0) {
+#pragma unroll
+        for (int p = 0; p < KPT; ++p) pre[p] = i0 + p * TC_M < n ? keys[i0 + p * TC_M] : (W)0;
+    };
+    if (st < total) fetch((uint64_t)st * (KPT * TC_M) + gt);
+    for (; st < total; st += stride) {
+        const uint64_t i = (uint64_t)st * (KPT * TC_M) + gt;
+        W wv[KPT];
+        unsigned long long xx[KPT];
+        bool in_range = true;
+#pragma unroll
+        for (int p = 0; p < KPT; ++p) {
+            wv[p] = pre[p];
+            if (key_is_nan(word64(wv[p]), a.dtype)) err |= ERR_NAN;  // (a zero word past the end is no NaN)
+            const float x = translate_key<W>(wv[p], cst.norm);
+            in_range = in_range && fabsf(x) <= cst.xlim;
+            xx[p] = pk2(x, x);
         }
-        const float x = valid ? translate_key<W>((W)wv, sg.norm) : 0.0f;
-        const unsigned long long xx = pk2(x, x);
+        // the group's next sub-tile's keys, loaded while this one is computed
+        if (total - st > stride) fetch(i + (uint64_t)stride * (KPT * TC_M));
+        const bool plain = __all_sync(0xFFFFFFFFu, in_range);
 #pragma unroll
         for (int j0 = 0; j0 < H; j0 += 8) {
-            uint32_t hi[4], lo[4];
+            uint32_t hi[KPT][4], lo[KPT][4];
 #pragma unroll
             for (int q = 0; q < 4; ++q) {
                 const int j = j0 + 2 * q;
-                const unsigned long long hh =
-                    fma2_rn(pk2(cst.w1[j], cst.w1[j + 1]), xx, pk2(cst.b1[j], cst.b1[j + 1]));
-                float h0, h1;
-                upk2(hh, h0, h1);
-                if (!SPLIT) {
-                    hi[q] = cvt_bf16x2_rn_relu(h0, h1);
-                } else {
-                    hi[q] = cvt_bf16x2_rz_relu(h0, h1);
-                    const unsigned long long tr = pk2(__uint_as_float(__float_as_uint(h0) & 0xFFFF0000u),
-                                                      __uint_as_float(__float_as_uint(h1) & 0xFFFF0000u));
-                    float r0, r1;
-                    upk2(sub2_rn(hh, tr), r0, r1);
-                    lo[q] = cvt_f16x2_rn_relu(r0, r1);
+                const unsigned long long w1 = pk2(cst.w1[j], cst.w1[j + 1]), b1 = pk2(cst.b1[j], cst.b1[j + 1]);
+#pragma unroll
+                for (int p = 0; p < KPT; ++p) {
+                    const unsigned long long hh = fma2_rn(w1, xx[p], b1);
+                    float h0, h1;
+                    upk2(hh, h0, h1);
+                    if (!SPLIT) {
+                        hi[p][q] = cvt_bf16x2_rn_relu(h0, h1);
+                    } else {
+                        // the rest after the truncation; where h < 0 the part is 0 and the rest's ReLU is too.
+                        // (the low half's shift can run on the FMA pipe, a mask of h could not)
+                        hi[p][q] = cvt_bf16x2_rz_relu(h0, h1);
+                        const unsigned long long tr = pk2(__uint_as_float(hi[p][q] << 16),
+                                                          __uint_as_float(hi[p][q] & 0xFFFF0000u));
+                        float r0, r1;
+                        upk2(sub2_rn(hh, tr), r0, r1);
+                        lo[p][q] = cvt_f16x2_rn_relu(r0, r1);
+                    }
                 }
             }
-            unsigned char *t0 = myA + aoff + (j0 / 8) * LBO;
-            *reinterpret_cast<uint4 *>(t0) = make_uint4(hi[0], hi[1], hi[2], hi[3]);
-            if (SPLIT) *reinterpret_cast<uint4 *>(t0 + TILE_B) = make_uint4(lo[0], lo[1], lo[2], lo[3]);
+#pragma unroll
+            for (int p = 0; p < KPT; ++p) {
+                unsigned char *t0 = myA + p * NT * TILE_B + aoff + (j0 / 8) * LBO;
+                *reinterpret_cast<uint4 *>(t0) = make_uint4(hi[p][0], hi[p][1], hi[p][2], hi[p][3]);
+                if (SPLIT)
+                    *reinterpret_cast<uint4 *>(t0 + TILE_B) = make_uint4(lo[p][0], lo[p][1], lo[p][2], lo[p][3]);
+            }
         }
         fence_async_smem();
         tc_fence_before();
         grp_sync(bid);
         tc_fence_after();
-        if (gt == 0 && !dead) {
-            const uint32_t a0 = smem_u32(myA), b0 = smem_u32(sB);
-            // the bias slab first (it starts the accumulator), then A_hi W2^T (and A_lo W2^T)
-            mma_bf16(dcol, mdesc(smem_u32(sOnes), SLAB_LBO, SLAB_SBO), mdesc(smem_u32(sBias), SLAB_LBO, SLAB_SBO),
-                     idesc, 0u);
+        if ((warp & 3) == 0 && !dead) {
+            // the bias slab first (it starts the accumulator), then A_hi W2^T (and A_lo W2^T), issued
+            // by one elected lane of a warp-uniform sequence
 #pragma unroll
-            for (int ks = 0; ks < H / 16; ++ks)
-                mma_bf16(dcol, mdesc(a0 + ks * 2 * LBO, LBO, SBO), mdesc(b0 + ks * 2 * LBO, LBO, SBO), idesc, 1u);
-            if (SPLIT) {
+            for (int p = 0; p < KPT; ++p) {
+                const uint64_t dAp = dA + ((p * NT * TILE_B) >> 4);
+                mma_bf16_warp(dcol + p * H, dOnes, dBias, idesc, 0u);
 #pragma unroll
                 for (int ks = 0; ks < H / 16; ++ks)
-                    mma_bf16(dcol, mdesc(a0 + TILE_B + ks * 2 * LBO, LBO, SBO),
-                             mdesc(smem_u32(sB16) + ks * 2 * LBO, LBO, SBO), idesc_lo, 1u);
+                    mma_bf16_warp(dcol + p * H, dAp + ks * KSTEP, dB + ks * KSTEP, idesc, 1u);
+                if (SPLIT) {
+#pragma unroll
+                    for (int ks = 0; ks < H / 16; ++ks)
+                        mma_bf16_warp(dcol + p * H, dAp + (TILE_B >> 4) + ks * KSTEP,
+                                      dB + ((H * H * 2) >> 4) + ks * KSTEP, idesc_lo, 1u);
+                }
             }
-            mma_commit(mybar);
-            // one thread of the group waits for the MMAs; the others sleep in the barrier below
-            if (!mbar_wait(mybar, phase)) {
-                dead = true;
-                dead_parity = phase;
-                err |= ERR_TIMEOUT;
-            }
-            tc_fence_before();
+            mma_commit_warp(mybar);
+        }
+        // every thread waits for the group's MMAs itself (asleep in try_wait); it writes the A tiles again
+        // only after that
+        if (!dead && !mbar_wait(mybar, phase)) {
+            dead = true;
+            dead_parity = phase;
+            err |= ERR_TIMEOUT;
         }
         phase ^= 1u;
-        dead = grp_or(bid, dead);
+        dead = __any_sync(0xFFFFFFFFu, dead);
         tc_fence_after();
-        unsigned long long yy = pk2(cst.b3, 0.0f);
+        unsigned long long yy[KPT];
 #pragma unroll
-        for (int c0 = 0; c0 < H; c0 += 16) {
-            float acc[16];
-            if (!dead) {
-                tmem_ld16(lane_addr + c0, acc);
-                tmem_wait_ld();
-            } else {
+        for (int p = 0; p < KPT; ++p) yy[p] = pk2(cst.b3, 0.0f);
+        if (plain && !dead) {
+            // 2 ReLU(z) = z + |z| on the FMA pipe (a maximum takes two cycles of the ALU pipe); the halved
+            // W3 makes each product, and so each rounding, the same
+            // (the next columns are loaded while these are used)
+            float acc[2][KPT][16];
 #pragma unroll
-                for (int q = 0; q < 16; ++q) acc[q] = 0.0f;
+            for (int p = 0; p < KPT; ++p) tmem_ld16(lane_addr + p * H, acc[0][p]);
+            tmem_wait_ld();
+#pragma unroll
+            for (int c0 = 0; c0 < H; c0 += 16) {
+                float (*cur)[16] = acc[(c0 / 16) & 1], (*nxt)[16] = acc[(c0 / 16 + 1) & 1];
+                if (c0 + 16 < H) {
+#pragma unroll
+                    for (int p = 0; p < KPT; ++p) tmem_ld16(lane_addr + p * H + c0 + 16, nxt[p]);
+                }
+#pragma unroll
+                for (int q = 0; q < 16; q += 2) {
+                    const unsigned long long w = pk2(cst.w3h[c0 + q], cst.w3h[c0 + q + 1]);
+#pragma unroll
+                    for (int p = 0; p < KPT; ++p)
+                        yy[p] = fma2_rn(w, pk2(__fadd_rn(cur[p][q], fabsf(cur[p][q])),
+                                               __fadd_rn(cur[p][q + 1], fabsf(cur[p][q + 1]))), yy[p]);
+                }
+                if (c0 + 16 < H) tmem_wait_ld();
             }
+        } else {
+#pragma unroll 1
+            for (int p = 0; p < KPT; ++p) {
+                unsigned long long t = pk2(cst.b3, 0.0f);
+#pragma unroll 1
+                for (int c0 = 0; c0 < H; c0 += 16) {
+                    float acc[16];
+                    if (!dead) {
+                        tmem_ld16(lane_addr + p * H + c0, acc);
+                        tmem_wait_ld();
+                    } else {
 #pragma unroll
-            for (int q = 0; q < 16; q += 2)
-                yy = fma2_rn(pk2(cst.w3[c0 + q], cst.w3[c0 + q + 1]), pk2(relu_f(acc[q]), relu_f(acc[q + 1])), yy);
+                        for (int q = 0; q < 16; ++q) acc[q] = 0.0f;
+                    }
+#pragma unroll
+                    for (int q = 0; q < 16; q += 2) {
+                        const unsigned long long w = pk2(cst.w3h[c0 + q], cst.w3h[c0 + q + 1]);
+                        t = fma2_rn(add2_rn(w, w), pk2(relu_f(acc[q]), relu_f(acc[q + 1])), t);
+                    }
+                }
+                if (p == 0) yy[0] = t;
+                else yy[KPT - 1] = t;
+            }
         }
         tc_fence_before();
-        if (!valid) continue;
-        float ye, yo;
-        upk2(yy, ye, yo);
-        const float y = __fadd_rn(ye, yo);
-        const uint32_t slot = slot_of(y, sg.nm_hi, sg.nm_lo, sg.L);
-        const uint64_t e = sg.ebase + i;
-        const uint32_t gpos = (uint32_t)(sg.gs_base + slot);
-        if (a.gs) a.gs[e] = gpos;
-        if (a.key_copy) reinterpret_cast<W *>(a.key_copy)[e] = (W)wv;
-        if (a.pay_copy && sg.payload) a.pay_copy[e] = (uint32_t)sg.payload[i];
-        if (a.row_init) a.row_init[e] = (uint32_t)i;
-        if (a.slots_out) a.slots_out[e] = slot;
-        if (a.y_out) a.y_out[e] = y;
+#pragma unroll
+        for (int p = 0; p < KPT; ++p) {
+            const uint64_t ip = i + p * TC_M;
+            if (ip >= n) break;
+            float ye, yo;
+            upk2(yy[p], ye, yo);
+            const float y = __fadd_rn(ye, yo);
+            const uint32_t slot = slot_of(y, cst.nm_hi, cst.nm_lo, cst.L);
+            const uint64_t e = cst.ebase + ip;
+            if (a.gs) a.gs[e] = cst.gs_base + slot;
+            if (a.key_copy) reinterpret_cast<W *>(a.key_copy)[e] = wv[p];
+            if (a.pay_copy && cst.payload) a.pay_copy[e] = (uint32_t)cst.payload[ip];
+            if (a.row_init) a.row_init[e] = (uint32_t)ip;
+            if (a.slots_out) a.slots_out[e] = slot;
+            if (a.y_out) a.y_out[e] = y;
+        }
     }
     if (err) atomicOr(a.err, err);
     // an MMA whose completion was not seen may still be running: wait for it (bounded) before the
@@ -539,7 +597,26 @@ __global__ void __launch_bounds__(NG * TC_THREADS, 1) k_predict_bf16_mg(PredictA
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    if (warp == 0) tmem_free<NCOL>(tbase);
+    if (warp == 0) tmem_free<NCOL>(tmem_base);
+}
+
+// The largest |x| for which the activations stay below 10^6 (so that the split's FP16 part is finite)
+// and every z far below the overflow of 2 z; -1 when a weight is not finite, or too large, or its half is
+// not exact.
+template <int H> static float plain_limit(const float *P) {
+    float w1 = 0.0f, b1 = 0.0f, w2 = 0.0f, b2 = 0.0f;
+    bool ok = true;
+    for (int i = 0; i < 4 * H + H * H + 1; ++i) ok = ok && std::isfinite(P[i]);
+    for (int j = 0; j < H; ++j) {
+        w1 = std::max(w1, std::fabs(P[j]));
+        b1 = std::max(b1, std::fabs(P[H + j]));
+        b2 = std::max(b2, std::fabs(P[2 * H + H * H + j]));
+        const float w3 = std::fabs(P[3 * H + H * H + j]);
+        ok = ok && (w3 == 0.0f || w3 >= 1e-30f);
+    }
+    for (int i = 0; i < H * H; ++i) w2 = std::max(w2, std::fabs(P[2 * H + i]));
+    if (!ok || b1 > 1e5f || w2 > 1e20f || b2 > 1e30f) return -1.0f;
+    return w1 > 0.0f ? std::min(1e30f, 5e5f / w1) : 1e30f;
 }
 
 template <int H, bool SPLIT>
@@ -549,20 +626,33 @@ static cudaError_t bf16_mg_go(const PredictArgs &p, int sms, cudaStream_t s) {
     for (int j = 0; j < H; ++j) {
         c.w1[j] = p.host_pad[j];
         c.b1[j] = p.host_pad[H + j];
-        c.w3[j] = p.host_pad[3 * H + H * H + j];
+        c.w3h[j] = 0.5f * p.host_pad[3 * H + H * H + j];
     }
+    c.xlim = plain_limit<H>(p.host_pad);
     c.b3 = p.host_pad[4 * H + H * H];
-    const uint64_t n_sub = (uint64_t)p.total_tiles * (PRED_TILE / TC_M);
-    const size_t smem = tcmg_smem_bytes<H, SPLIT, TC_NG>();
-    const int grid = (int)std::min<uint64_t>((n_sub + TC_NG - 1) / TC_NG, (uint64_t)sms);
+    const Seg &g = *p.host_seg;
+    c.nm_hi = g.nm_hi;
+    c.nm_lo = g.nm_lo;
+    c.gs_base = (uint32_t)g.gs_base;
+    c.n = g.n;
+    c.ebase = g.ebase;
+    c.L = g.L;
+    c.keys = g.keys;
+    c.payload = g.payload;
+    c.norm = g.norm;
+    // two keys per thread; as many groups as their A tiles leave room for (H = 64: 64 KB each)
+    constexpr int KPT = 2, NG = H == 64 ? 3 : 6;
+    const uint64_t n_sub = (c.n + KPT * TC_M - 1) / (KPT * TC_M);
+    const size_t smem = tcmg_smem_bytes<H, SPLIT, NG, KPT>();
+    const int grid = (int)std::min<uint64_t>(n_sub, (uint64_t)sms);
     if (grid == 0) return cudaSuccess;
-    auto k4 = k_predict_bf16_mg<H, uint32_t, SPLIT, TC_NG>;
-    auto k8 = k_predict_bf16_mg<H, uint64_t, SPLIT, TC_NG>;
+    auto k4 = k_predict_bf16_mg<H, uint32_t, SPLIT, NG, KPT>;
+    auto k8 = k_predict_bf16_mg<H, uint64_t, SPLIT, NG, KPT>;
     cudaError_t e = cudaFuncSetAttribute(p.key_bytes == 4 ? k4 : k8,
                                          cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    if (p.key_bytes == 4) k4<<<grid, TC_NG * TC_THREADS, smem, s>>>(p, c);
-    else k8<<<grid, TC_NG * TC_THREADS, smem, s>>>(p, c);
+    if (p.key_bytes == 4) k4<<<grid, NG * TC_THREADS, smem, s>>>(p, c);
+    else k8<<<grid, NG * TC_THREADS, smem, s>>>(p, c);
     return nns_launched(cudaGetLastError());
 }
 
@@ -598,7 +688,7 @@ constexpr int TC_KPT = 2, TC_KPT_SPLIT = 1;
 
 cudaError_t launch_predict_bf16(const PadArch &a, const PredictArgs &p, bool split, int sms, cudaStream_t s) {
     if (a.layers != 2) return cudaErrorNotSupported;
-    if (p.nseg == 1 && p.single_model && p.host_pad) {
+    if (p.nseg == 1 && p.single_model && p.host_pad && p.host_seg) {
         switch (a.h1) {
         case 16: return split ? bf16_mg_go<16, true>(p, sms, s) : bf16_mg_go<16, false>(p, sms, s);
         case 32: return split ? bf16_mg_go<32, true>(p, sms, s) : bf16_mg_go<32, false>(p, sms, s);
