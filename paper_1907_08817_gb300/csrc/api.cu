@@ -815,11 +815,11 @@ int run_sort(const std::vector<SegIn> &in, const nnsort_sort_opts *op, int dtype
     if ((rc = ensure_arena(w, pwl_off + pwl_bytes, s))) return rc;
     if ((rc = ensure_part(w, P.N, s))) return rc;
     // staging: the segment table, then the statistics, the seam counters and the long seam ranges
-    // (disjoint and longer than SEAM_CTA_MAX each, so at most N / SEAM_CTA_MAX of them)
+    // (disjoint and longer than SEAM_CTA_LEAST each, so at most N / SEAM_CTA_LEAST of them)
     const size_t pin_stats = align_up(sizeof(Seg) * nseg, 64);
     const size_t pin_cnt = pin_stats + align_up(sizeof(SegStats) * nseg + 16, 64);
     const size_t pin_rng = pin_cnt + 64;
-    const size_t pin_big = align_up(pin_rng + sizeof(SeamRange) * (P.N / SEAM_CTA_MAX + 1), 64);
+    const size_t pin_big = align_up(pin_rng + sizeof(SeamRange) * (P.N / SEAM_CTA_LEAST + 1), 64);
     const size_t pin_pwl = align_up(pin_big + sizeof(BigRange) * (P.N / POLISH_BIG + 1), 64);
     const size_t pin_need = pin_pwl + pwl_bytes + 256;
     if ((rc = ensure_pinned(w, pin_need, s))) return rc;
@@ -939,11 +939,13 @@ int run_sort(const std::vector<SegIn> &in, const nnsort_sort_opts *op, int dtype
     const bool onepass = buckets_ok(P.wlog, rows);
     uint64_t heavy = (uint64_t)sa.polish_cap;  // elements of a bucket that the front of the order exceeds
     sa.giant_min = POLISH_BIG;
+    sa.seam_max = (uint32_t)SEAM_CTA_MAX;
     if (onepass) {
         sa.bucket_cap[0] = bucket_capacity(kb, anypay, 2);
         sa.bucket_cap[1] = bucket_capacity(kb, anypay, 1);
         heavy = (uint64_t)sa.bucket_cap[0];
         sa.giant_min = (uint32_t)sa.bucket_cap[1];
+        sa.seam_max = std::min<uint32_t>(sa.seam_max, (uint32_t)sa.bucket_cap[0]);
         // the other pair of partition buffers holds the runs until their carries are known
         sa.rk = L.key[oi];
         sa.rt = L.gs[oi];
@@ -1016,14 +1018,14 @@ int run_sort(const std::vector<SegIn> &in, const nnsort_sort_opts *op, int dtype
     }
     CK(mark(6));
     CK(launch_seam_repair(sa, sms, s));
-    if (sa.allow_defer) {
+    if (P.N > sa.seam_max) {
         // one wait at the end of the pipeline: long seam ranges run as one multi-block sort
         uint32_t *hc = reinterpret_cast<uint32_t *>(w->pinned + pin_cnt);
         CK(cudaMemcpyAsync(hc, L.seam_cnt, 4 * sizeof(uint32_t), cudaMemcpyDeviceToHost, s));
         CK(cudaStreamSynchronize(s));
         const uint32_t nlong = hc[1];
         if (nlong) {
-            if (nlong > P.N / SEAM_CTA_MAX + 1) return NNSORT_E_STATE;
+            if (nlong > P.N / SEAM_CTA_LEAST + 1) return NNSORT_E_STATE;
             SeamRange *hr = reinterpret_cast<SeamRange *>(w->pinned + pin_rng);
             CK(cudaMemcpyAsync(hr, L.ranges + (sa.max_ranges - nlong), sizeof(SeamRange) * nlong,
                                cudaMemcpyDeviceToHost, s));
@@ -1490,7 +1492,7 @@ int nnsort_train_batch(void *const *d_keys, const uint64_t *ns, int32_t count, i
     a.loss_out = h_loss ? reinterpret_cast<float *>(dev + off_loss) : nullptr;
     a.err = reinterpret_cast<uint32_t *>(dev + off_err);
     for (int c = 0; c < 3 && e == cudaSuccess; ++c) {
-        uint32_t cap = 2;
+        uint32_t cap = 8;
         for (uint32_t i = first[c]; i < first[c + 1]; ++i)
             while (cap < S[ids[i]]) cap <<= 1;
         a.ids = reinterpret_cast<const uint32_t *>(dev + off_ids) + first[c];

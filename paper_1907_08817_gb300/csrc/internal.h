@@ -153,8 +153,9 @@ struct SolveArgs {
     int key_bytes, dtype;
     int polish_cap;           // elements a bucket may hold on chip
     size_t polish_smem;
-    int allow_defer;          // 1: seam repairs above SEAM_CTA_MAX are left to the host's
+    int allow_defer;          // 1: seam repairs above seam_max are left to the host's
                               //    multi-block sort (never when rows are carried)
+    uint32_t seam_max;
     SeamRange *ranges;        // [max_ranges]: block-sized repairs from the front, large from the back
     uint32_t max_ranges;      // >= NB + nseg
     uint32_t *seam_cnt;       // [4]: block-sized ranges, large ranges, next range to repair
@@ -175,7 +176,10 @@ struct SolveArgs {
     BigRange *big;            // nullable: k_polish lists buckets above POLISH_BIG here (and only
     uint32_t *big_cnt;        //   splits their runs); their sort is left to the host's multi-block sort
 };
-constexpr uint64_t SEAM_CTA_MAX = 1u << 16;  // largest seam repair one block performs
+// largest seam repair one block performs (less where its on-chip form holds less, at least SEAM_CTA_LEAST):
+// blocks that took up to 65,536 elements, with their lists in global memory, held the whole sort up (1,024
+// arrays, 147M keys: 0.65 ms of repairs; 0.18 with 16,384, 0.07 with 8,192)
+constexpr uint64_t SEAM_CTA_MAX = 1u << 13, SEAM_CTA_LEAST = 1u << 12;
 // order[]: buckets holding more than `heavy` elements first (they run longest), the rest after
 cudaError_t launch_bucket_order(const SolveArgs &a, uint32_t heavy, uint32_t *order,
                                 uint32_t *cnt /*[2], zeroed here*/, cudaStream_t s);
