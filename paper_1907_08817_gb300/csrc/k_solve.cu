@@ -1219,24 +1219,114 @@ __device__ __forceinline__ W key_of_okey(W o) {  // the inverse of okey_of
     }
 }
 
+// minimum and maximum over a warp (every lane gets them)
+template <typename W> __device__ __forceinline__ void warp_extremes(W &lo, W &hi) {
+    if constexpr (sizeof(W) == 4) {
+        lo = __reduce_min_sync(0xFFFFFFFFu, lo);
+        hi = __reduce_max_sync(0xFFFFFFFFu, hi);
+    } else {
+#pragma unroll
+        for (int o = 16; o; o >>= 1) {
+            const W l2 = __shfl_xor_sync(0xFFFFFFFFu, lo, o), h2 = __shfl_xor_sync(0xFFFFFFFFu, hi, o);
+            lo = l2 < lo ? l2 : lo;
+            hi = h2 > hi ? h2 : hi;
+        }
+    }
+}
 // the block's extremes from its threads' (complete after the next barrier, by read_extremes)
 template <typename W> __device__ __forceinline__ void put_extremes(BucketSmem<W> &sm, W lo, W hi) {
-#pragma unroll
-    for (int o = 16; o; o >>= 1) {
-        const W l2 = __shfl_xor_sync(0xFFFFFFFFu, lo, o), h2 = __shfl_xor_sync(0xFFFFFFFFu, hi, o);
-        lo = l2 < lo ? l2 : lo;
-        hi = h2 > hi ? h2 : hi;
-    }
+    warp_extremes(lo, hi);
     if ((threadIdx.x & 31) == 0) { sm.lo[threadIdx.x >> 5] = lo; sm.hi[threadIdx.x >> 5] = hi; }
 }
 template <typename W> __device__ __forceinline__ void read_extremes(const BucketSmem<W> &sm, W &lo, W &hi) {
-    lo = sm.lo[0];
-    hi = sm.hi[0];
+    lo = sm.lo[threadIdx.x & (SNW - 1)];
+    hi = sm.hi[threadIdx.x & (SNW - 1)];
+    warp_extremes(lo, hi);
+}
+
+// The same for elements that crowd into few bins (clusters far apart, as a model that folds two key ranges
+// onto one bucket leaves them): the counts of the first bins say where the elements lie, so each bin is
+// cut again into a share of CROWD_BINS finer ones in proportion to its count, a map that keeps the order.
+// Words are the fine bins, with the index beside; bin-mates are put in order by key and index. False, with
+// K and P intact, when some fine bin is crowded too. On entry sm.bins holds the counts of the first
+// bins; out of line, so that it costs the common path no registers.
+constexpr uint32_t CROWD_BINS = 2048, CROWD_MAX = 8192;
+template <typename W, bool FL, bool PAY>
+__device__ __noinline__ bool sort_crowded(BucketSmem<W> &sm, const W *K, uint32_t *word, const uint32_t *P,
+                                          uint16_t *idx, uint32_t nbk, W lo, W hi, W *outk, int32_t *outp) {
+    const int tid = threadIdx.x;
+    uint32_t *fine = sm.bins + NBIN;  // the rest of the radix sort's tables
+    static_assert(sizeof(sm.hist) + sizeof(sm.wcnt) >= (NBIN + CROWD_BINS) * sizeof(uint32_t), "room for the fine bins");
+    constexpr int BPT = NBIN / SOLVE_THREADS, FPT = CROWD_BINS / SOLVE_THREADS;
+    const W range = hi - lo;
+    int br = 0;
+    if constexpr (sizeof(W) == 8) br = range ? 64 - __clzll((long long)range) : 0;
+    else br = range ? 32 - __clz((int)range) : 0;
+    const int ib = nbk > 1 ? 32 - __clz((int)(nbk - 1)) : 0;
+    const int sh = br - NBIN_LOG;  // a first bin holds 2^sh keys (all of them, for crowded ones: no index bits)
+    if (sh <= 0 || br + ib <= NBIN_LOG) return false;
+    // starts of the first bins, and the fine bins that follow from them: bin b's are
+    // [start(b) F / nbk, start(b + 1) F / nbk)
+    uint32_t c[BPT], sum = 0;
 #pragma unroll
-    for (int q = 1; q < SNW; ++q) {
-        lo = sm.lo[q] < lo ? sm.lo[q] : lo;
-        hi = sm.hi[q] > hi ? sm.hi[q] : hi;
+    for (int q = 0; q < BPT; ++q) { c[q] = sm.bins[tid * BPT + q]; sum += c[q]; }
+    uint32_t st = block_excl_sum(sum, sm.scratch, nullptr);
+#pragma unroll
+    for (int q = 0; q < BPT; ++q) {
+        sm.bins[tid * BPT + q] = st * CROWD_BINS / nbk;
+        st += c[q];
     }
+#pragma unroll
+    for (int q = 0; q < FPT; ++q) fine[tid * FPT + q] = 0;
+    __syncthreads();
+    const int low = sh < 16 ? sh : 16;  // bits of the place inside a first bin that the map looks at
+    auto fine_of = [&](W k) -> uint32_t {
+        const W d = k - lo;
+        const uint32_t b = (uint32_t)(d >> sh), f0 = sm.bins[b], f1 = b + 1 < NBIN ? sm.bins[b + 1] : CROWD_BINS;
+        const uint32_t part = (uint32_t)(d >> (sh - low)) & ((1u << low) - 1u);
+        const uint32_t f = f0 + ((f1 - f0) * part >> low);
+        return f < CROWD_BINS ? f : CROWD_BINS - 1;
+    };
+    for (uint32_t i = tid; i < nbk; i += SOLVE_THREADS) {
+        const uint32_t f = fine_of(K[i]);
+        const uint32_t at = atomicAdd(&fine[f], 1u);
+        word[i] = (f << 16) | at;  // arrival order inside the bin
+    }
+    __syncthreads();
+    uint32_t g[FPT], m = 0;
+    sum = 0;
+#pragma unroll
+    for (int q = 0; q < FPT; ++q) { g[q] = fine[tid * FPT + q]; sum += g[q]; m = max(m, g[q]); }
+    if (__syncthreads_or(m > BIN_MAX)) return false;
+    st = block_excl_sum(sum, sm.scratch, nullptr);
+    const uint32_t beg = st;
+#pragma unroll
+    for (int q = 0; q < FPT; ++q) { fine[tid * FPT + q] = st; st += g[q]; }
+    const uint32_t end = st;
+    __syncthreads();
+    for (uint32_t i = tid; i < nbk; i += SOLVE_THREADS) idx[fine[word[i] >> 16] + (word[i] & 0xFFFFu)] = (uint16_t)i;
+    __syncthreads();
+    // each thread's bins follow one another: insertion by key and index
+    for (uint32_t j = beg + 1; j < end; ++j) {
+        const uint32_t y = idx[j];
+        const W ky = K[y];
+        uint32_t k = j;
+        while (k > beg) {
+            const uint32_t x = idx[k - 1];
+            const W kx = K[x];
+            if (kx < ky || (kx == ky && x < y)) break;
+            idx[k] = (uint16_t)x;
+            --k;
+        }
+        idx[k] = (uint16_t)y;
+    }
+    __syncthreads();
+    for (uint32_t j = tid; j < nbk; j += SOLVE_THREADS) {
+        const uint32_t x = idx[j];
+        outk[j] = key_of_okey<W, FL>(K[x]);
+        if constexpr (PAY) { if (outp) outp[j] = (int32_t)P[x]; }
+    }
+    return true;
 }
 
 // `nbk` elements in shared memory (K: order images with extremes lo, hi; P: payload) to their output in
@@ -1270,6 +1360,10 @@ __device__ __forceinline__ void sort_chip(BucketSmem<W> &sm, const W *K, uint32_
         uint4 c0 = t4[2 * tid], c1 = t4[2 * tid + 1];
         const uint32_t m = max(max(max(c0.x, c0.y), max(c0.z, c0.w)), max(max(c1.x, c1.y), max(c1.z, c1.w)));
         binned = !__syncthreads_or(m > BIN_MAX);
+        if (!binned && nbk <= CROWD_MAX) {
+            if (sort_crowded<W, FL, PAY>(sm, K, word, P, idx, nbk, lo, hi, outk, outp)) return;
+            __syncthreads();
+        }
         if (binned) {
             const uint32_t sum = c0.x + c0.y + c0.z + c0.w + c1.x + c1.y + c1.z + c1.w;
             uint32_t st = block_excl_sum(sum, sm.scratch, nullptr), t;
@@ -1426,7 +1520,7 @@ __device__ __forceinline__ void bucket_one(const SolveArgs &a, unsigned char *br
         for (uint32_t q = 0; q < PER; ++q) {
             x[q] = (q < per && p0 + q < Wn) ? sm.tbl[p0 + q] : EMPTY32;
             if (x[q] != EMPTY32) {
-                F[x[q]] = 1;
+                if (r + 1 < eps) F[x[q]] = 1;
                 e[q] = OPair<W>::make(K[x[q]], x[q]);
                 if (loc.less(e[q])) loc = e[q];
             }
