@@ -941,11 +941,10 @@ int run_sort(const std::vector<SegIn> &in, const nnsort_sort_opts *op, int dtype
     sa.giant_min = POLISH_BIG;
     sa.seam_max = (uint32_t)SEAM_CTA_MAX;
     if (onepass) {
-        sa.bucket_cap[0] = bucket_capacity(kb, anypay, 2);
-        sa.bucket_cap[1] = bucket_capacity(kb, anypay, 1);
+        bucket_capacities(sa, anypay);
         heavy = (uint64_t)sa.bucket_cap[0];
-        sa.giant_min = (uint32_t)sa.bucket_cap[1];
-        sa.seam_max = std::min<uint32_t>(sa.seam_max, (uint32_t)sa.bucket_cap[0]);
+        sa.giant_min = (uint32_t)sa.bucket_cap[2];
+        sa.seam_max = std::min<uint32_t>(sa.seam_max, (uint32_t)sa.seam_cap);
         // the other pair of partition buffers holds the runs until their carries are known
         sa.rk = L.key[oi];
         sa.rt = L.gs[oi];

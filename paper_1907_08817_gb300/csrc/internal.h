@@ -167,7 +167,10 @@ struct SolveArgs {
     void *rk;                 // [N] keys' width
     uint32_t *rt;             // [N]
     uint32_t *rend;           // [NB * MAXR]
-    int bucket_cap[2];        // elements that a one-pass block holds with two and with one block per SM
+    int bucket_cap[3];        // elements that a one-pass block holds: of the width's own size, with two
+                              //   512-thread blocks per SM, with one
+    int bucket_threads;       // threads of the first of these
+    int seam_cap;             // elements that a block of the on-chip seam repair holds
     const uint32_t *heavy_cnt;  // with rk: the order's first *heavy_cnt buckets exceed bucket_cap[0]
     uint32_t giant_min;       // buckets above this many elements are listed in giant
     const uint32_t *order;    // [NB] nullable: block i of k_rounds / k_polish takes bucket order[i]
@@ -200,11 +203,11 @@ struct GiantRounds {
 cudaError_t launch_giant_buckets(const SolveArgs &a, const GiantRounds &g, int eps, int sms, cudaStream_t s);
 cudaError_t launch_giant_rounds(const SolveArgs &a, const GiantRounds &g, int eps, int sms, cudaStream_t s);
 cudaError_t launch_rounds(const SolveArgs &a, cudaStream_t s);
-// every bucket of at most bucket_cap[1] elements in one pass (rounds, runs and sorted output), and their
+// every bucket of at most bucket_cap[2] elements in one pass (rounds, runs and sorted output), and their
 // out-of-order counts once the carries are known; larger ones are left to launch_giant_buckets and the
 // host's multi-block sort
 bool buckets_ok(int wlog, bool rows);
-int bucket_capacity(int key_bytes, bool payload, int blocks_per_sm);
+void bucket_capacities(SolveArgs &a, bool payload);
 cudaError_t launch_buckets(const SolveArgs &a, int sms, cudaStream_t s);
 cudaError_t launch_carried(const SolveArgs &a, cudaStream_t s);
 cudaError_t launch_finalize(const SolveArgs &a, cudaStream_t s);

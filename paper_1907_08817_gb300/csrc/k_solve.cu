@@ -529,18 +529,18 @@ __global__ void __launch_bounds__(MT_THREADS) k_finalize_apply(SolveArgs a, cons
 // with the running per-digit base folded in, and each element is written straight to its place.
 // Returns the buffer holding the result.
 constexpr int SORT_ITEMS = 8;
-constexpr uint32_t SORT_TILE = SOLVE_THREADS * SORT_ITEMS;
-template <typename Idx, typename KeyFn>
+template <typename Idx, int T = SOLVE_THREADS, typename KeyFn>
 __device__ Idx *cta_radix_sort(Idx *src, Idx *dst, uint32_t cnt, int keybits, KeyFn kf,
-                               uint32_t *hist /*[8][256]*/, uint32_t *wcnt /*[SNW][256]*/,
+                               uint32_t *hist /*[8][256]*/, uint32_t *wcnt /*[(T / 32)][256]*/,
                                uint32_t *scratch /*33*/) {
     const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
     const unsigned lt = (1u << lane) - 1u;
     const int npass = keybits / 8;
-    for (int i = tid; i < npass * 256; i += SOLVE_THREADS) hist[i] = 0;
-    for (int i = tid; i < SNW * 256; i += SOLVE_THREADS) wcnt[i] = 0;
+    for (int i = tid; i < npass * 256; i += T) hist[i] = 0;
+    for (int i = tid; i < (T / 32) * 256; i += T) wcnt[i] = 0;
+    static_assert(T >= 256 || T == 128, "a thread per digit, or two");
     __syncthreads();
-    for (uint32_t i = tid; i < cnt; i += SOLVE_THREADS) {
+    for (uint32_t i = tid; i < cnt; i += T) {
         const unsigned long long k = kf(src[i]);
         for (int p = 0; p < npass; ++p) atomicAdd(&hist[p * 256 + (uint32_t)((k >> (8 * p)) & 0xFFu)], 1u);
     }
@@ -551,11 +551,19 @@ __device__ Idx *cta_radix_sort(Idx *src, Idx *dst, uint32_t cnt, int keybits, Ke
         uint32_t *h = hist + p * 256;
         const int shift = 8 * p;
         if (h[(uint32_t)((kfirst >> shift) & 0xFFu)] == cnt) continue;  // same decision on every thread
-        const uint32_t hv = (tid < 256) ? h[tid] : 0u;
-        const uint32_t ex = block_excl_sum(hv, scratch, nullptr);
-        if (tid < 256) h[tid] = ex;  // running base per digit
+        // running base per digit (DP digits per thread)
+        constexpr int DP = T >= 256 ? 1 : 256 / T;
+        uint32_t hv[DP], hs = 0;
+#pragma unroll
+        for (int q = 0; q < DP; ++q) { hv[q] = tid * DP + q < 256 ? h[tid * DP + q] : 0u; hs += hv[q]; }
+        uint32_t ex = block_excl_sum(hs, scratch, nullptr);
+#pragma unroll
+        for (int q = 0; q < DP; ++q) {
+            if (tid * DP + q < 256) h[tid * DP + q] = ex;
+            ex += hv[q];
+        }
         __syncthreads();
-        for (uint32_t t0 = 0; t0 < cnt; t0 += SORT_TILE) {
+        for (uint32_t t0 = 0; t0 < cnt; t0 += (uint32_t)(T * SORT_ITEMS)) {
             Idx x[SORT_ITEMS];
             uint32_t d[SORT_ITEMS], wr[SORT_ITEMS];
 #pragma unroll
@@ -582,21 +590,21 @@ __device__ Idx *cta_radix_sort(Idx *src, Idx *dst, uint32_t cnt, int keybits, Ke
                 __syncwarp();
             }
             __syncthreads();
-            if (tid < 256) {
-                uint32_t run = h[tid];
-                for (int ww = 0; ww < SNW; ++ww) {
-                    const uint32_t c = wcnt[ww * 256 + tid];
-                    wcnt[ww * 256 + tid] = run;
+            for (int d8 = tid; d8 < 256; d8 += T) {
+                uint32_t run = h[d8];
+                for (int ww = 0; ww < (T / 32); ++ww) {
+                    const uint32_t c = wcnt[ww * 256 + d8];
+                    wcnt[ww * 256 + d8] = run;
                     run += c;
                 }
-                h[tid] = run;
+                h[d8] = run;
             }
             __syncthreads();
 #pragma unroll
             for (int r = 0; r < SORT_ITEMS; ++r)
                 if (d[r] < 256u) dst[wcnt[w * 256 + d[r]] + wr[r]] = x[r];
             __syncthreads();
-            for (int i = tid; i < SNW * 256; i += SOLVE_THREADS) wcnt[i] = 0;
+            for (int i = tid; i < (T / 32) * 256; i += T) wcnt[i] = 0;
             __syncthreads();
         }
         Idx *tmp = src; src = dst; dst = tmp;
@@ -1158,7 +1166,7 @@ template <> struct OPair<uint64_t> {
     }
 };
 
-// block-wide exclusive prefix maximum; `scratch` (SNW entries) may be written again after one more barrier
+// block-wide exclusive prefix maximum; `scratch` (an entry per warp, at most 16) may be written again after one more barrier
 template <typename W>
 __device__ __forceinline__ OPair<W> block_excl_max_pair(OPair<W> v, OPair<W> *scratch) {
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
@@ -1183,28 +1191,37 @@ __device__ __forceinline__ OPair<W> block_excl_max_pair(OPair<W> v, OPair<W> *sc
     m = OPair<W>::make((W)__shfl_sync(0xFFFFFFFFu, m.key(), 0), __shfl_sync(0xFFFFFFFFu, m.tie(), 0));
     return ex.less(m) ? m : ex;
 }
-static_assert(SNW == 16, "one half warp holds the warps' maxima");
+static_assert(SNW <= 16, "one half warp holds the warps' maxima");
 
-// longest list that the bins take: four elements per bin, of which a thread orders eight bins
-constexpr uint32_t BUCKET_BIN_MAX = 4 * NBIN;
+// Blocks of T threads serve buckets of at most 8 T positions (eight per thread) with 8 T bins: a bucket of
+// 2^10 positions in a block sized for 2^12 spent most of its time on empty bins and idle threads (26M f32
+// keys in 32,001 such buckets, three rounds: 1.31 ms; 0.57 ms with 128 threads).
+constexpr int bucket_log(int T) { return T == 512 ? 12 : T == 256 ? 11 : 10; }  // log2 of positions and bins
 
-template <typename W> struct BucketSmem {
+template <typename W, int T> struct BucketSmem {
+    static constexpr int NW = T / 32;
+    static constexpr uint32_t NBIN = 8u * T;
+    static constexpr int NBIN_LOG = bucket_log(T);
+    static_assert(NBIN == 1u << NBIN_LOG, "a power of two");
+    static constexpr uint32_t CROWD_BINS = NBIN / 2;
+    // longest list that the bins take: four elements per bin, of which a thread orders eight bins
+    static constexpr uint32_t BIN_SORT = 4 * NBIN;
     union {
-        uint32_t tbl[NBIN];   // claims of at most 2^12 positions
-        uint32_t bins[NBIN];
+        uint32_t tbl[NBIN];   // claims
+        uint32_t bins[NBIN + CROWD_BINS];
         struct {
             uint32_t hist[8 * 256];
-            uint32_t wcnt[SNW * 256];
+            uint32_t wcnt[NW * 256];
         };
     };
-    OPair<W> pmax[SNW];
-    W lo[SNW], hi[SNW];
+    OPair<W> pmax[NW];
+    W lo[NW], hi[NW];
     uint32_t scratch[33];
     int seg;
 };
 
-template <typename W>
-__host__ __device__ constexpr size_t bucket_fixed() { return (sizeof(BucketSmem<W>) + 15) & ~(size_t)15; }
+template <typename W, int T>
+__host__ __device__ constexpr size_t bucket_fixed() { return (sizeof(BucketSmem<W, T>) + 15) & ~(size_t)15; }
 // per element: key, word (the radix sort's index lists in its place), position (later the index), flag,
 // payload
 template <typename W>
@@ -1234,13 +1251,13 @@ template <typename W> __device__ __forceinline__ void warp_extremes(W &lo, W &hi
     }
 }
 // the block's extremes from its threads' (complete after the next barrier, by read_extremes)
-template <typename W> __device__ __forceinline__ void put_extremes(BucketSmem<W> &sm, W lo, W hi) {
+template <typename W, int T> __device__ __forceinline__ void put_extremes(BucketSmem<W, T> &sm, W lo, W hi) {
     warp_extremes(lo, hi);
     if ((threadIdx.x & 31) == 0) { sm.lo[threadIdx.x >> 5] = lo; sm.hi[threadIdx.x >> 5] = hi; }
 }
-template <typename W> __device__ __forceinline__ void read_extremes(const BucketSmem<W> &sm, W &lo, W &hi) {
-    lo = sm.lo[threadIdx.x & (SNW - 1)];
-    hi = sm.hi[threadIdx.x & (SNW - 1)];
+template <typename W, int T> __device__ __forceinline__ void read_extremes(const BucketSmem<W, T> &sm, W &lo, W &hi) {
+    lo = sm.lo[threadIdx.x & (T / 32 - 1)];
+    hi = sm.hi[threadIdx.x & (T / 32 - 1)];
     warp_extremes(lo, hi);
 }
 
@@ -1250,14 +1267,16 @@ template <typename W> __device__ __forceinline__ void read_extremes(const Bucket
 // Words are the fine bins, with the index beside; bin-mates are put in order by key and index. False, with
 // K and P intact, when some fine bin is crowded too. On entry sm.bins holds the counts of the first
 // bins; out of line, so that it costs the common path no registers.
-constexpr uint32_t CROWD_BINS = 2048, CROWD_MAX = 8192;
-template <typename W, bool FL, bool PAY>
-__device__ __noinline__ bool sort_crowded(BucketSmem<W> &sm, const W *K, uint32_t *word, const uint32_t *P,
+constexpr uint32_t CROWD_MAX = 8192;
+template <typename W, bool FL, bool PAY, int T>
+__device__ __noinline__ bool sort_crowded(BucketSmem<W, T> &sm, const W *K, uint32_t *word, const uint32_t *P,
                                           uint16_t *idx, uint32_t nbk, W lo, W hi, W *outk, int32_t *outp) {
     const int tid = threadIdx.x;
-    uint32_t *fine = sm.bins + NBIN;  // the rest of the radix sort's tables
-    static_assert(sizeof(sm.hist) + sizeof(sm.wcnt) >= (NBIN + CROWD_BINS) * sizeof(uint32_t), "room for the fine bins");
-    constexpr int BPT = NBIN / SOLVE_THREADS, FPT = CROWD_BINS / SOLVE_THREADS;
+    using B = BucketSmem<W, T>;
+    constexpr uint32_t NBIN = B::NBIN, CROWD_BINS = B::CROWD_BINS;
+    constexpr int NBIN_LOG = B::NBIN_LOG;
+    uint32_t *fine = sm.bins + NBIN;
+    constexpr int BPT = NBIN / T, FPT = CROWD_BINS / T;
     const W range = hi - lo;
     int br = 0;
     if constexpr (sizeof(W) == 8) br = range ? 64 - __clzll((long long)range) : 0;
@@ -1287,7 +1306,7 @@ __device__ __noinline__ bool sort_crowded(BucketSmem<W> &sm, const W *K, uint32_
         const uint32_t f = f0 + ((f1 - f0) * part >> low);
         return f < CROWD_BINS ? f : CROWD_BINS - 1;
     };
-    for (uint32_t i = tid; i < nbk; i += SOLVE_THREADS) {
+    for (uint32_t i = tid; i < nbk; i += T) {
         const uint32_t f = fine_of(K[i]);
         const uint32_t at = atomicAdd(&fine[f], 1u);
         word[i] = (f << 16) | at;  // arrival order inside the bin
@@ -1304,7 +1323,7 @@ __device__ __noinline__ bool sort_crowded(BucketSmem<W> &sm, const W *K, uint32_
     for (int q = 0; q < FPT; ++q) { fine[tid * FPT + q] = st; st += g[q]; }
     const uint32_t end = st;
     __syncthreads();
-    for (uint32_t i = tid; i < nbk; i += SOLVE_THREADS) idx[fine[word[i] >> 16] + (word[i] & 0xFFFFu)] = (uint16_t)i;
+    for (uint32_t i = tid; i < nbk; i += T) idx[fine[word[i] >> 16] + (word[i] & 0xFFFFu)] = (uint16_t)i;
     __syncthreads();
     // each thread's bins follow one another: insertion by key and index
     for (uint32_t j = beg + 1; j < end; ++j) {
@@ -1321,7 +1340,7 @@ __device__ __noinline__ bool sort_crowded(BucketSmem<W> &sm, const W *K, uint32_
         idx[k] = (uint16_t)y;
     }
     __syncthreads();
-    for (uint32_t j = tid; j < nbk; j += SOLVE_THREADS) {
+    for (uint32_t j = tid; j < nbk; j += T) {
         const uint32_t x = idx[j];
         outk[j] = key_of_okey<W, FL>(K[x]);
         if constexpr (PAY) { if (outp) outp[j] = (int32_t)P[x]; }
@@ -1332,10 +1351,12 @@ __device__ __noinline__ bool sort_crowded(BucketSmem<W> &sm, const W *K, uint32_
 // `nbk` elements in shared memory (K: order images with extremes lo, hi; P: payload) to their output in
 // (key, index) order. word, idx: one entry per element (word also holds the radix sort's lists). A barrier
 // has passed since the last use of sm's tables and the writes of K and P; none is left behind.
-template <typename W, bool FL, bool PAY>
-__device__ __forceinline__ void sort_chip(BucketSmem<W> &sm, const W *K, uint32_t *word, const uint32_t *P,
+template <typename W, bool FL, bool PAY, int T>
+__device__ __forceinline__ void sort_chip(BucketSmem<W, T> &sm, const W *K, uint32_t *word, const uint32_t *P,
                                           uint16_t *idx, uint32_t nbk, uint32_t cap, W lo, W hi, W *outk,
                                           int32_t *outp) {
+    constexpr uint32_t NBIN = BucketSmem<W, T>::NBIN, BUCKET_BIN_MAX = BucketSmem<W, T>::BIN_SORT;
+    constexpr int NBIN_LOG = BucketSmem<W, T>::NBIN_LOG;
     const int tid = threadIdx.x;
     const W range = hi - lo;
     int br = 0;
@@ -1351,17 +1372,17 @@ __device__ __forceinline__ void sort_chip(BucketSmem<W> &sm, const W *K, uint32_
     bool binned = nbk <= BUCKET_BIN_MAX;
     if (binned) {
         uint4 *t4 = reinterpret_cast<uint4 *>(sm.bins);
-        for (uint32_t j = tid; j < NBIN / 4; j += SOLVE_THREADS) t4[j] = make_uint4(0u, 0u, 0u, 0u);
+        for (uint32_t j = tid; j < NBIN / 4; j += T) t4[j] = make_uint4(0u, 0u, 0u, 0u);
         __syncthreads();
-        for (uint32_t i = tid; i < nbk; i += SOLVE_THREADS) atomicAdd(&sm.bins[word_of(i, K[i]) >> bs], 1u);
+        for (uint32_t i = tid; i < nbk; i += T) atomicAdd(&sm.bins[word_of(i, K[i]) >> bs], 1u);
         __syncthreads();
-        constexpr int BPT = NBIN / SOLVE_THREADS;
+        constexpr int BPT = NBIN / T;
         static_assert(BPT == 8, "two 16-byte reads per thread");
         uint4 c0 = t4[2 * tid], c1 = t4[2 * tid + 1];
         const uint32_t m = max(max(max(c0.x, c0.y), max(c0.z, c0.w)), max(max(c1.x, c1.y), max(c1.z, c1.w)));
         binned = !__syncthreads_or(m > BIN_MAX);
         if (!binned && nbk <= CROWD_MAX) {
-            if (sort_crowded<W, FL, PAY>(sm, K, word, P, idx, nbk, lo, hi, outk, outp)) return;
+            if (sort_crowded<W, FL, PAY, T>(sm, K, word, P, idx, nbk, lo, hi, outk, outp)) return;
             __syncthreads();
         }
         if (binned) {
@@ -1378,7 +1399,7 @@ __device__ __forceinline__ void sort_chip(BucketSmem<W> &sm, const W *K, uint32_
             t4[2 * tid] = c0;
             t4[2 * tid + 1] = c1;
             __syncthreads();
-            for (uint32_t i = tid; i < nbk; i += SOLVE_THREADS) {
+            for (uint32_t i = tid; i < nbk; i += T) {
                 const uint32_t w = word_of(i, K[i]);
                 const uint32_t slot = atomicAdd(&sm.bins[w >> bs], 1u);
                 word[slot] = w;
@@ -1424,7 +1445,7 @@ __device__ __forceinline__ void sort_chip(BucketSmem<W> &sm, const W *K, uint32_
             }
             __syncthreads();
             const uint32_t imask = (1u << ib) - 1u;
-            for (uint32_t j = tid; j < nbk; j += SOLVE_THREADS) {
+            for (uint32_t j = tid; j < nbk; j += T) {
                 const uint32_t c = word[j];
                 const uint32_t x = drop ? (uint32_t)idx[j] : (c & imask);
                 W o;
@@ -1437,12 +1458,12 @@ __device__ __forceinline__ void sort_chip(BucketSmem<W> &sm, const W *K, uint32_
     }
     if (!binned) {
         uint16_t *X = reinterpret_cast<uint16_t *>(word), *Y = X + cap;
-        for (uint32_t i = tid; i < nbk; i += SOLVE_THREADS) X[i] = (uint16_t)i;
+        for (uint32_t i = tid; i < nbk; i += T) X[i] = (uint16_t)i;
         __syncthreads();
         auto kf = [&](uint16_t x) -> W { return K[x]; };
-        const uint16_t *A = cta_radix_sort<uint16_t>(X, Y, nbk, 8 * (int)sizeof(W), kf, sm.hist, sm.wcnt, sm.scratch);
+        const uint16_t *A = cta_radix_sort<uint16_t, T>(X, Y, nbk, 8 * (int)sizeof(W), kf, sm.hist, sm.wcnt, sm.scratch);
         __syncthreads();
-        for (uint32_t q = tid; q < nbk; q += SOLVE_THREADS) {
+        for (uint32_t q = tid; q < nbk; q += T) {
             const uint32_t x = A[q];
             outk[q] = key_of_okey<W, FL>(K[x]);
             if constexpr (PAY) { if (outp) outp[q] = (int32_t)P[x]; }
@@ -1450,12 +1471,12 @@ __device__ __forceinline__ void sort_chip(BucketSmem<W> &sm, const W *K, uint32_
     }
 }
 
-template <typename W, bool FL, bool PAY>
+template <typename W, bool FL, bool PAY, int T>
 __device__ __forceinline__ void bucket_one(const SolveArgs &a, unsigned char *braw, uint32_t b, uint32_t cap) {
-    BucketSmem<W> &sm = *reinterpret_cast<BucketSmem<W> *>(braw);
+    BucketSmem<W, T> &sm = *reinterpret_cast<BucketSmem<W, T> *>(braw);
     const int tid = threadIdx.x;
     const uint32_t s0 = a.bstart[b], nbk = a.bstart[b + 1] - s0;
-    unsigned char *p = braw + bucket_fixed<W>();
+    unsigned char *p = braw + bucket_fixed<W, T>();
     W *K = reinterpret_cast<W *>(p); p += sizeof(W) * cap;
     uint32_t *word = reinterpret_cast<uint32_t *>(p); p += (size_t)4 * cap;
     uint32_t *P = nullptr;
@@ -1470,12 +1491,12 @@ __device__ __forceinline__ void bucket_one(const SolveArgs &a, unsigned char *br
     // the bucket, as order images, with its extremes
     W lo = (W)~(W)0, hi = 0;
     constexpr int LB = 8;  // loads per thread issued together
-    for (uint32_t i0 = 0; i0 < nbk; i0 += SOLVE_THREADS * LB) {
+    for (uint32_t i0 = 0; i0 < nbk; i0 += T * LB) {
         W k[LB];
         uint32_t g[LB], q4[LB];
 #pragma unroll
         for (int q = 0; q < LB; ++q) {
-            const uint32_t i = i0 + q * SOLVE_THREADS + tid;
+            const uint32_t i = i0 + q * T + tid;
             if (i < nbk) {
                 k[q] = ldk<W>(a.keys, s0 + i);
                 g[q] = a.gs[s0 + i];
@@ -1484,7 +1505,7 @@ __device__ __forceinline__ void bucket_one(const SolveArgs &a, unsigned char *br
         }
 #pragma unroll
         for (int q = 0; q < LB; ++q) {
-            const uint32_t i = i0 + q * SOLVE_THREADS + tid;
+            const uint32_t i = i0 + q * T + tid;
             if (i < nbk) {
                 const W o = okey_of<W, FL>(k[q]);
                 K[i] = o;
@@ -1500,18 +1521,18 @@ __device__ __forceinline__ void bucket_one(const SolveArgs &a, unsigned char *br
 
     // rounds (Fig. "Algorithm NN-sort"): every element still unplaced claims its position, the first to
     // arrive is stored; the position table then gives o_r in position order
-    constexpr uint32_t PER = NBIN / SOLVE_THREADS;  // positions per thread at most
-    const uint32_t per = (Wn + SOLVE_THREADS - 1) / SOLVE_THREADS, p0 = (uint32_t)tid * per;
+    constexpr uint32_t PER = 8;  // positions per thread at most
+    const uint32_t per = (Wn + T - 1) / T, p0 = (uint32_t)tid * per;
     int eps = 0, r = 0;
     uint32_t roff = 0, left = nbk;
     W *rk = reinterpret_cast<W *>(a.rk) + s0;
     for (;; ++r) {
         uint4 *t4 = reinterpret_cast<uint4 *>(sm.tbl);
-        for (uint32_t j = tid; j < Wn / 4; j += SOLVE_THREADS) t4[j] = make_uint4(EMPTY32, EMPTY32, EMPTY32, EMPTY32);
+        for (uint32_t j = tid; j < Wn / 4; j += T) t4[j] = make_uint4(EMPTY32, EMPTY32, EMPTY32, EMPTY32);
         __syncthreads();
         if (r == 0) eps = (int)a.segs[sm.seg].eps;
         if (r >= eps || left == 0) break;  // uniform
-        for (uint32_t i = tid; i < nbk; i += SOLVE_THREADS)
+        for (uint32_t i = tid; i < nbk; i += T)
             if (r == 0 || !F[i]) atomicMin(&sm.tbl[pos[i]], i);
         __syncthreads();
         uint32_t x[PER];
@@ -1546,7 +1567,7 @@ __device__ __forceinline__ void bucket_one(const SolveArgs &a, unsigned char *br
         const uint32_t in = tot & 0xFFFFu, out = tot >> 16;
         roff += in;
         left -= in + out;
-        if (tid == SOLVE_THREADS - 1) {
+        if (tid == T - 1) {
             OKey o; o.k = run.key(); o.tb = run.tie(); o.valid = in ? 1u : 0u;
             a.bmax[(size_t)b * MAXR + r] = o;
         }
@@ -1576,20 +1597,22 @@ __device__ __forceinline__ void bucket_one(const SolveArgs &a, unsigned char *br
     W *outk = reinterpret_cast<W *>(sg.keys) + off;
     int32_t *outp = (PAY && sg.payload) ? sg.payload + off : nullptr;
     // (the barrier that ended the rounds also ended their reads of the table)
-    sort_chip<W, FL, PAY>(sm, K, word, P, pos, nbk, cap, lo, hi, outk, outp);
+    sort_chip<W, FL, PAY, T>(sm, K, word, P, pos, nbk, cap, lo, hi, outk, outp);
 }
 
-// SECOND: the heavy buckets of the order's front that a block alone on its SM can hold
-template <typename W, bool FL, bool PAY, bool SECOND>
-__global__ void __launch_bounds__(SOLVE_THREADS, SECOND ? 1 : 2) k_bucket(SolveArgs a) {
+// TIER 0: every bucket of the order that fits. TIER 1 and 2: of the heavy buckets at the order's front, those
+// that two blocks per SM, or one, can hold.
+template <typename W, bool FL, bool PAY, int TIER, int T>
+__global__ void __launch_bounds__(T, TIER == 0 ? 1024 / T : TIER == 1 ? 2 : 1) k_bucket(SolveArgs a) {
     extern __shared__ __align__(16) unsigned char braw[];
     if (*a.err) return;  // NaN keys or bad positions: leave the caller's arrays untouched
-    if constexpr (SECOND) {
-        const uint32_t nb = *a.heavy_cnt;
+    const uint32_t cap = (uint32_t)a.bucket_cap[TIER];
+    if constexpr (TIER > 0) {
+        const uint32_t nb = *a.heavy_cnt, least = (uint32_t)a.bucket_cap[TIER - 1];
         for (uint32_t j = blockIdx.x; j < nb; j += gridDim.x) {
             const uint32_t b = a.order[j], nbk = a.bstart[b + 1] - a.bstart[b];
-            if (nbk > (uint32_t)a.bucket_cap[1]) continue;  // launch_giant_buckets
-            bucket_one<W, FL, PAY>(a, braw, b, (uint32_t)a.bucket_cap[1]);
+            if (nbk <= least || nbk > cap) continue;  // another tier, or launch_giant_buckets
+            bucket_one<W, FL, PAY, T>(a, braw, b, cap);
             __syncthreads();  // the next bucket reuses the shared arrays
         }
     } else {
@@ -1602,8 +1625,8 @@ __global__ void __launch_bounds__(SOLVE_THREADS, SECOND ? 1 : 2) k_bucket(SolveA
             }
             return;
         }
-        if (nbk > (uint32_t)a.bucket_cap[0]) return;
-        bucket_one<W, FL, PAY>(a, braw, b, (uint32_t)a.bucket_cap[0]);
+        if (nbk > cap) return;
+        bucket_one<W, FL, PAY, T>(a, braw, b, cap);
     }
 }
 
@@ -1852,36 +1875,68 @@ __global__ void __launch_bounds__(256) k_carried(SolveArgs a) {
 // the position table of a block holds NBIN positions; rows (traces) need every element's round
 bool buckets_ok(int wlog, bool rows) { return !rows && wlog <= NBIN_LOG; }
 
-// elements of a bucket that fit on chip with this many one-pass blocks per SM (228 KB, of which a block
-// reserves 1 KB and can use 227)
-int bucket_capacity(int key_bytes, bool payload, int blocks_per_sm) {
-    const size_t budget = blocks_per_sm == 1 ? 227 * 1024 : (228 * 1024) / blocks_per_sm - 1024 - 512;
-    const size_t cap = key_bytes == 4 ? (budget - bucket_fixed<uint32_t>()) / bucket_per<uint32_t>(payload)
-                                      : (budget - bucket_fixed<uint64_t>()) / bucket_per<uint64_t>(payload);
+// elements that fit on chip at `blocks` blocks of T threads per SM (228 KB, of which a block reserves 1 KB
+// and can use 227)
+template <int T> static int chip_cap(int key_bytes, bool payload, int blocks) {
+    const size_t budget = blocks == 1 ? 227 * 1024 : (228 * 1024) / blocks - 1024 - 512;
+    const size_t cap = key_bytes == 4 ? (budget - bucket_fixed<uint32_t, T>()) / bucket_per<uint32_t>(payload)
+                                      : (budget - bucket_fixed<uint64_t, T>()) / bucket_per<uint64_t>(payload);
     return (int)(std::min<size_t>(cap, 65534) & ~(size_t)15);
 }
+// The smallest block (128, 256 or 512 threads; 6, 3 and 2 per SM) whose eight positions per thread cover the
+// bucket's W positions and whose memory holds 2 W elements: a bucket has 0.8 W on average, but models
+// leave some several times as full, and those take the slower tiers. 64M u64 key-value pairs in buckets
+// of 2^11 positions: 256 threads hold 3,080 elements, and the tiers take 1.90 ms together; 512 threads
+// hold 4,733 and take 1.87.
+void bucket_capacities(SolveArgs &a, bool payload) {
+    const int want = 2 << a.wlog;
+    a.seam_cap = chip_cap<512>(a.key_bytes, payload, 2);
+    a.bucket_threads = 512;
+    a.bucket_cap[0] = a.seam_cap;
+    if (const int c = chip_cap<128>(a.key_bytes, payload, 6); a.wlog <= 10 && c >= want) {
+        a.bucket_threads = 128;
+        a.bucket_cap[0] = c;
+    } else if (const int d = chip_cap<256>(a.key_bytes, payload, 3); a.wlog <= 11 && d >= want) {
+        a.bucket_threads = 256;
+        a.bucket_cap[0] = d;
+    }
+    a.bucket_cap[1] = std::max(a.bucket_cap[0], a.seam_cap);
+    a.bucket_cap[2] = chip_cap<512>(a.key_bytes, payload, 1);
+}
 
-template <typename W, bool FL, bool PAY, bool SECOND>
+template <typename W, bool FL, bool PAY, int TIER, int T>
 static cudaError_t bucket_go(const SolveArgs &a, unsigned grid, cudaStream_t s) {
-    const size_t smem = bucket_fixed<W>() + (size_t)a.bucket_cap[SECOND ? 1 : 0] * bucket_per<W>(PAY);
-    auto kfn = k_bucket<W, FL, PAY, SECOND>;
+    const size_t smem = bucket_fixed<W, T>() + (size_t)a.bucket_cap[TIER] * bucket_per<W>(PAY);
+    auto kfn = k_bucket<W, FL, PAY, TIER, T>;
     cudaError_t e = cudaFuncSetAttribute(kfn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    kfn<<<grid, SOLVE_THREADS, smem, s>>>(a);
+    kfn<<<grid, T, smem, s>>>(a);
     return nns_launched(cudaGetLastError());
 }
-template <typename W, bool SECOND>
+template <typename W, int TIER, int T>
 static cudaError_t bucket_go2(const SolveArgs &a, unsigned grid, cudaStream_t s) {
     const bool fl = a.dtype == NNSORT_F32 || a.dtype == NNSORT_F64;
-    if (a.pay) return fl ? bucket_go<W, true, true, SECOND>(a, grid, s) : bucket_go<W, false, true, SECOND>(a, grid, s);
-    return fl ? bucket_go<W, true, false, SECOND>(a, grid, s) : bucket_go<W, false, false, SECOND>(a, grid, s);
+    if (a.pay)
+        return fl ? bucket_go<W, true, true, TIER, T>(a, grid, s) : bucket_go<W, false, true, TIER, T>(a, grid, s);
+    return fl ? bucket_go<W, true, false, TIER, T>(a, grid, s) : bucket_go<W, false, false, TIER, T>(a, grid, s);
+}
+template <typename W> static cudaError_t buckets_go(const SolveArgs &a, int sms, cudaStream_t s) {
+    cudaError_t e;
+    switch (a.bucket_threads) {
+    case 512: e = bucket_go2<W, 0, 512>(a, a.NB, s); break;
+    case 256: e = bucket_go2<W, 0, 256>(a, a.NB, s); break;
+    default: e = bucket_go2<W, 0, 128>(a, a.NB, s);
+    }
+    if (e != cudaSuccess || !a.heavy_cnt) return e;
+    if (a.bucket_cap[1] > a.bucket_cap[0] &&
+        (e = bucket_go2<W, 1, 512>(a, std::min<unsigned>(a.NB, 2u * (unsigned)sms), s)) != cudaSuccess)
+        return e;
+    if (a.N <= (uint64_t)a.bucket_cap[1]) return cudaSuccess;
+    return bucket_go2<W, 2, 512>(a, std::min<unsigned>(a.NB, (unsigned)sms), s);
 }
 cudaError_t launch_buckets(const SolveArgs &a, int sms, cudaStream_t s) {
     if (a.NB == 0) return cudaSuccess;
-    const cudaError_t e = a.key_bytes == 4 ? bucket_go2<uint32_t, false>(a, a.NB, s) : bucket_go2<uint64_t, false>(a, a.NB, s);
-    if (e != cudaSuccess || !a.heavy_cnt) return e;
-    const unsigned grid = std::min<unsigned>(a.NB, (unsigned)sms);
-    return a.key_bytes == 4 ? bucket_go2<uint32_t, true>(a, grid, s) : bucket_go2<uint64_t, true>(a, grid, s);
+    return a.key_bytes == 4 ? buckets_go<uint32_t>(a, sms, s) : buckets_go<uint64_t>(a, sms, s);
 }
 cudaError_t launch_carried(const SolveArgs &a, cudaStream_t s) {
     if (a.NB == 0) return cudaSuccess;
@@ -2300,12 +2355,13 @@ __global__ void __launch_bounds__(SOLVE_THREADS) k_seam_fix(SolveArgs a) {
 template <typename W, bool FL, bool PAY>
 __global__ void __launch_bounds__(SOLVE_THREADS, 2) k_seam_sort(SolveArgs a) {
     extern __shared__ __align__(16) unsigned char braw[];
-    BucketSmem<W> &sm = *reinterpret_cast<BucketSmem<W> *>(braw);
+    constexpr int T = SOLVE_THREADS;
+    BucketSmem<W, T> &sm = *reinterpret_cast<BucketSmem<W, T> *>(braw);
     __shared__ uint32_t sh_r;
     if (*a.err) return;
     const int tid = threadIdx.x;
-    const uint32_t cap = (uint32_t)a.bucket_cap[0], nr = a.seam_cnt[0];
-    unsigned char *p = braw + bucket_fixed<W>();
+    const uint32_t cap = (uint32_t)a.seam_cap, nr = a.seam_cnt[0];
+    unsigned char *p = braw + bucket_fixed<W, T>();
     W *K = reinterpret_cast<W *>(p); p += sizeof(W) * cap;
     uint32_t *word = reinterpret_cast<uint32_t *>(p); p += (size_t)4 * cap;
     uint32_t *P = nullptr;
@@ -2349,7 +2405,7 @@ __global__ void __launch_bounds__(SOLVE_THREADS, 2) k_seam_sort(SolveArgs a) {
         put_extremes(sm, lo, hi);
         __syncthreads();
         read_extremes(sm, lo, hi);
-        sort_chip<W, FL, PAY>(sm, K, word, P, idx, len, cap, lo, hi, outk, outp);
+        sort_chip<W, FL, PAY, T>(sm, K, word, P, idx, len, cap, lo, hi, outk, outp);
         __syncthreads();
     }
 }
@@ -2549,7 +2605,7 @@ template <typename W> static cudaError_t seam_go(const SolveArgs &a, int sms, cu
     k_seam_emit<<<a.nseg, SCAN_THREADS, 0, s>>>(a);
     if ((e = nns_launched(cudaGetLastError())) != cudaSuccess) return e;
     if (a.rk) {  // one-pass buckets
-        const size_t smem = bucket_fixed<W>() + (size_t)a.bucket_cap[0] * bucket_per<W>(a.pay != nullptr);
+        const size_t smem = bucket_fixed<W, SOLVE_THREADS>() + (size_t)a.seam_cap * bucket_per<W>(a.pay != nullptr);
         const bool fl = a.dtype == NNSORT_F32 || a.dtype == NNSORT_F64;
         auto kfn = a.pay ? (fl ? k_seam_sort<W, true, true> : k_seam_sort<W, false, true>)
                          : (fl ? k_seam_sort<W, true, false> : k_seam_sort<W, false, false>);
