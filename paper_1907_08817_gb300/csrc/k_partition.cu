@@ -32,7 +32,7 @@ namespace nns {
 // histograms instead of from waits on earlier tiles, so every block is independent: two blocks run
 // on each SM and one block's loads overlap the other's ranking and stores.
 namespace {
-constexpr int TH_THREADS = 512, TH_ITEMS = SC_TILE / TH_THREADS, TH_NW = TH_THREADS / 32;  // histogram blocks
+constexpr int TH_THREADS = 256, TH_ITEMS = SC_TILE / TH_THREADS, TH_NW = TH_THREADS / 32;  // histogram blocks
 constexpr int SC_THREADS = 256, SC_ITEMS = SC_TILE / SC_THREADS, SC_NW = SC_THREADS / 32;  // scatter blocks
 
 template <typename W, bool KEYDIG>
@@ -42,42 +42,48 @@ __device__ __forceinline__ uint32_t sc_digit(const PartitionArgs &a, W key, uint
 }
 }  // namespace
 
-// per tile: the digit histogram (per-warp counters, so that equal digits contend within a warp only)
+// per tile: the digit histogram (per-warp counters, so that equal digits contend within a warp only;
+// sixteen elements per thread keep the counters to clear and to add up few against the elements)
 template <typename W, bool KEYDIG>
 __global__ void __launch_bounds__(TH_THREADS) k_tile_hist(PartitionArgs a) {
     __shared__ uint32_t h[TH_NW][RADIX_BINS];
     const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
-    for (int i = lane; i < RADIX_BINS; i += 32) h[w][i] = 0;
-    __syncwarp();
+    const uint32_t bins = max(32u, 1u << a.bits), mask = (1u << a.bits) - 1u;
     const uint64_t base = (uint64_t)blockIdx.x * SC_TILE;
     const uint32_t cnt = (uint32_t)min((uint64_t)SC_TILE, a.N - base);
-    const uint32_t mask = (1u << a.bits) - 1u;
-    const W *kin = reinterpret_cast<const W *>(a.key_in);
+    const W *kin = reinterpret_cast<const W *>(a.key_in) + base;
+    const uint32_t *gin = KEYDIG ? nullptr : a.gs_in + base;
+    const uint32_t loc0 = (uint32_t)w * (32 * TH_ITEMS) + lane;
     uint32_t d[TH_ITEMS];
 #pragma unroll
     for (int r = 0; r < TH_ITEMS; ++r) {
-        const uint32_t loc = (uint32_t)w * (32 * TH_ITEMS) + r * 32 + lane;
+        const uint32_t loc = loc0 + r * 32;
         d[r] = 0xFFFFFFFFu;
         if (loc < cnt) {
-            if constexpr (KEYDIG) d[r] = sc_digit<W, true>(a, kin[base + loc], 0u, mask);
-            else d[r] = sc_digit<W, false>(a, W(0), a.gs_in[base + loc], mask);
+            if constexpr (KEYDIG) d[r] = sc_digit<W, true>(a, kin[loc], 0u, mask);
+            else d[r] = sc_digit<W, false>(a, W(0), gin[loc], mask);
         }
     }
+    for (uint32_t i = lane; i < bins; i += 32) h[w][i] = 0;
+    __syncwarp();
 #pragma unroll
     for (int r = 0; r < TH_ITEMS; ++r)
         if (d[r] != 0xFFFFFFFFu) atomicAdd(&h[w][d[r]], 1u);
     __syncthreads();
-    uint32_t t = 0;
+    for (uint32_t i = tid; i < bins; i += TH_THREADS) {
+        uint32_t t = 0;
 #pragma unroll
-    for (int ww = 0; ww < TH_NW; ++ww) t += h[ww][tid];  // TH_THREADS == RADIX_BINS
-    a.tile_hist[(size_t)blockIdx.x * RADIX_BINS + tid] = (uint16_t)t;
-    if (blockIdx.x == 0) a.bin_total[tid] = 0;  // summed by k_chunk_prefix, which runs after
+        for (int ww = 0; ww < TH_NW; ++ww) t += h[ww][i];
+        a.tile_hist[(size_t)blockIdx.x * RADIX_BINS + i] = (uint16_t)t;
+    }
+    if (blockIdx.x == 0)  // summed by k_chunk_prefix, which runs after; k_chunk_base scans all of them
+        for (int i = tid; i < RADIX_BINS; i += TH_THREADS) a.bin_total[i] = 0;
 }
 
 // per chunk of SC_CHUNK tiles: each tile's histogram becomes its exclusive prefix inside the chunk,
 // the chunk's totals go to chunk[c] and are added to the digit totals
 __global__ void __launch_bounds__(RADIX_BINS) k_chunk_prefix(PartitionArgs a, uint32_t tiles) {
-    const uint32_t c = blockIdx.x, d = threadIdx.x;
+    const uint32_t c = blockIdx.x, d = threadIdx.x;  // a thread per digit
     const uint32_t t0 = c * SC_CHUNK;
     uint16_t v[SC_CHUNK];
 #pragma unroll
@@ -91,6 +97,23 @@ __global__ void __launch_bounds__(RADIX_BINS) k_chunk_prefix(PartitionArgs a, ui
     }
     a.chunk[(size_t)c * RADIX_BINS + d] = run;
     if (run) atomicAdd(&a.bin_total[d], run);
+}
+
+// one chunk (at most SC_CHUNK tiles): the tiles' prefixes and the digit bases in one block, a digit per
+// thread
+__global__ void __launch_bounds__(RADIX_BINS) k_chunk_one(PartitionArgs a, uint32_t tiles) {
+    __shared__ uint32_t scratch[33];
+    const uint32_t d = threadIdx.x;
+    uint16_t v[SC_CHUNK];
+#pragma unroll
+    for (int j = 0; j < SC_CHUNK; ++j) v[j] = (uint32_t)j < tiles ? a.tile_hist[(size_t)j * RADIX_BINS + d] : (uint16_t)0;
+    uint32_t run = 0;
+#pragma unroll
+    for (int j = 0; j < SC_CHUNK; ++j) {
+        if ((uint32_t)j < tiles) a.tile_hist[(size_t)j * RADIX_BINS + d] = (uint16_t)run;
+        run += v[j];
+    }
+    a.chunk[d] = block_excl_sum(run, scratch, nullptr);
 }
 
 // chunk totals -> chunk bases, the digit's base (elements of all smaller digits) plus the sum over
@@ -304,10 +327,16 @@ static cudaError_t sc_go(const PartitionArgs &a, cudaStream_t s) {
     k_tile_hist<W, KD><<<(unsigned)tiles, TH_THREADS, 0, s>>>(a);
     cudaError_t e = nns_launched(cudaGetLastError());
     if (e != cudaSuccess) return e;
-    k_chunk_prefix<<<(unsigned)chunks, RADIX_BINS, 0, s>>>(a, (uint32_t)tiles);
-    if ((e = nns_launched(cudaGetLastError())) != cudaSuccess) return e;
-    k_chunk_base<<<RADIX_BINS / 32, 1024, 0, s>>>(a, (uint32_t)chunks);
-    if ((e = nns_launched(cudaGetLastError())) != cudaSuccess) return e;
+    const unsigned bins = (unsigned)std::max(32, 1 << a.bits);
+    if (chunks == 1) {
+        k_chunk_one<<<1, bins, 0, s>>>(a, (uint32_t)tiles);
+        if ((e = nns_launched(cudaGetLastError())) != cudaSuccess) return e;
+    } else {
+        k_chunk_prefix<<<(unsigned)chunks, bins, 0, s>>>(a, (uint32_t)tiles);
+        if ((e = nns_launched(cudaGetLastError())) != cudaSuccess) return e;
+        k_chunk_base<<<bins / 32, 1024, 0, s>>>(a, (uint32_t)chunks);
+        if ((e = nns_launched(cudaGetLastError())) != cudaSuccess) return e;
+    }
     const bool pay = a.pay_in != nullptr, row = a.row_in != nullptr;
     // resident blocks per SM: with four-byte keys three (four without positions to carry) pay although
     // a few of the sixteen elements' registers spill (2^28 keys, 8-bit pass: 1.44, 1.26 and 1.29 ms at
