@@ -536,8 +536,14 @@ Layout carve(unsigned char *base, int nseg, uint64_t N, uint32_t NB, int kb, boo
     c.base = base;
     Layout L{};
     L.segs = c.take<Seg>(nseg);
+    // what a call clears first, in one piece: the statistics and the error word (also read back in one
+    // piece), then the counters
     L.stats = c.take<SegStats>(nseg);
     L.err = c.take<uint32_t>(4);
+    L.order_cnt = c.take<uint32_t>(4);
+    L.seam_cnt = c.take<uint32_t>(4);
+    L.big_cnt = c.take<uint32_t>(4);
+    L.giant_cnt = c.take<uint32_t>(4);
     for (int i = 0; i < 2; ++i) {
         L.gs[i] = c.take<uint32_t>(N);
         L.key[i] = c.take<unsigned char>(N * kb);
@@ -555,14 +561,10 @@ Layout carve(unsigned char *base, int nseg, uint64_t N, uint32_t NB, int kb, boo
     L.blo = c.take<OKey>(NB);
     L.bhi = c.take<OKey>(NB);
     L.ranges = c.take<SeamRange>((size_t)NB + nseg);
-    L.seam_cnt = c.take<uint32_t>(4);
     L.order = c.take<uint32_t>(NB);
-    L.order_cnt = c.take<uint32_t>(4);
     L.rend = rows ? nullptr : c.take<uint32_t>((size_t)NB * MAXR);
     L.big = c.take<BigRange>(N / POLISH_BIG + 1);
-    L.big_cnt = c.take<uint32_t>(4);
     L.giant = c.take<BigRange>(N / GIANT_LEAST + 1);
-    L.giant_cnt = c.take<uint32_t>(4);
     L.g_cnt = c.take<unsigned int>((N / GIANT_LEAST + 1) * MAXR);
     L.g_tbmax = c.take<unsigned int>((N / POLISH_BIG + 1) * MAXR);
     L.g_kmax = c.take<unsigned long long>((N / POLISH_BIG + 1) * MAXR);
@@ -817,7 +819,7 @@ int run_sort(const std::vector<SegIn> &in, const nnsort_sort_opts *op, int dtype
     // staging: the segment table, then the statistics, the seam counters and the long seam ranges
     // (disjoint and longer than SEAM_CTA_LEAST each, so at most N / SEAM_CTA_LEAST of them)
     const size_t pin_stats = align_up(sizeof(Seg) * nseg, 64);
-    const size_t pin_cnt = pin_stats + align_up(sizeof(SegStats) * nseg + 16, 64);
+    const size_t pin_cnt = pin_stats + align_up(align_up(sizeof(SegStats) * nseg, 256) + 16, 64);
     const size_t pin_rng = pin_cnt + 64;
     const size_t pin_big = align_up(pin_rng + sizeof(SeamRange) * (P.N / SEAM_CTA_LEAST + 1), 64);
     const size_t pin_pwl = align_up(pin_big + sizeof(BigRange) * (P.N / POLISH_BIG + 1), 64);
@@ -841,8 +843,7 @@ int run_sort(const std::vector<SegIn> &in, const nnsort_sort_opts *op, int dtype
         pwl_dev.tab = dp;
         pwl_dev.S = (uint32_t)pbrk.size();
     }
-    CK(cudaMemsetAsync(L.stats, 0, sizeof(SegStats) * nseg, s));
-    CK(cudaMemsetAsync(L.err, 0, 16, s));
+    CK(cudaMemsetAsync(L.stats, 0, (size_t)((unsigned char *)(L.giant_cnt + 4) - (unsigned char *)L.stats), s));
 
     const bool timing = o.timing && st;
     if (timing && !w->ev[0])
@@ -895,8 +896,6 @@ int run_sort(const std::vector<SegIn> &in, const nnsort_sort_opts *op, int dtype
     }
     const int fi = P.pp.npass & 1, oi = fi ^ 1;
     CK(mark(2));
-    CK(launch_bucket_bounds(L.gs[fi], P.N, P.NB, P.wlog, L.bstart, s));
-    CK(mark(3));
 
     SolveArgs sa{};
     sa.segs = L.segs;
@@ -944,6 +943,11 @@ int run_sort(const std::vector<SegIn> &in, const nnsort_sort_opts *op, int dtype
         bucket_capacities(sa, anypay);
         heavy = (uint64_t)sa.bucket_cap[0];
         sa.giant_min = (uint32_t)sa.bucket_cap[2];
+        // an array that one block alone on its SM can hold needs no deferred repair, and so no wait for one
+        if (P.N <= (uint64_t)sa.bucket_cap[2]) {
+            sa.seam_cap = std::max(sa.seam_cap, (int)align_up(P.N, 16));
+            sa.seam_max = (uint32_t)sa.seam_cap;
+        }
         sa.seam_max = std::min<uint32_t>(sa.seam_max, (uint32_t)sa.seam_cap);
         // the other pair of partition buffers holds the runs until their carries are known
         sa.rk = L.key[oi];
@@ -966,8 +970,16 @@ int run_sort(const std::vector<SegIn> &in, const nnsort_sort_opts *op, int dtype
         gr.tbmax = L.g_tbmax;
         gr.cap = (uint32_t)(P.N / sa.giant_min + 1);
     }
-    if (P.N > heavy || !onepass) {  // no bucket can exceed it otherwise
-        CK(launch_bucket_order(sa, (uint32_t)heavy, L.order, L.order_cnt, s));
+    const bool ordered = P.N > heavy || !onepass;  // no bucket can exceed it otherwise
+    if (small_solve(sa)) {
+        CK(launch_bounds_order_small(sa, L.bstart, (uint32_t)heavy, ordered ? L.order : nullptr, L.order_cnt, s));
+        CK(mark(3));
+    } else {
+        CK(launch_bucket_bounds(L.gs[fi], P.N, P.NB, P.wlog, L.bstart, s));
+        CK(mark(3));
+        if (ordered) CK(launch_bucket_order(sa, (uint32_t)heavy, L.order, L.order_cnt, s));
+    }
+    if (ordered) {
         sa.order = L.order;
         if (onepass) sa.heavy_cnt = L.order_cnt;
     }
@@ -978,16 +990,16 @@ int run_sort(const std::vector<SegIn> &in, const nnsort_sort_opts *op, int dtype
         if (!rows) {
             sa.big = L.big;
             sa.big_cnt = L.big_cnt;
-            CK(cudaMemsetAsync(L.big_cnt, 0, sizeof(uint32_t), s));
         }
         CK(launch_rounds(sa, s));
         if (giants) CK(launch_giant_rounds(sa, gr, o.eps, sms, s));
     }
     CK(mark(4));
-    CK(launch_finalize(sa, s));
+    const bool small = small_solve(sa);
+    CK(small ? launch_finalize_small(sa, s) : launch_finalize(sa, s));
     CK(mark(5));
-    if (onepass) CK(launch_carried(sa, s));
-    else CK(launch_polish(sa, s));
+    if (!onepass) CK(launch_polish(sa, s));
+    else if (!small) CK(launch_carried(sa, s));
     if (giants && !rows) {
         // buckets too large for one block: one wait, then one multi-block sort of all of them
         uint32_t *hc = reinterpret_cast<uint32_t *>(w->pinned + pin_cnt);
@@ -1040,11 +1052,11 @@ int run_sort(const std::vector<SegIn> &in, const nnsort_sort_opts *op, int dtype
 
     if (o.no_sync && !st) return NNSORT_OK;
     unsigned char *hp = w->pinned + pin_stats;
-    CK(cudaMemcpyAsync(hp, L.stats, sizeof(SegStats) * nseg, cudaMemcpyDeviceToHost, s));
-    CK(cudaMemcpyAsync(hp + sizeof(SegStats) * nseg, L.err, 4, cudaMemcpyDeviceToHost, s));
+    const size_t err_off = (size_t)((unsigned char *)L.err - (unsigned char *)L.stats);
+    CK(cudaMemcpyAsync(hp, L.stats, err_off + 4, cudaMemcpyDeviceToHost, s));
     CK(cudaStreamSynchronize(s));
     uint32_t err = 0;
-    std::memcpy(&err, hp + sizeof(SegStats) * nseg, 4);
+    std::memcpy(&err, hp + err_off, 4);
     if (st) {
         for (int i = 0; i < nseg; ++i) {
             SegStats d;

@@ -158,7 +158,7 @@ struct SolveArgs {
     uint32_t seam_max;
     SeamRange *ranges;        // [max_ranges]: block-sized repairs from the front, large from the back
     uint32_t max_ranges;      // >= NB + nseg
-    uint32_t *seam_cnt;       // [4]: block-sized ranges, large ranges, next range to repair
+    uint32_t *seam_cnt;       // [4], zero before the seam: block-sized ranges, large ranges, next range to repair
     OKey *seam_suf;           // [NB] scratch: smallest element of the later buckets
     OKey *seam_pre;           // [NB] scratch: largest element of the earlier buckets
     unsigned long long *seam_cut;  // [2 NB] scratch: first and last sorted-boundary cut per bucket
@@ -185,7 +185,7 @@ struct SolveArgs {
 constexpr uint64_t SEAM_CTA_MAX = 1u << 13, SEAM_CTA_LEAST = 1u << 12;
 // order[]: buckets holding more than `heavy` elements first (they run longest), the rest after
 cudaError_t launch_bucket_order(const SolveArgs &a, uint32_t heavy, uint32_t *order,
-                                uint32_t *cnt /*[2], zeroed here*/, cudaStream_t s);
+                                uint32_t *cnt /*[2], zero, as giant_cnt*/, cudaStream_t s);
 // buckets above POLISH_BIG elements run their rounds on the whole GPU (global claim tables); the
 // list, its count and the per-(bucket, round) statistics live in GiantRounds
 struct GiantRounds {
@@ -210,6 +210,11 @@ bool buckets_ok(int wlog, bool rows);
 void bucket_capacities(SolveArgs &a, bool payload);
 cudaError_t launch_buckets(const SolveArgs &a, int sms, cudaStream_t s);
 cudaError_t launch_carried(const SolveArgs &a, cudaStream_t s);
+// one array of few buckets: bounds and order, finalize and carried counts, in one launch each
+bool small_solve(const SolveArgs &a);
+cudaError_t launch_bounds_order_small(const SolveArgs &a, uint32_t *bstart, uint32_t heavy, uint32_t *order,
+                                      uint32_t *cnt, cudaStream_t s);
+cudaError_t launch_finalize_small(const SolveArgs &a, cudaStream_t s);
 cudaError_t launch_finalize(const SolveArgs &a, cudaStream_t s);
 cudaError_t launch_polish(const SolveArgs &a, cudaStream_t s);
 cudaError_t launch_seam_repair(const SolveArgs &a, int sms, cudaStream_t s);

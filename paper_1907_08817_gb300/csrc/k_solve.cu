@@ -89,10 +89,50 @@ __global__ void k_bucket_order(SolveArgs a, uint32_t heavy, uint32_t *order, uin
 cudaError_t launch_bucket_order(const SolveArgs &a, uint32_t heavy, uint32_t *order, uint32_t *cnt,
                                 cudaStream_t s) {
     if (a.NB == 0) return cudaSuccess;
-    cudaError_t e = cudaMemsetAsync(cnt, 0, 2 * sizeof(uint32_t), s);
-    if (e == cudaSuccess && a.giant_cnt) e = cudaMemsetAsync(a.giant_cnt, 0, 2 * sizeof(uint32_t), s);
-    if (e != cudaSuccess) return e;
     k_bucket_order<<<(a.NB + 255) / 256, 256, 0, s>>>(a, heavy, order, cnt);
+    return nns_launched(cudaGetLastError());
+}
+
+// One array of at most SMALL_BUCKETS buckets: steps that are a launch each for larger ones share a launch of
+// one block here (a sort of 10,000 keys is bound by its launches and waits).
+constexpr uint32_t SMALL_BUCKETS = 1024;
+
+// k_bucket_bounds and k_bucket_order
+__global__ void __launch_bounds__(SMALL_BUCKETS) k_bounds_order_small(SolveArgs a, uint32_t *bstart, uint32_t heavy,
+                                                                      uint32_t *order, uint32_t *cnt) {
+    __shared__ uint32_t sh[SMALL_BUCKETS + 1], c[2];
+    const uint32_t tid = threadIdx.x;
+    if (tid < 2) c[tid] = 0;
+    for (uint32_t b = tid; b <= a.NB; b += SMALL_BUCKETS) {
+        uint64_t lo = 0, hi = b == a.NB ? 0 : a.N;
+        if (b == a.NB) lo = a.N;
+        while (lo < hi) {
+            const uint64_t mid = (lo + hi) >> 1;
+            if ((a.gs[mid] >> a.wlog) < b) lo = mid + 1; else hi = mid;
+        }
+        sh[b] = (uint32_t)lo;
+        bstart[b] = (uint32_t)lo;
+    }
+    __syncthreads();
+    if (!order || tid >= a.NB) return;
+    const uint32_t nbk = sh[tid + 1] - sh[tid];
+    if (nbk > heavy) {
+        const uint32_t i = atomicAdd(&c[0], 1u);
+        order[i] = tid;
+        atomicAdd(&cnt[0], 1u);
+    } else {
+        order[a.NB - 1 - atomicAdd(&c[1], 1u)] = tid;
+    }
+    if (a.giant && nbk > a.giant_min) {
+        BigRange r;
+        r.lo = sh[tid]; r.hi = sh[tid + 1]; r.seg = 0; r.off = 0; r.b = tid; r.pad = 0;
+        a.giant[atomicAdd(a.giant_cnt, 1u)] = r;
+    }
+}
+bool small_solve(const SolveArgs &a) { return a.nseg == 1 && a.rk && a.NB <= SMALL_BUCKETS; }
+cudaError_t launch_bounds_order_small(const SolveArgs &a, uint32_t *bstart, uint32_t heavy, uint32_t *order,
+                                      uint32_t *cnt, cudaStream_t s) {
+    k_bounds_order_small<<<1, SMALL_BUCKETS, 0, s>>>(a, bstart, heavy, order, cnt);
     return nns_launched(cudaGetLastError());
 }
 
@@ -1827,6 +1867,19 @@ cudaError_t launch_giant_buckets(const SolveArgs &a, const GiantRounds &g, int e
     return cudaSuccess;
 }
 
+// how many of the ascending run [beg, end) lie below the carry (most runs start above it: one read)
+template <typename W>
+__device__ __forceinline__ uint32_t below_carry(const W *rk, const uint32_t *rt, uint32_t beg, uint32_t end,
+                                                unsigned long long ck, uint32_t ct) {
+    if (end <= beg || !okey_less(rk[beg], rt[beg], ck, ct)) return 0;
+    uint32_t l = beg + 1, h = end;
+    while (l < h) {
+        const uint32_t mid = (l + h) >> 1;
+        if (okey_less(rk[mid], rt[mid], ck, ct)) l = mid + 1; else h = mid;
+    }
+    return l - beg;
+}
+
 // The out-of-order elements that only the carry makes so: of each one-pass bucket's in-order runs, the
 // elements below the carry. A thread per bucket; most runs start above their carry and cost one read.
 template <typename W>
@@ -1852,15 +1905,7 @@ __global__ void __launch_bounds__(256) k_carried(SolveArgs a) {
         if (nbk) {
             const uint32_t end = a.rend[(size_t)b * MAXR + r];
             const OKey c = a.carry[(size_t)b * MAXR + r];
-            if (c.valid && end > beg) {
-                uint32_t l = beg, h = end;
-                if (!okey_less(rk[l], rt[l], c.k, c.tb)) h = l;
-                while (l < h) {
-                    const uint32_t mid = (l + h) >> 1;
-                    if (okey_less(rk[mid], rt[mid], c.k, c.tb)) l = mid + 1; else h = mid;
-                }
-                n = l - beg;
-            }
+            if (c.valid) n = below_carry(rk, rt, beg, end, c.k, c.tb);
             beg = end;
         }
         if (a.nseg == 1) {
@@ -1869,6 +1914,41 @@ __global__ void __launch_bounds__(256) k_carried(SolveArgs a) {
         } else if (n) {
             atomicAdd(&a.stats[seg].ooo[r], (unsigned long long)n);
         }
+    }
+}
+
+// k_finalize and k_carried of a small array: thread b holds bucket b's carry
+template <typename W>
+__global__ void __launch_bounds__(SMALL_BUCKETS) k_finalize_small(SolveArgs a) {
+    __shared__ KMax scratch[33];
+    __shared__ int sh_t;
+    const uint32_t b = threadIdx.x;
+    const Seg &sg = a.segs[0];
+    SegStats &st = a.stats[0];
+    if (b == 0) {
+        const int t = rounds_of(sg, st);
+        st.count_ge[0] = sg.n;
+        st.t = (uint32_t)t;
+        sh_t = t;
+    }
+    __syncthreads();
+    if (*a.err) return;
+    const int t = sh_t;
+    uint32_t s0 = 0, nbk = 0, beg = 0;
+    if (b < a.NB) { s0 = a.bstart[b]; nbk = a.bstart[b + 1] - s0; }
+    const W *rk = reinterpret_cast<const W *>(a.rk) + s0;
+    const uint32_t *rt = a.rt + s0;
+    for (int r = 0; r < t; ++r) {
+        const KMax v = b < a.NB ? kmax_of(a.bmax[(size_t)b * MAXR + r]) : kmax_none();
+        const KMax c = block_excl_max(v, scratch, nullptr);
+        uint32_t n = 0;
+        if (nbk) {
+            const uint32_t end = a.rend[(size_t)b * MAXR + r];
+            if (c.valid) n = below_carry(rk, rt, beg, end, c.k, c.tb);
+            beg = end;
+        }
+        n = __reduce_add_sync(0xFFFFFFFFu, n);
+        if ((b & 31) == 0 && n) atomicAdd(&st.ooo[r], (unsigned long long)n);
     }
 }
 
@@ -1937,6 +2017,11 @@ template <typename W> static cudaError_t buckets_go(const SolveArgs &a, int sms,
 cudaError_t launch_buckets(const SolveArgs &a, int sms, cudaStream_t s) {
     if (a.NB == 0) return cudaSuccess;
     return a.key_bytes == 4 ? buckets_go<uint32_t>(a, sms, s) : buckets_go<uint64_t>(a, sms, s);
+}
+cudaError_t launch_finalize_small(const SolveArgs &a, cudaStream_t s) {
+    if (a.key_bytes == 4) k_finalize_small<uint32_t><<<1, SMALL_BUCKETS, 0, s>>>(a);
+    else k_finalize_small<uint64_t><<<1, SMALL_BUCKETS, 0, s>>>(a);
+    return nns_launched(cudaGetLastError());
 }
 cudaError_t launch_carried(const SolveArgs &a, cudaStream_t s) {
     if (a.NB == 0) return cudaSuccess;
@@ -2162,53 +2247,69 @@ __global__ void __launch_bounds__(MT_THREADS) k_seam_apply(SolveArgs a, const OK
     }
 }
 
+// the first and last sound cut of bucket bi of array sg, whose neighbours' extremes are P and S (all ones when
+// it has none)
+template <typename W>
+__device__ __forceinline__ void seam_cuts(const SolveArgs &a, const Seg &sg, uint32_t bi, const KMax &P, const KMax &S,
+                                          unsigned long long &fg, unsigned long long &lg) {
+    fg = lg = ~0ull;
+    if (a.bstart[bi + 1] == a.bstart[bi]) return;
+    const W *outk = reinterpret_cast<const W *>(sg.keys);
+    auto elem = [&](unsigned long long pos, unsigned long long &k, uint32_t &tb) {
+        k = ordbits(word64(outk[pos]), a.dtype);
+        tb = a.out_rows ? a.out_rows[sg.ebase + pos] : 0u;
+    };
+    const unsigned long long b0 = a.bstart[bi] - sg.ebase, b1 = a.bstart[bi + 1] - sg.ebase;
+    if (P.valid && S.valid && okey_less(S.k, S.tb, P.k, P.tb)) return;
+    unsigned long long l = b0, h = b1;  // A = #{e < P}
+    if (P.valid) {
+        while (l < h) {
+            const unsigned long long mid = (l + h) >> 1;
+            unsigned long long k; uint32_t tb;
+            elem(mid, k, tb);
+            if (okey_less(k, tb, P.k, P.tb)) l = mid + 1; else h = mid;
+        }
+    }
+    fg = l;
+    h = b1;  // B = #{e <= S}
+    if (S.valid) {
+        while (l < h) {
+            const unsigned long long mid = (l + h) >> 1;
+            unsigned long long k; uint32_t tb;
+            elem(mid, k, tb);
+            if (!okey_less(S.k, S.tb, k, tb)) l = mid + 1; else h = mid;
+        }
+    } else {
+        l = b1;
+    }
+    lg = l;
+}
+
 // 2) k_seam_cuts (one thread per bucket of every array): the bucket's first and last sound cut.
 template <typename W>
 __global__ void k_seam_cuts(SolveArgs a) {
     const uint32_t bi = blockIdx.x * blockDim.x + threadIdx.x;
     if (bi >= a.NB || *a.err) return;
-    const unsigned long long NONE = ~0ull;
-    if (a.bstart[bi + 1] == a.bstart[bi]) {
-        a.seam_cut[2 * (size_t)bi] = NONE;
-        a.seam_cut[2 * (size_t)bi + 1] = NONE;
-        return;
-    }
-    const Seg &sg = a.segs[seg_of_bucket(a.segs, a.nseg, bi)];
-    const W *outk = reinterpret_cast<const W *>(sg.keys);
-    auto okey = [&](const OKey &o) { KMax x; x.k = o.k; x.tb = o.tb; x.valid = o.valid; return x; };
-    auto elem = [&](unsigned long long pos, unsigned long long &k, uint32_t &tb) {
-        k = ordbits(word64(outk[pos]), a.dtype);
-        tb = a.out_rows ? a.out_rows[sg.ebase + pos] : 0u;
-    };
-    const KMax P = okey(a.seam_pre[bi]), S = okey(a.seam_suf[bi]);
-    const unsigned long long b0 = a.bstart[bi] - sg.ebase, b1 = a.bstart[bi + 1] - sg.ebase;
-    unsigned long long fg = NONE, lg = NONE;
-    if (!(P.valid && S.valid && okey_less(S.k, S.tb, P.k, P.tb))) {
-        unsigned long long l = b0, h = b1;  // A = #{e < P}
-        if (P.valid) {
-            while (l < h) {
-                const unsigned long long mid = (l + h) >> 1;
-                unsigned long long k; uint32_t tb;
-                elem(mid, k, tb);
-                if (okey_less(k, tb, P.k, P.tb)) l = mid + 1; else h = mid;
-            }
-        }
-        fg = l;
-        l = fg; h = b1;  // B = #{e <= S}
-        if (S.valid) {
-            while (l < h) {
-                const unsigned long long mid = (l + h) >> 1;
-                unsigned long long k; uint32_t tb;
-                elem(mid, k, tb);
-                if (!okey_less(S.k, S.tb, k, tb)) l = mid + 1; else h = mid;
-            }
-        } else {
-            l = b1;
-        }
-        lg = l;
-    }
+    unsigned long long fg = ~0ull, lg = ~0ull;
+    if (a.bstart[bi + 1] != a.bstart[bi])  // (an empty bucket's extremes are not written)
+        seam_cuts<W>(a, a.segs[seg_of_bucket(a.segs, a.nseg, bi)], bi, kmax_of(a.seam_pre[bi]), kmax_of(a.seam_suf[bi]),
+                     fg, lg);
     a.seam_cut[2 * (size_t)bi] = fg;
     a.seam_cut[2 * (size_t)bi + 1] = lg;
+}
+
+// an output range of array s to be sorted again, if it holds two or more elements
+__device__ __forceinline__ void seam_range(const SolveArgs &a, int s, unsigned long long lo, unsigned long long hi) {
+    if (hi - lo < 2) return;
+    atomicAdd(&a.stats[s].repaired, hi - lo);
+    atomicAdd(&a.stats[s].ranges, 1u);
+    SeamRange r; r.lo = lo; r.hi = hi; r.seg = (uint32_t)s; r.pad = 0;
+    if (a.allow_defer && !a.out_rows && hi - lo > a.seam_max) {
+        const uint32_t i = atomicAdd(&a.seam_cnt[1], 1u);
+        a.ranges[a.max_ranges - 1 - i] = r;
+    } else {
+        a.ranges[atomicAdd(&a.seam_cnt[0], 1u)] = r;
+    }
 }
 
 // 3) k_seam_emit (one block per array): the runs between consecutive sound cuts that hold two or
@@ -2222,18 +2323,7 @@ __global__ void __launch_bounds__(SCAN_THREADS) k_seam_emit(SolveArgs a) {
     const uint32_t nb = sg.nb, bb = sg.bbase;
     // a sound cut is a position below n, so NONE (all ones) is the identity of the minimum
     const unsigned long long n = sg.n, NONE = ~0ull;
-    auto emit = [&](unsigned long long lo, unsigned long long hi) {
-        if (hi - lo < 2) return;
-        atomicAdd(&a.stats[s].repaired, hi - lo);
-        atomicAdd(&a.stats[s].ranges, 1u);
-        SeamRange r; r.lo = lo; r.hi = hi; r.seg = (uint32_t)s; r.pad = 0;
-        if (a.allow_defer && !a.out_rows && hi - lo > a.seam_max) {
-            const uint32_t i = atomicAdd(&a.seam_cnt[1], 1u);
-            a.ranges[a.max_ranges - 1 - i] = r;
-        } else {
-            a.ranges[atomicAdd(&a.seam_cnt[0], 1u)] = r;
-        }
-    };
+    auto emit = [&](unsigned long long lo, unsigned long long hi) { seam_range(a, s, lo, hi); };
     auto umin = [](unsigned long long x, unsigned long long y) { return y < x ? y : x; };
     // tiles of PSI * SCAN_THREADS buckets, PSI consecutive ones per thread (later ones first)
     constexpr int PSI = 8;
@@ -2281,6 +2371,51 @@ __global__ void __launch_bounds__(SCAN_THREADS) k_seam_emit(SolveArgs a) {
         t1 = t0;
     }
     if (tid == 0) emit(0, carry != NONE ? carry : n);  // before the first sound cut
+}
+
+// The three steps of a small array in one block: thread t holds bucket t going forward and bucket nb - 1 - t
+// going back.
+template <typename W>
+__global__ void __launch_bounds__(SMALL_BUCKETS) k_seam_small(SolveArgs a) {
+    __shared__ KMax ks[33];
+    __shared__ OKey suf[SMALL_BUCKETS];
+    __shared__ unsigned long long cut[2][SMALL_BUCKETS], wmin[SMALL_BUCKETS / 32];
+    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+    if (*a.err) return;
+    const Seg &sg = a.segs[0];
+    const uint32_t nb = sg.nb, t = (uint32_t)tid;
+    const unsigned long long n = sg.n, NONE = ~0ull;
+    auto full = [&](uint32_t b) { return b < nb && a.bstart[b + 1] > a.bstart[b]; };
+    const uint32_t rb = nb - 1 - t;  // (of no bucket when t >= nb)
+    const KMax later = block_excl_max(t < nb && full(rb) ? kinv(kmax_of(a.blo[rb])) : kmax_none(), ks, nullptr);
+    if (t < nb) suf[rb] = okey_of_kmax(kinv(later));
+    const KMax pre = block_excl_max(full(t) ? kmax_of(a.bhi[t]) : kmax_none(), ks, nullptr);
+    unsigned long long fg = NONE, lg = NONE;
+    if (full(t)) seam_cuts<W>(a, sg, t, pre, kmax_of(suf[t]), fg, lg);
+    cut[0][t] = fg;
+    cut[1][t] = lg;
+    __syncthreads();
+    // the next later bucket's first sound cut: an exclusive minimum over the threads before this one
+    auto umin = [](unsigned long long x, unsigned long long y) { return y < x ? y : x; };
+    unsigned long long x = t < nb ? cut[0][rb] : NONE;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const unsigned long long y = __shfl_up_sync(0xFFFFFFFFu, x, o);
+        if (lane >= o) x = umin(x, y);
+    }
+    unsigned long long ex = __shfl_up_sync(0xFFFFFFFFu, x, 1);
+    if (lane == 0) ex = NONE;
+    if (lane == 31) wmin[wid] = x;
+    __syncthreads();
+    unsigned long long before = lane < wid ? wmin[lane] : NONE, all = wmin[lane];
+#pragma unroll
+    for (int o = 16; o; o >>= 1) {
+        before = umin(before, __shfl_xor_sync(0xFFFFFFFFu, before, o));
+        all = umin(all, __shfl_xor_sync(0xFFFFFFFFu, all, o));
+    }
+    const unsigned long long next = umin(before, ex);
+    if (t < nb && cut[1][rb] != NONE) seam_range(a, 0, cut[1][rb], next != NONE ? next : n);
+    if (tid == 0) seam_range(a, 0, 0, all != NONE ? all : n);  // before the first sound cut
 }
 
 // re-sort out[lo, lo + len) of one array by (key, row): the range is a union of sorted runs. The
@@ -2585,10 +2720,12 @@ cudaError_t launch_polish(const SolveArgs &a, cudaStream_t s) {
 }
 
 template <typename W> static cudaError_t seam_go(const SolveArgs &a, int sms, cudaStream_t s) {
-    cudaError_t e = cudaMemsetAsync(a.seam_cnt, 0, 4 * sizeof(uint32_t), s);
-    if (e != cudaSuccess) return e;
+    cudaError_t e;
     const uint32_t nt = (a.NB + MT_TILE - 1) / MT_TILE;
-    if (a.nseg == 1 && a.NB >= MT_MIN_BUCKETS && nt <= MT_TILE) {
+    const bool small = small_solve(a);
+    if (small) {
+        k_seam_small<W><<<1, SMALL_BUCKETS, 0, s>>>(a);
+    } else if (a.nseg == 1 && a.NB >= MT_MIN_BUCKETS && nt <= MT_TILE) {
         // tile extrema in the cut scratch (free until k_seam_cuts): 2 nt <= 2 NB entries of 16 bytes
         OKey *agg = reinterpret_cast<OKey *>(a.seam_cut);
         k_seam_tiles<<<nt, MT_THREADS, 0, s>>>(a, agg);
@@ -2600,10 +2737,12 @@ template <typename W> static cudaError_t seam_go(const SolveArgs &a, int sms, cu
         k_seam_ps<<<a.nseg, SCAN_THREADS, 0, s>>>(a);
     }
     if ((e = nns_launched(cudaGetLastError())) != cudaSuccess) return e;
-    k_seam_cuts<W><<<(a.NB + 255) / 256, 256, 0, s>>>(a);
-    if ((e = nns_launched(cudaGetLastError())) != cudaSuccess) return e;
-    k_seam_emit<<<a.nseg, SCAN_THREADS, 0, s>>>(a);
-    if ((e = nns_launched(cudaGetLastError())) != cudaSuccess) return e;
+    if (!small) {
+        k_seam_cuts<W><<<(a.NB + 255) / 256, 256, 0, s>>>(a);
+        if ((e = nns_launched(cudaGetLastError())) != cudaSuccess) return e;
+        k_seam_emit<<<a.nseg, SCAN_THREADS, 0, s>>>(a);
+        if ((e = nns_launched(cudaGetLastError())) != cudaSuccess) return e;
+    }
     if (a.rk) {  // one-pass buckets
         const size_t smem = bucket_fixed<W, SOLVE_THREADS>() + (size_t)a.seam_cap * bucket_per<W>(a.pay != nullptr);
         const bool fl = a.dtype == NNSORT_F32 || a.dtype == NNSORT_F64;
@@ -2611,7 +2750,7 @@ template <typename W> static cudaError_t seam_go(const SolveArgs &a, int sms, cu
                          : (fl ? k_seam_sort<W, true, false> : k_seam_sort<W, false, false>);
         if ((e = cudaFuncSetAttribute(kfn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess)
             return e;
-        kfn<<<2 * sms, SOLVE_THREADS, smem, s>>>(a);
+        kfn<<<std::min<unsigned>(a.max_ranges, 2u * (unsigned)sms), SOLVE_THREADS, smem, s>>>(a);
         return nns_launched(cudaGetLastError());
     }
     const size_t fix_smem = ((sizeof(PolishSmem) + 15) & ~(size_t)15) + 2 * sizeof(uint32_t) * SEAM_SMEM_IDX;

@@ -254,6 +254,7 @@ extern "C" int nnsort_sort_noalloc(void *d_keys, int32_t *d_payload, uint64_t n,
     NA_CK(launch_rounds(sa, s));
     NA_CK(launch_finalize(sa, s));
     NA_CK(launch_polish(sa, s));
+    NA_CK(cudaMemsetAsync(L.seam_cnt, 0, 4 * sizeof(uint32_t), s));
     NA_CK(launch_seam_repair(sa, sms, s));
 
     // results: device statistics and the error word, read into host stack memory
