@@ -139,7 +139,8 @@ typedef struct {
     int32_t timing;           /* 1: record per-stage CUDA events into nnsort_stats.ms_stage */
     int32_t polish_blocks;    /* 0: automatic (3); 1, 2 or 3 polish blocks per SM: fewer blocks
                                  let a bucket hold more keys on chip, more blocks leave more L1
-                                 and overlap more buckets */
+                                 and overlap more buckets. Only where the polish is a pass of its
+                                 own (a row trace, or bucket_log2 of 13 and 14) */
 } nnsort_sort_opts;
 
 /* Per-array statistics (Sec. "Model Analysis", Eq. (sorting rate), Eq. (ratio)). */

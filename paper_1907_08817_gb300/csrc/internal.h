@@ -233,9 +233,6 @@ int polish_capacity(int key_bytes, bool payload, bool rows, int wlog, int blocks
 cudaError_t launch_sample(const void *keys, uint64_t n, int key_bytes, int dtype, uint64_t S,
                           uint64_t stream_seed, void *sample_keys, uint32_t *sample_rows,
                           uint32_t *err, cudaStream_t s);
-cudaError_t launch_minmax_norm(const void *sorted_keys, uint64_t S, int key_bytes, int dtype,
-                               int translate, double *norm_out /*lo_val, scale*/,
-                               unsigned long long *lobits_out, cudaStream_t s);
 cudaError_t launch_make_xy(const void *sorted_keys, uint64_t S, int key_bytes, const Norm *nm_dev,
                            float *x, float *label, cudaStream_t s);
 // a training run of the two-layer model of width 64 (k_train_tc.cu)

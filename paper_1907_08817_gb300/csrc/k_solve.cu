@@ -19,6 +19,11 @@
 //                 sorting the leftover and merging it with R_1..R_t is the bucket's elements in
 //                 (key, row) order, so the bucket is sorted whole (a counting pass over bins of
 //                 its key range, or a stable radix sort by key where bins crowd).
+//   k_bucket   -- k_rounds, the out-of-order split and the sort in one block per bucket, where no row trace is
+//                 asked for: the bucket is read once and written once, sorted. The split needs the carry
+//                 from earlier buckets, which is known only after k_finalize: the block writes each round's
+//                 in-order run to memory and k_carried counts its elements below the carry. Buckets too
+//                 large for a block run grid-wide (launch_giant_buckets).
 //   k_seam     -- the buckets' outputs are each sorted; where a non-monotone f lets a later
 //                 bucket hold a key smaller than an earlier bucket's, the affected range is
 //                 located and re-sorted (the polish Remark: out-of-order elements end up at their
@@ -78,7 +83,8 @@ __global__ void k_bucket_order(SolveArgs a, uint32_t heavy, uint32_t *order, uin
     const uint32_t nbk = a.bstart[b + 1] - a.bstart[b];
     if (nbk > heavy) order[atomicAdd(&cnt[0], 1u)] = b;
     else order[a.NB - 1 - atomicAdd(&cnt[1], 1u)] = b;
-    if (a.giant && nbk > a.giant_min) {
+    // after an error (NaN keys, bad positions) no bucket is listed: the listed ones are written back
+    if (a.giant && nbk > a.giant_min && !*a.err) {
         BigRange r;
         r.lo = a.bstart[b]; r.hi = a.bstart[b + 1];
         r.seg = (uint32_t)seg_of_bucket(a.segs, a.nseg, b); r.off = 0; r.b = b; r.pad = 0;
@@ -123,7 +129,8 @@ __global__ void __launch_bounds__(SMALL_BUCKETS) k_bounds_order_small(SolveArgs 
     } else {
         order[a.NB - 1 - atomicAdd(&c[1], 1u)] = tid;
     }
-    if (a.giant && nbk > a.giant_min) {
+    // after an error (NaN keys, bad positions) no bucket is listed: the listed ones are written back
+    if (a.giant && nbk > a.giant_min && !*a.err) {
         BigRange r;
         r.lo = sh[tid]; r.hi = sh[tid + 1]; r.seg = 0; r.off = 0; r.b = tid; r.pad = 0;
         a.giant[atomicAdd(a.giant_cnt, 1u)] = r;

@@ -81,3 +81,30 @@ def test_equal_keys_keep_their_payload_order(dtype, n):
         order = np.argsort(keys, kind="stable")
         np.testing.assert_array_equal(from_dev(dk, keys), keys[order])
         np.testing.assert_array_equal(pay.cpu().numpy(), order)
+
+
+@pytest.mark.parametrize("n,spread", [(40_000, 1.0), (140_000, 0.02), (1_400_000, 0.01), (1_400_000, 1.0)])
+@pytest.mark.parametrize("payload", [False, True])
+def test_refused_calls_leave_the_arrays_untouched(n, spread, payload):
+    """A NaN key, or a position out of range: buckets of every size, those that no block holds included."""
+    rs = np.random.RandomState(n)
+    keys = rs.standard_normal(n).astype(np.float32)
+    L, _, _ = orc.nm_split(n)
+    good = (rs.uniform(0, spread, n) * (L - 1)).astype(np.int64)
+    for fault in ("nan", "slot"):
+        k, sl = keys.copy(), good.copy()
+        if fault == "nan":
+            k[n // 3] = np.nan
+        else:
+            sl[n // 3] = L
+        dk, kt = to_dev(k)
+        pay = torch.arange(n, dtype=torch.int32, device="cuda") if payload else None
+        ds = torch.from_numpy(sl.astype(np.uint32).view(np.int32)).cuda()
+        f = nns.Model.create(orc.F32, 1, 8, 0, np.zeros(25, np.float32), translate="ordbits")
+        before = dk.clone().view(torch.int32)
+        for kw in ({"slots": ds}, {}) if fault == "nan" else ({"slots": ds},):
+            with pytest.raises(nns.NNSortError):
+                nns.sort(dk, pay, None if kw else f, eps=2, key_type=kt, **kw)
+            assert torch.equal(dk.view(torch.int32), before)
+            if payload:
+                assert torch.equal(pay, torch.arange(n, dtype=torch.int32, device="cuda"))
