@@ -165,9 +165,13 @@ namespace {
 std::map<int, cudaMemPool_t> g_pools;  // one per device, made on first use (guarded by g_mu)
 }
 cudaError_t nns::pool_alloc(void **p, size_t bytes, cudaStream_t s) {
-    int dev = 0;
-    cudaError_t e = cudaGetDevice(&dev);
+    // a captured allocation belongs to its graph, and a pool cannot be made during a capture
+    cudaStreamCaptureStatus cap;
+    cudaError_t e = cudaStreamIsCapturing(s, &cap);
     if (e != cudaSuccess) return e;
+    if (cap != cudaStreamCaptureStatusNone) return cudaMallocAsync(p, bytes, s);
+    int dev = 0;
+    if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
     cudaMemPool_t pool;
     {
         std::lock_guard<std::mutex> lk(g_mu);

@@ -52,3 +52,23 @@ def test_server_trains_side_by_side_and_fails_alone(arch):
             else:
                 srv.wait(t)
                 np.testing.assert_array_equal(work[j].view(np.uint64), want[j].view(np.uint64))
+
+
+@pytest.mark.parametrize("h", [5, 32])  # padded and exact widths
+def test_captured_passes_replay_the_same_bits(h):
+    """Buffers of a captured call belong to its graph, not to the library's pool."""
+    rs = np.random.RandomState(h)
+    p, x, gy = (torch.from_numpy(rs.uniform(-1, 1, n).astype(np.float32)).cuda() for n in (3 * h + 1, 4097, 4097))
+
+    def both():
+        return (nns.mlp_forward(p, x, 1, h, 0),) + nns.mlp_backward(p, x, gy, 1, h, 0)
+
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g):
+        got = both()
+    want = both()
+    for _ in range(2):
+        g.replay()
+        torch.cuda.synchronize()
+        for a, b in zip(got, want):
+            assert torch.equal(a, b)
