@@ -46,9 +46,8 @@ WORKLOAD = ("268,435,456 float32 keys lognormal(0,2) with 5% exact duplicates, k
 # recipe; traffic grows in proportion to the keys. A kernel changed since its capture has no entry.
 TRAFFIC_PER_KEY = {
     ("predict", "bf16x2"): 7.363,   # k_predict_bf16_mg<64, split>
-    ("partition", None): 19.78,     # per pass: k_tile_hist 4.22 + k_scatter 15.56
-    ("rounds", None): 6.79,         # k_rounds
-    ("polish", None): 12.58,        # k_polish
+    ("partition", None): 19.53,     # per pass: k_tile_hist 4.10 + k_scatter 15.43
+    ("rounds", None): 12.10,        # k_bucket
 }
 TRAFFIC_SOURCE = "ncu capture of the kernel at 2^26 keys, scaled to the launch's keys"
 # binary32 operations per key on the CUDA cores in the tensor-core predict (layer 1: H FMA; split
@@ -461,14 +460,14 @@ def roofline_of(stage, ms, n, kb, pb, precision, arch, npass, pk):
     elif stage == "predict" and precision == "fp32":
         fpk = mlp_flop_per_key(*arch)
         ach = n * fpk / (ms / 1e3) / 1e12
-        r = {"kernel": "predict (k_predict, binary32 FFMA)", "bound": "alu", "achieved": ach,
+        r = {"kernel": "predict (k_predict1 / k_predict2, binary32 FFMA)", "bound": "alu", "achieved": ach,
              "peak": fp32_peak, "unit": "TFLOP/s", "frac": ach / fp32_peak,
              "peak_kind": "152 SMs x 128 FP32 lanes x 2 FLOP x max SM clock",
              "work": f"{fpk} FLOP per key x {n} keys"}
     else:
         per = {"predict": kb + 4 + pb, "partition": npass * 2 * (kb + 4 + pb),
-               "bucket_bounds": 0, "rounds": kb + 4 + 1, "finalize": 0,
-               "polish": 2 * kb + 5 + 2 * pb, "seam": 0}[stage]
+               "bucket_bounds": 0, "rounds": 2 * kb + 4 + 2 * pb, "finalize": 0,
+               "polish": 0, "seam": 0}[stage]
         ach = n * per / (ms / 1e3) / 1e9
         r = {"kernel": stage, "bound": "hbm", "achieved": ach, "peak": pk["hbm_gbs"],
              "unit": "GB/s", "frac": ach / pk["hbm_gbs"], "peak_kind": f"copy bandwidth, {pk['source']}",
