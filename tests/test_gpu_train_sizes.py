@@ -72,3 +72,21 @@ def test_captured_passes_replay_the_same_bits(h):
         torch.cuda.synchronize()
         for a, b in zip(got, want):
             assert torch.equal(a, b)
+
+
+@pytest.mark.parametrize("n", [1, 63, 65, 4096, 16_384, 16_385, 32_768, 32_769])
+def test_block_product_gradient_at_the_edges_of_its_split(n):
+    """Batches of up to 256 chunks, 512 and beyond take one, two and four chunks of 64 samples per block.
+    Bound: the gradient's stated 1e-4 of the largest component against binary64."""
+    rs = np.random.RandomState(n)
+    h = 32
+    p, x, lab = (torch.from_numpy(rs.uniform(-1, 1, m).astype(np.float32)).cuda() for m in (h * h + 4 * h + 1, n, n))
+    loss, gp = nns.mlp_loss_grad(p, x, lab, 2, h, h)
+    q = p.double().requires_grad_(True)
+    w1, b1, w2, b2, w3, b3 = torch.split(q, [h, h, h * h, h, h, 1])
+    a = torch.relu(x.double()[:, None] * w1 + b1)
+    y = torch.relu(a @ w2.view(h, h).T + b2) @ w3 + b3
+    want = (y - lab.double()).square().mean()
+    want.backward()
+    assert abs(loss.item() - want.item()) <= 1e-5 * want.item()
+    assert (gp.double() - q.grad).abs().max().item() <= 1e-4 * q.grad.abs().max().item()
