@@ -123,7 +123,7 @@ struct BigRange {
     unsigned long long lo, hi;
     uint32_t seg, off, b, pad;
 };
-constexpr uint32_t POLISH_BIG = 1u << 16;  // buckets above this many elements sort multi-block
+constexpr uint32_t POLISH_BIG = 1u << 16;  // two-kernel form: larger buckets sort multi-block
 constexpr uint32_t GIANT_LEAST = 8192;     // no listed bucket is smaller (sizes the lists)
 
 struct SolveArgs {

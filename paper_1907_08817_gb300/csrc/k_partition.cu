@@ -9,8 +9,8 @@
 // One pass reads and writes each element once, in tiles of 4,096. Its offsets come from a scan
 // over per-tile digit histograms (reduce, then scan, then scatter), so no block ever waits on
 // another and several blocks share each SM. A tile ranks its elements per digit stably (a warp finds
-// the lanes holding the same digit through shared-memory match words); writes go out through a shared-memory reorder buffer in digit order, so each digit's run leaves as
-// coalesced stores.
+// the lanes holding the same digit through shared-memory match words); writes go out through a
+// shared-memory reorder buffer in digit order, so each digit's run leaves as coalesced stores.
 #include <algorithm>
 #include <cstddef>
 #include <type_traits>
@@ -29,8 +29,8 @@ namespace nns {
 
 // ---------------------------------------------------------------------------------------------
 // The partition pass without look-back. The tiles' global offsets come from a scan over tile
-// histograms instead of from waits on earlier tiles, so every block is independent: two blocks run
-// on each SM and one block's loads overlap the other's ranking and stores.
+// histograms instead of from waits on earlier tiles, so every block is independent: several run
+// on each SM and one block's loads overlap the others' ranking and stores.
 namespace {
 constexpr int TH_THREADS = 256, TH_ITEMS = SC_TILE / TH_THREADS, TH_NW = TH_THREADS / 32;  // histogram blocks
 constexpr int SC_THREADS = 256, SC_ITEMS = SC_TILE / SC_THREADS, SC_NW = SC_THREADS / 32;  // scatter blocks
