@@ -601,9 +601,10 @@ __global__ void __launch_bounds__(NG * TC_THREADS, 1) k_predict_bf16_mg(PredictA
 }
 
 // The largest |x| for which the activations stay below 10^6 (so that the split's FP16 part is finite)
-// and every z far below the overflow of 2 z; -1 when a weight is not finite, or too large, or its half is
-// not exact.
-template <int H> static float plain_limit(const float *P) {
+// and every z is finite and far below the overflow of 2 z; -1 when a weight is not finite, or too large
+// (in the split form W2 is held as FP16 too: from 65,520 on that copy is infinite, and z infinite or NaN,
+// which ReLU turns into 0 and z + |z| does not), or its half is not exact.
+template <int H, bool SPLIT> static float plain_limit(const float *P) {
     float w1 = 0.0f, b1 = 0.0f, w2 = 0.0f, b2 = 0.0f;
     bool ok = true;
     for (int i = 0; i < 4 * H + H * H + 1; ++i) ok = ok && std::isfinite(P[i]);
@@ -615,7 +616,7 @@ template <int H> static float plain_limit(const float *P) {
         ok = ok && (w3 == 0.0f || w3 >= 1e-30f);
     }
     for (int i = 0; i < H * H; ++i) w2 = std::max(w2, std::fabs(P[2 * H + i]));
-    if (!ok || b1 > 1e5f || w2 > 1e20f || b2 > 1e30f) return -1.0f;
+    if (!ok || b1 > 1e5f || w2 > (SPLIT ? 65504.0f : 1e20f) || b2 > 1e30f) return -1.0f;
     return w1 > 0.0f ? std::min(1e30f, 5e5f / w1) : 1e30f;
 }
 
@@ -628,7 +629,7 @@ static cudaError_t bf16_mg_go(const PredictArgs &p, int sms, cudaStream_t s) {
         c.b1[j] = p.host_pad[H + j];
         c.w3h[j] = 0.5f * p.host_pad[3 * H + H * H + j];
     }
-    c.xlim = plain_limit<H>(p.host_pad);
+    c.xlim = plain_limit<H, SPLIT>(p.host_pad);
     c.b3 = p.host_pad[4 * H + H * H];
     const Seg &g = *p.host_seg;
     c.nm_hi = g.nm_hi;

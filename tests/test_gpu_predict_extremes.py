@@ -1,0 +1,40 @@
+"""F(x) and positions where a model's numbers are far from a trained one's: weights that the split form's
+FP16 part cannot hold."""
+import numpy as np
+import pytest
+
+from helpers import to_dev
+from oracle import oracle as orc
+import workloads as W
+
+pytestmark = pytest.mark.gpu
+
+torch = pytest.importorskip("torch")
+if not torch.cuda.is_available():
+    pytest.skip("needs a GPU", allow_module_level=True)
+import paper_1907_08817_gb300 as nns  # noqa: E402
+
+
+@pytest.mark.parametrize("h", [16, 32, 64])
+@pytest.mark.parametrize("w2", [65_504.0, 65_520.0, 1e5, -1e5])
+def test_wide_second_layer_weights_do_not_depend_on_the_warp(h, w2):
+    """A second-layer weight beyond FP16's range makes the split form's product with the low part infinite
+    or NaN; the epilogues must agree on it: a key's F(x) may not depend on its warp's other keys."""
+    n = 4096
+    near = (np.uint64(1 << 40) + W.uniform_u64(n, 5) % np.uint64(1 << 30)).astype(np.uint64)
+    near[1::7] = np.uint64(1 << 40)  # x = 0: activations without a low part
+    mixed = near.copy()
+    far = np.arange(0, n, 32)  # one in every warp
+    mixed[far] = np.uint64((1 << 63) + 12345)
+    p = orc.init_params(2, h, h, 3)
+    p[2 * h:2 * h + h * h:h + 1] = w2  # the diagonal
+    f = nns.Model.create(orc.U64, 2, h, h, p, translate="ordbits", lo_bits=1 << 40, scale=2.0 ** -30)
+    keep = np.ones(n, bool)
+    keep[far] = False
+    got = []
+    for keys in (near, mixed):
+        dk, kt = to_dev(keys)
+        s, y = nns.predict(dk, f, precision="bf16x2", key_type=kt)
+        got.append((s.cpu().numpy()[keep], y.cpu().numpy()[keep].view(np.uint32)))
+    np.testing.assert_array_equal(got[0][0], got[1][0])
+    np.testing.assert_array_equal(got[0][1], got[1][1])
