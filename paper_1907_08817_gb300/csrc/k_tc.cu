@@ -549,6 +549,8 @@ __global__ void __launch_bounds__(NG * TC_THREADS, 1) k_predict_bf16_mg(PredictA
                 if (c0 + 16 < H) tmem_wait_ld();
             }
         } else {
+            // W3 itself (halving may have rounded it)
+            const float *W3 = a.segs[0].params + 3 * H + H * H;
 #pragma unroll 1
             for (int p = 0; p < KPT; ++p) {
                 unsigned long long t = pk2(cst.b3, 0.0f);
@@ -564,8 +566,8 @@ __global__ void __launch_bounds__(NG * TC_THREADS, 1) k_predict_bf16_mg(PredictA
                     }
 #pragma unroll
                     for (int q = 0; q < 16; q += 2) {
-                        const unsigned long long w = pk2(cst.w3h[c0 + q], cst.w3h[c0 + q + 1]);
-                        t = fma2_rn(add2_rn(w, w), pk2(relu_f(acc[q]), relu_f(acc[q + 1])), t);
+                        const unsigned long long w = pk2(__ldg(W3 + c0 + q), __ldg(W3 + c0 + q + 1));
+                        t = fma2_rn(w, pk2(relu_f(acc[q]), relu_f(acc[q + 1])), t);
                     }
                 }
                 if (p == 0) yy[0] = t;

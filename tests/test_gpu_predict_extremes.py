@@ -1,5 +1,5 @@
 """F(x) and positions where a model's numbers are far from a trained one's: weights that the split form's
-FP16 part cannot hold."""
+FP16 part cannot hold, and output weights whose half is not a binary32 number."""
 import numpy as np
 import pytest
 
@@ -38,3 +38,16 @@ def test_wide_second_layer_weights_do_not_depend_on_the_warp(h, w2):
         got.append((s.cpu().numpy()[keep], y.cpu().numpy()[keep].view(np.uint32)))
     np.testing.assert_array_equal(got[0][0], got[1][0])
     np.testing.assert_array_equal(got[0][1], got[1][1])
+
+
+@pytest.mark.parametrize("h", [16, 32, 64])
+def test_output_weights_below_the_normal_range(h):
+    """W3 = 2^-149 has no half; with z = 2^126 every unit adds exactly 2^-23."""
+    p = np.zeros(h * h + 4 * h + 1, np.float32)
+    p[2 * h + h * h:3 * h + h * h] = 2.0 ** 126  # b2
+    p[3 * h + h * h:4 * h + h * h] = np.float32(2.0 ** -149)  # W3
+    f = nns.Model.create(orc.U64, 2, h, h, p, translate="ordbits", lo_bits=0, scale=2.0 ** -30)
+    dk, kt = to_dev(W.uniform_u64(1000, 7) % np.uint64(1 << 30))
+    for precision in ("bf16", "bf16x2"):
+        _, y = nns.predict(dk, f, precision=precision, key_type=kt)
+        assert torch.equal(y, torch.full_like(y, h * 2.0 ** -23))
