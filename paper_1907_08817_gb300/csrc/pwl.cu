@@ -272,17 +272,25 @@ __global__ void __launch_bounds__(PRED_THREADS) k_predict_pwl(PredictArgs a) {
             float yh, ye;
             two_sum(p, c.z, yh, ye);
             const float yl = __fadd_rn(__fadd_rn(e, c.w), ye);
-            // floor(yh + yl), clamped to [0, L - 1]; below -1 or from 2^32 on the pair's low part (at most
-            // 256 there) cannot move the result, since L <= 2^32 - 512; NaN (an infinite or NaN key) goes
-            // to position 0
+            // floor(yh + yl), clamped to [0, L - 1]; below -1 or from 2^33 on the pair's low part is left
+            // out, and NaN (an infinite or NaN key) goes to position 0. The low part is within 2^-24 of A d
+            // and C, which cancel: where the model is steep it is many positions, and the sum takes 64 bits
+            // when it or the high part leaves the 32 that nearly every key's fit.
             uint32_t slot = 0;
-            if (yh >= 4294967296.0f) {
-                slot = Lm1;
-            } else if (yh >= -1.0f) {
-                const float f = floorf(yh);
-                const float g = floorf(__fadd_rn(__fsub_rn(yh, f), yl));
-                const long long sl = (f < 0.0f ? -1ll : (long long)__float2uint_rz(f)) + (long long)__float2int_rz(g);
-                slot = sl < 0 ? 0u : (sl > (long long)Lm1 ? Lm1 : (uint32_t)sl);
+            if (fabsf(yl) < 1073741824.0f) {
+                if (yh >= 8589934592.0f) {
+                    slot = Lm1;
+                } else if (yh >= -1.0f) {
+                    const float f = floorf(yh);
+                    const float g = floorf(__fadd_rn(__fsub_rn(yh, f), yl));
+                    const long long fi = yh < 4294967296.0f ? (f < 0.0f ? -1ll : (long long)__float2uint_rz(f))
+                                                            : __float2ll_rz(f);
+                    const long long sl = fi + (long long)__float2int_rz(g);
+                    slot = sl < 0 ? 0u : (sl > (long long)Lm1 ? Lm1 : (uint32_t)sl);
+                }
+            } else {  // (NaN where the high part is infinite)
+                const double v = isfinite(yl) ? (double)yh + (double)yl : (double)yh;
+                slot = v >= (double)Lm1 ? Lm1 : (v > 0.0 ? (uint32_t)__double2uint_rz(v) : 0u);
             }
             if (a.gs) a.gs[i] = gs_base + slot;
             if (a.row_init) a.row_init[i] = (uint32_t)i;

@@ -1,5 +1,8 @@
 """F(x) and positions where a model's numbers are far from a trained one's: weights that the split form's
-FP16 part cannot hold, and output weights whose half is not a binary32 number."""
+FP16 part cannot hold, weights whose half is not a binary32 number, and slopes so steep that the low part
+of the compiled form's pair carries many positions."""
+from fractions import Fraction
+
 import numpy as np
 import pytest
 
@@ -51,3 +54,27 @@ def test_output_weights_below_the_normal_range(h):
     for precision in ("bf16", "bf16x2"):
         _, y = nns.predict(dk, f, precision=precision, key_type=kt)
         assert torch.equal(y, torch.full_like(y, h * 2.0 ** -23))
+
+
+@pytest.mark.parametrize("log_slope", [1, 10, 20, 26])
+@pytest.mark.parametrize("dtype", ["u32", "u64"])
+@pytest.mark.parametrize("m", [1.25, 4294000.0])
+def test_compiled_positions_of_steep_models(log_slope, dtype, m):
+    """F = slope (x - c) around one key c, with few positions and with nearly 2^32. The pair of binary32
+    holds A d, of magnitude slope * n m, to 47 bits and adds C of the same magnitude: positions are within
+    2^-46 of that of the exact line's, and one of rounding."""
+    n, slope = 1000, 2 ** log_slope
+    step = max(1, 2 ** 32 // slope // n)
+    b1 = np.float32(-((1 << 31) + 12345) / 2.0 ** 32)
+    c = int(-Fraction(float(b1)) * 2 ** 32)  # the key where F leaves 0
+    keys = np.minimum(c - 20 + step * np.arange(n, dtype=np.int64), (1 << 32) - 1).astype(
+        np.uint32 if dtype == "u32" else np.uint64)
+    f = nns.Model.create(getattr(orc, dtype.upper()), 1, 1, 0, np.array([1.0, b1, slope, 0.0], np.float32),
+                         translate="ordbits", lo_bits=0, scale=2.0 ** -32)
+    dk, kt = to_dev(keys)
+    got = nns.predict(dk, f, m=m, precision="pwl", key_type=kt, want_y=False)[0].cpu().numpy()
+    nm = Fraction(n) * Fraction(float(np.float32(m)))
+    want = [min(max(int(nm * slope * (int(k) - c) / 2 ** 32 + Fraction(1, 2)), 0), int(nm)) if k > c else 0
+            for k in keys]
+    bound = 1 + int(nm * slope / 2 ** 46)
+    assert np.abs(got - np.array(want)).max() <= bound
