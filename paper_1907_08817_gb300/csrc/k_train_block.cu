@@ -46,6 +46,11 @@ __device__ __forceinline__ double value_of_key(uint64_t w, int dtype) {
     return __ull2double_rn(w);
 }
 
+template <int N> __device__ __forceinline__ float pairwise_sum(const float *v) {
+    if constexpr (N == 1) return v[0];
+    else return __fadd_rn(pairwise_sum<N / 2>(v), pairwise_sum<N / 2>(v + N / 2));
+}
+
 // fixed-order sum of v over the 32 lanes (the result in lane 0)
 __device__ __forceinline__ float tb_warp_sum(float v) {
 #pragma unroll
@@ -66,9 +71,11 @@ template <int H> __host__ __device__ constexpr size_t tb_smem(uint32_t cap) {
 // A step in three phases: (1) four samples per thread: forward pass, loss term and upstream gradient gy;
 // (2) a (row, unit) per thread: over the row's samples with a positive activation, the sums of gy, gy x and
 // gy h (two samples per packed instruction; the gradients of W1 and b1 are W3 times the first two); (3)
-// a parameter per thread: its row sums in order, then Adam. Every sum has a fixed order. The first form
+// a parameter per thread: its row sums pairwise, then Adam. Every sum has a fixed order. The first form
 // kept all 3 H + 1 sums per thread and reduced each over the block by shuffles; 1,024 models of
-// 1-16-1 on 1% samples of 1K..1M keys, 100 full-batch steps: 4.42 ms, now 2.70 ms.
+// 1-16-1 on 1% samples of 1K..1M keys, 100 full-batch steps: 4.42 ms, now 2.59 ms. Rows of consecutive
+// samples, added one after another, took the sums' rms error from 4.6e-8 to 8.3e-8 of their terms'
+// magnitudes (and 2.70 ms); dealt out and added pairwise it is 4.6e-8 again.
 template <typename W, int H, int T>
 __global__ void __launch_bounds__(T) k_train_block(TrainBlockArgs a) {
     constexpr int P = 3 * H + 1;  // W1[H] b1[H] W3[H] b3 (padded layout of one hidden layer)
@@ -235,17 +242,18 @@ __global__ void __launch_bounds__(T) k_train_block(TrainBlockArgs a) {
                 *reinterpret_cast<float4 *>(sgy + i) = make_float4(gy[0], gy[1], gy[2], gy[3]);
             }
             __syncthreads();
-            // rows of a multiple of four samples: enough of them to spread the chunk over the threads
-            uint32_t want = (cn + 15) / 16;
-            want = want < TB_ROWS ? want : TB_ROWS;
-            const uint32_t per = ((cn + want - 1) / want + 3) & ~3u, nrow = (cn + per - 1) / per;
+            // rows of groups of four samples, enough of them to spread the chunk over the threads. Row k takes
+            // groups k, k + nrow, ...: neighbours in the sorted sample share their residual's sign, and a sum
+            // that runs through neighbours grows, and rounds, far beyond the whole sum
+            uint32_t nrow = (cn + 15) / 16;
+            nrow = nrow < TB_ROWS ? nrow : TB_ROWS;
+            const uint32_t stride = 4 * nrow;
             for (uint32_t t = tid; t < nrow * H; t += T) {
                 const uint32_t k = t / H, j = t % H;
-                const uint32_t i0 = k * per, i1 = min(cn4, i0 + per);
                 const unsigned long long w1 = pk2(sp[j], sp[j]), b1 = pk2(sp[H + j], sp[H + j]);
-                unsigned long long s1 = 0, s2 = 0, s3 = 0;
+                unsigned long long sa1 = 0, sa2 = 0, sa3 = 0, sb1 = 0, sb2 = 0, sb3 = 0;
 #pragma unroll 2
-                for (uint32_t i = i0; i < i1; i += 4) {
+                for (uint32_t i = 4 * k; i < cn4; i += stride) {
                     const ulonglong2 xv = *reinterpret_cast<const ulonglong2 *>(cx + i);
                     const float4 gv = *reinterpret_cast<const float4 *>(sgy + i);
                     const unsigned long long ha = fma2_rn(w1, xv.x, b1), hb = fma2_rn(w1, xv.y, b1);
@@ -254,25 +262,24 @@ __global__ void __launch_bounds__(T) k_train_block(TrainBlockArgs a) {
                     upk2(hb, h2, h3);
                     const unsigned long long ga = pk2(h0 > 0.0f ? gv.x : 0.0f, h1 > 0.0f ? gv.y : 0.0f);
                     const unsigned long long gb = pk2(h2 > 0.0f ? gv.z : 0.0f, h3 > 0.0f ? gv.w : 0.0f);
-                    s1 = fma2_rn(ga, xv.x, s1);
-                    s2 = add2_rn(s2, ga);
-                    s3 = fma2_rn(ga, ha, s3);
-                    s1 = fma2_rn(gb, xv.y, s1);
-                    s2 = add2_rn(s2, gb);
-                    s3 = fma2_rn(gb, hb, s3);
+                    sa1 = fma2_rn(ga, xv.x, sa1);
+                    sa2 = add2_rn(sa2, ga);
+                    sa3 = fma2_rn(ga, ha, sa3);
+                    sb1 = fma2_rn(gb, xv.y, sb1);
+                    sb2 = add2_rn(sb2, gb);
+                    sb3 = fma2_rn(gb, hb, sb3);
                 }
-                float e, f;
                 float *o = part + k * (3 * H);
                 const bool add = c0 && k < rows;  // a row of an earlier chunk
-                upk2(s1, e, f);
-                e = __fadd_rn(e, f);
-                o[j] = add ? __fadd_rn(o[j], e) : e;
-                upk2(s2, e, f);
-                e = __fadd_rn(e, f);
-                o[H + j] = add ? __fadd_rn(o[H + j], e) : e;
-                upk2(s3, e, f);
-                e = __fadd_rn(e, f);
-                o[2 * H + j] = add ? __fadd_rn(o[2 * H + j], e) : e;
+                auto put = [&](float *q, unsigned long long u, unsigned long long v) {
+                    float e, f;
+                    upk2(add2_rn(u, v), e, f);
+                    e = __fadd_rn(e, f);
+                    *q = add ? __fadd_rn(*q, e) : e;
+                };
+                put(o + j, sa1, sb1);
+                put(o + H + j, sa2, sb2);
+                put(o + 2 * H + j, sa3, sb3);
             }
             rows = rows > nrow ? rows : nrow;
         }
@@ -285,8 +292,17 @@ __global__ void __launch_bounds__(T) k_train_block(TrainBlockArgs a) {
         if (tid < P) {
             float gs = 0.0f;
             if (tid < 3 * H) {
-#pragma unroll 8
-                for (uint32_t k = 0; k < rows; ++k) gs = __fadd_rn(gs, part[k * (3 * H) + tid]);
+                // the rows pairwise, eight at a time
+                float blk[TB_ROWS / 8];
+#pragma unroll
+                for (uint32_t q = 0; q < TB_ROWS / 8; ++q) {
+                    float v[8];
+#pragma unroll
+                    for (uint32_t r = 0; r < 8; ++r)
+                        v[r] = 8 * q + r < rows ? part[(8 * q + r) * (3 * H) + tid] : 0.0f;
+                    blk[q] = pairwise_sum<8>(v);
+                }
+                gs = pairwise_sum<TB_ROWS / 8>(blk);
                 if (tid < 2 * H) gs = __fmul_rn(gs, sp[2 * H + tid % H]);
             } else {
 #pragma unroll
