@@ -61,6 +61,7 @@ struct Workspace {
     void *host_dev = nullptr;      // device staging for the host-array entry point
     size_t host_cap = 0;
     cudaEvent_t ev[8] = {};        // stage timing
+    cudaEvent_t counted = nullptr; // the bucket counts have reached the staging area
 };
 std::map<std::pair<int, cudaStream_t>, Workspace *> g_ws;
 
@@ -357,6 +358,7 @@ int nnsort_release(void) {
         if (w->part) cudaFree(w->part);
         if (w->pinned) cudaFreeHost(w->pinned);
         if (w->host_dev) cudaFree(w->host_dev);
+        if (w->counted) cudaEventDestroy(w->counted);
         delete w;
     }
     g_ws.clear();
@@ -820,11 +822,11 @@ int run_sort(const std::vector<SegIn> &in, const nnsort_sort_opts *op, int dtype
     if ((rc = get_ws(s, &w))) return rc;
     if ((rc = ensure_arena(w, pwl_off + pwl_bytes, s))) return rc;
     if ((rc = ensure_part(w, P.N, s))) return rc;
-    // staging: the segment table, then the statistics, the seam counters and the long seam ranges
+    // staging: the segment table, then the statistics, the counters and the long seam ranges
     // (disjoint and longer than SEAM_CTA_LEAST each, so at most N / SEAM_CTA_LEAST of them)
     const size_t pin_stats = align_up(sizeof(Seg) * nseg, 64);
     const size_t pin_cnt = pin_stats + align_up(align_up(sizeof(SegStats) * nseg, 256) + 16, 64);
-    const size_t pin_rng = pin_cnt + 64;
+    const size_t pin_rng = pin_cnt + 1024;
     const size_t pin_big = align_up(pin_rng + sizeof(SeamRange) * (P.N / SEAM_CTA_LEAST + 1), 64);
     const size_t pin_pwl = align_up(pin_big + sizeof(BigRange) * (P.N / POLISH_BIG + 1), 64);
     const size_t pin_need = pin_pwl + pwl_bytes + 256;
@@ -987,9 +989,28 @@ int run_sort(const std::vector<SegIn> &in, const nnsort_sort_opts *op, int dtype
         sa.order = L.order;
         if (onepass) sa.heavy_cnt = L.order_cnt;
     }
-    if (onepass) {
-        CK(launch_buckets(sa, sms, s));
-        if (giants) CK(launch_giant_buckets(sa, gr, o.eps, sms, s));
+    uint32_t nbig = 0, big_total = 0;  // one-pass form: listed giant buckets and their elements
+    if (onepass && !giants) {
+        CK(launch_buckets(sa, s));
+        CK(launch_heavy_buckets(sa, sms, s));
+    } else if (onepass) {
+        // few arrays hold a giant bucket or even a heavy one, and each of those paths is several launches:
+        // the host reads how many there are while the other buckets run (20,000 f32 keys: 251 us a sort, 303
+        // with every launch made in any case; 1,000,000 u64 key-value pairs with giants: 861, 868)
+        const size_t span = (size_t)((unsigned char *)(L.giant_cnt + 2) - (unsigned char *)L.order_cnt);
+        unsigned char *hc = w->pinned + pin_cnt;
+        if (!w->counted) CK(cudaEventCreateWithFlags(&w->counted, cudaEventDisableTiming));
+        CK(cudaMemcpyAsync(hc, L.order_cnt, span, cudaMemcpyDeviceToHost, s));
+        CK(cudaEventRecord(w->counted, s));
+        CK(launch_buckets(sa, s));
+        CK(cudaEventSynchronize(w->counted));
+        uint32_t nheavy = 0;
+        std::memcpy(&nheavy, hc, 4);
+        std::memcpy(&nbig, hc + span - 8, 4);
+        std::memcpy(&big_total, hc + span - 4, 4);
+        if (nbig > P.N / sa.giant_min + 1 || big_total > P.N) return NNSORT_E_STATE;
+        if (nheavy) CK(launch_heavy_buckets(sa, sms, s));
+        if (nbig) CK(launch_giant_buckets(sa, gr, o.eps, sms, s));
     } else {
         if (!rows) {
             sa.big = L.big;
@@ -1004,31 +1025,29 @@ int run_sort(const std::vector<SegIn> &in, const nnsort_sort_opts *op, int dtype
     CK(mark(5));
     if (!onepass) CK(launch_polish(sa, s));
     else if (!small) CK(launch_carried(sa, s));
-    if (giants && !rows) {
-        // buckets too large for one block: one wait, then one multi-block sort of all of them
+    if (onepass) {
+        // buckets too large for one block: one multi-block sort of all of them
+        if (nbig && (rc = sort_big_buckets(w, L, L.giant, nbig, big_total, fi, kb, dtype, anypay, s))) return rc;
+    } else if (giants && !rows) {
+        // the same after one wait for k_polish's list; the packed offsets are made here
         uint32_t *hc = reinterpret_cast<uint32_t *>(w->pinned + pin_cnt);
-        CK(cudaMemcpyAsync(hc, onepass ? L.giant_cnt : L.big_cnt, 2 * sizeof(uint32_t), cudaMemcpyDeviceToHost, s));
+        CK(cudaMemcpyAsync(hc, L.big_cnt, sizeof(uint32_t), cudaMemcpyDeviceToHost, s));
         CK(cudaStreamSynchronize(s));
-        const uint32_t nbig = hc[0];
+        nbig = hc[0];
         if (nbig) {
-            if (nbig > P.N / sa.giant_min + 1) return NNSORT_E_STATE;
-            uint64_t total = hc[1];
-            if (!onepass) {
-                // k_polish's list: the packed offsets are made here
-                BigRange *hb = reinterpret_cast<BigRange *>(w->pinned + pin_big);
-                CK(cudaMemcpyAsync(hb, L.big, sizeof(BigRange) * nbig, cudaMemcpyDeviceToHost, s));
-                CK(cudaStreamSynchronize(s));
-                total = 0;
-                for (uint32_t j = 0; j < nbig; ++j) {
-                    if (hb[j].seg >= (uint32_t)nseg || hb[j].lo >= hb[j].hi || hb[j].hi > P.N) return NNSORT_E_STATE;
-                    hb[j].off = (uint32_t)total;
-                    total += hb[j].hi - hb[j].lo;
-                }
-                CK(cudaMemcpyAsync(L.big, hb, sizeof(BigRange) * nbig, cudaMemcpyHostToDevice, s));
+            if (nbig > P.N / POLISH_BIG + 1) return NNSORT_E_STATE;
+            BigRange *hb = reinterpret_cast<BigRange *>(w->pinned + pin_big);
+            CK(cudaMemcpyAsync(hb, L.big, sizeof(BigRange) * nbig, cudaMemcpyDeviceToHost, s));
+            CK(cudaStreamSynchronize(s));
+            uint64_t total = 0;
+            for (uint32_t j = 0; j < nbig; ++j) {
+                if (hb[j].seg >= (uint32_t)nseg || hb[j].lo >= hb[j].hi || hb[j].hi > P.N) return NNSORT_E_STATE;
+                hb[j].off = (uint32_t)total;
+                total += hb[j].hi - hb[j].lo;
             }
             if (total > P.N) return NNSORT_E_STATE;
-            if ((rc = sort_big_buckets(w, L, onepass ? L.giant : L.big, nbig, total, fi, kb, dtype, anypay, s)))
-                return rc;
+            CK(cudaMemcpyAsync(L.big, hb, sizeof(BigRange) * nbig, cudaMemcpyHostToDevice, s));
+            if ((rc = sort_big_buckets(w, L, L.big, nbig, total, fi, kb, dtype, anypay, s))) return rc;
         }
     }
     CK(mark(6));

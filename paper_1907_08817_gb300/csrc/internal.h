@@ -198,17 +198,18 @@ struct GiantRounds {
     uint32_t cap;                 // list entries
 };
 // the same for buckets that no one-pass block holds, their runs split round by round from the claim
-// table (cnt: elements stored and run elements so far, two words per entry); count[1] receives the total
-// of their elements and the list their packed offsets
+// table (cnt: elements stored and run elements so far, two words per entry); the list receives their packed
+// offsets
 cudaError_t launch_giant_buckets(const SolveArgs &a, const GiantRounds &g, int eps, int sms, cudaStream_t s);
 cudaError_t launch_giant_rounds(const SolveArgs &a, const GiantRounds &g, int eps, int sms, cudaStream_t s);
 cudaError_t launch_rounds(const SolveArgs &a, cudaStream_t s);
-// every bucket of at most bucket_cap[2] elements in one pass (rounds, runs and sorted output), and their
-// out-of-order counts once the carries are known; larger ones are left to launch_giant_buckets and the
-// host's multi-block sort
+// every bucket of at most bucket_cap[0] elements in one pass (rounds, runs and sorted output), then the
+// heavy ones of at most bucket_cap[2] (if the array can hold any), and their out-of-order counts once the
+// carries are known; larger ones are left to launch_giant_buckets and the host's multi-block sort
 bool buckets_ok(int wlog, bool rows);
 void bucket_capacities(SolveArgs &a, bool payload);
-cudaError_t launch_buckets(const SolveArgs &a, int sms, cudaStream_t s);
+cudaError_t launch_buckets(const SolveArgs &a, cudaStream_t s);
+cudaError_t launch_heavy_buckets(const SolveArgs &a, int sms, cudaStream_t s);
 cudaError_t launch_carried(const SolveArgs &a, cudaStream_t s);
 // one array of few buckets: bounds and order, finalize and carried counts, in one launch each
 bool small_solve(const SolveArgs &a);

@@ -89,6 +89,7 @@ __global__ void k_bucket_order(SolveArgs a, uint32_t heavy, uint32_t *order, uin
         r.lo = a.bstart[b]; r.hi = a.bstart[b + 1];
         r.seg = (uint32_t)seg_of_bucket(a.segs, a.nseg, b); r.off = 0; r.b = b; r.pad = 0;
         a.giant[atomicAdd(a.giant_cnt, 1u)] = r;
+        atomicAdd(a.giant_cnt + 1, nbk);
     }
 }
 
@@ -134,6 +135,7 @@ __global__ void __launch_bounds__(SMALL_BUCKETS) k_bounds_order_small(SolveArgs 
         BigRange r;
         r.lo = sh[tid]; r.hi = sh[tid + 1]; r.seg = 0; r.off = 0; r.b = tid; r.pad = 0;
         a.giant[atomicAdd(a.giant_cnt, 1u)] = r;
+        atomicAdd(a.giant_cnt + 1, nbk);
     }
 }
 bool small_solve(const SolveArgs &a) { return a.nseg == 1 && a.rk && a.NB <= SMALL_BUCKETS; }
@@ -1682,7 +1684,7 @@ __global__ void __launch_bounds__(T, TIER == 0 ? 1024 / T : TIER == 1 ? 2 : 1) k
 // by one block per bucket from the claim table, right after the round's claims.
 constexpr int GT = 256, GI = 16;  // threads of a grid-wide block, elements per lane and chunk
 
-// packed offsets of the listed buckets (one block) and their total
+// packed offsets of the listed buckets (one block)
 __global__ void __launch_bounds__(1024) k_giant_offsets(GiantRounds g) {
     __shared__ uint32_t scratch[33];
     const uint32_t n = g.count[0];
@@ -1695,7 +1697,6 @@ __global__ void __launch_bounds__(1024) k_giant_offsets(GiantRounds g) {
         if (j < n) g.list[j].off = base + ex;
         base += tot;
     }
-    if (threadIdx.x == 0) g.count[1] = base;
 }
 
 // fn(j, element's place in the partitioned arrays, its index in the bucket) for every element
@@ -2007,23 +2008,30 @@ static cudaError_t bucket_go2(const SolveArgs &a, unsigned grid, cudaStream_t s)
         return fl ? bucket_go<W, true, true, TIER, T>(a, grid, s) : bucket_go<W, false, true, TIER, T>(a, grid, s);
     return fl ? bucket_go<W, true, false, TIER, T>(a, grid, s) : bucket_go<W, false, false, TIER, T>(a, grid, s);
 }
-template <typename W> static cudaError_t buckets_go(const SolveArgs &a, int sms, cudaStream_t s) {
+template <typename W> static cudaError_t buckets_go(const SolveArgs &a, cudaStream_t s) {
     cudaError_t e;
     switch (a.bucket_threads) {
     case 512: e = bucket_go2<W, 0, 512>(a, a.NB, s); break;
     case 256: e = bucket_go2<W, 0, 256>(a, a.NB, s); break;
     default: e = bucket_go2<W, 0, 128>(a, a.NB, s);
     }
-    if (e != cudaSuccess || !a.heavy_cnt) return e;
+    return e;
+}
+template <typename W> static cudaError_t heavy_buckets_go(const SolveArgs &a, int sms, cudaStream_t s) {
+    cudaError_t e;
     if (a.bucket_cap[1] > a.bucket_cap[0] &&
         (e = bucket_go2<W, 1, 512>(a, std::min<unsigned>(a.NB, 2u * (unsigned)sms), s)) != cudaSuccess)
         return e;
     if (a.N <= (uint64_t)a.bucket_cap[1]) return cudaSuccess;
     return bucket_go2<W, 2, 512>(a, std::min<unsigned>(a.NB, (unsigned)sms), s);
 }
-cudaError_t launch_buckets(const SolveArgs &a, int sms, cudaStream_t s) {
+cudaError_t launch_buckets(const SolveArgs &a, cudaStream_t s) {
     if (a.NB == 0) return cudaSuccess;
-    return a.key_bytes == 4 ? buckets_go<uint32_t>(a, sms, s) : buckets_go<uint64_t>(a, sms, s);
+    return a.key_bytes == 4 ? buckets_go<uint32_t>(a, s) : buckets_go<uint64_t>(a, s);
+}
+cudaError_t launch_heavy_buckets(const SolveArgs &a, int sms, cudaStream_t s) {
+    if (a.NB == 0 || !a.heavy_cnt) return cudaSuccess;
+    return a.key_bytes == 4 ? heavy_buckets_go<uint32_t>(a, sms, s) : heavy_buckets_go<uint64_t>(a, sms, s);
 }
 cudaError_t launch_finalize_small(const SolveArgs &a, cudaStream_t s) {
     if (a.key_bytes == 4) k_finalize_small<uint32_t><<<1, SMALL_BUCKETS, 0, s>>>(a);
