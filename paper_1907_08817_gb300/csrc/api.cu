@@ -949,9 +949,12 @@ int run_sort(const std::vector<SegIn> &in, const nnsort_sort_opts *op, int dtype
         bucket_capacities(sa, anypay);
         heavy = (uint64_t)sa.bucket_cap[0];
         sa.giant_min = (uint32_t)sa.bucket_cap[2];
-        // an array that one block alone on its SM can hold needs no deferred repair, and so no wait for one
-        if (P.N <= (uint64_t)sa.bucket_cap[2]) {
-            sa.seam_cap = std::max(sa.seam_cap, (int)align_up(P.N, 16));
+        // a small array has few ranges to repair, and a block alone on its SM sorts one faster than the
+        // multi-block sort's 14 launches or more (40,000 f32 keys: 285 us a sort, 337 through that, 328 by
+        // index lists in one block; 65,000: 300 and 359, 434 by index lists); an array that such a block
+        // holds whole needs no deferred repair, and so no wait for one
+        if (P.N <= SEAM_SMALL) {
+            sa.seam_cap = std::max(sa.seam_cap, (int)std::min<uint64_t>(align_up(P.N, 16), (uint64_t)sa.bucket_cap[2]));
             sa.seam_max = (uint32_t)sa.seam_cap;
         }
         sa.seam_max = std::min<uint32_t>(sa.seam_max, (uint32_t)sa.seam_cap);

@@ -183,6 +183,7 @@ struct SolveArgs {
 // blocks that took up to 65,536 elements, with their lists in global memory, held the whole sort up (1,024
 // arrays, 147M keys: 0.65 ms of repairs; 0.18 with 16,384, 0.07 with 8,192)
 constexpr uint64_t SEAM_CTA_MAX = 1u << 13, SEAM_CTA_LEAST = 1u << 12;
+constexpr uint64_t SEAM_SMALL = 1u << 16;  // arrays of at most this many elements: what one block can hold
 // order[]: buckets holding more than `heavy` elements first (they run longest), the rest after
 cudaError_t launch_bucket_order(const SolveArgs &a, uint32_t heavy, uint32_t *order,
                                 uint32_t *cnt /*[2], zero, as giant_cnt*/, cudaStream_t s);
