@@ -61,7 +61,7 @@ struct Workspace {
     void *host_dev = nullptr;      // device staging for the host-array entry point
     size_t host_cap = 0;
     cudaEvent_t ev[8] = {};        // stage timing
-    cudaEvent_t counted = nullptr; // the bucket counts have reached the staging area
+    cudaEvent_t arrived = nullptr; // a call's early results have reached the staging area
 };
 std::map<std::pair<int, cudaStream_t>, Workspace *> g_ws;
 
@@ -358,7 +358,7 @@ int nnsort_release(void) {
         if (w->part) cudaFree(w->part);
         if (w->pinned) cudaFreeHost(w->pinned);
         if (w->host_dev) cudaFree(w->host_dev);
-        if (w->counted) cudaEventDestroy(w->counted);
+        if (w->arrived) cudaEventDestroy(w->arrived);
         delete w;
     }
     g_ws.clear();
@@ -1002,11 +1002,11 @@ int run_sort(const std::vector<SegIn> &in, const nnsort_sort_opts *op, int dtype
         // with every launch made in any case; 1,000,000 u64 key-value pairs with giants: 861, 868)
         const size_t span = (size_t)((unsigned char *)(L.giant_cnt + 2) - (unsigned char *)L.order_cnt);
         unsigned char *hc = w->pinned + pin_cnt;
-        if (!w->counted) CK(cudaEventCreateWithFlags(&w->counted, cudaEventDisableTiming));
+        if (!w->arrived) CK(cudaEventCreateWithFlags(&w->arrived, cudaEventDisableTiming));
         CK(cudaMemcpyAsync(hc, L.order_cnt, span, cudaMemcpyDeviceToHost, s));
-        CK(cudaEventRecord(w->counted, s));
+        CK(cudaEventRecord(w->arrived, s));
         CK(launch_buckets(sa, s));
-        CK(cudaEventSynchronize(w->counted));
+        CK(cudaEventSynchronize(w->arrived));
         uint32_t nheavy = 0;
         std::memcpy(&nheavy, hc, 4);
         std::memcpy(&nbig, hc + span - 8, 4);
@@ -1710,6 +1710,7 @@ int nnsort_train_models(const void *const *d_keys, const uint64_t *ns, uint32_t 
     if (count == 0) return NNSORT_OK;
     if (count > 65535u || !dtype_ok(dtype) || !arch_ok(o.layers, o.h1, o.h2) || o.loss < 0 || o.loss > 1)
         return NNSORT_E_INVALID_ARG;
+    if (o.translate != NNSORT_TRANSLATE_ORDBITS && o.translate != NNSORT_TRANSLATE_VALUE) return NNSORT_E_INVALID_ARG;
     const PadArch pa = pad_arch(o.layers, o.h1, o.h2);
     const size_t Pp = padded_param_count(pa), P = param_count(o.layers, o.h1, o.h2);
     const int kb = key_bytes_of(dtype);
@@ -1835,7 +1836,8 @@ int nnsort_train_models(const void *const *d_keys, const uint64_t *ns, uint32_t 
     uint32_t *const G[2] = {L.grp[0], L.grp[1]};
     int fin = 0;
     if ((rc = sort_packed(w, total, kb, dtype, K, none, G, count - 1, &fin, s))) return rc;
-    CK(launch_norm_xy(L.jobs, count, max_S, kb, dtype, o.translate, L.key[fin], L.norms, s));
+    // (a model whose sample holds a NaN is refused here: its job is left without blocks, and the steps skip it)
+    CK(launch_norm_xy(L.jobs, count, max_S, kb, dtype, o.translate, L.key[fin], L.norms, L.err, s));
     TrainHyper h{};
     h.steps = (int)o.steps; h.batch = o.batch; h.loss = o.loss; h.delta = o.huber_delta;
     h.lr = o.lr; h.b1 = o.beta1; h.b2 = o.beta2; h.eps = o.adam_eps; h.c12 = L.c12;
@@ -1849,21 +1851,36 @@ int nnsort_train_models(const void *const *d_keys, const uint64_t *ns, uint32_t 
             t.x = hj[j].x; t.label = hj[j].label; t.S = S[j]; t.batch = o.batch; t.batch_seed = hj[j].bseed;
             t.loss = o.loss; t.delta = o.huber_delta;
             t.lr = o.lr; t.b1 = o.beta1; t.b2 = o.beta2; t.eps = o.adam_eps; t.mask = hj[j].mask;
+            t.refused = L.err + j;
             // every step in one cooperative launch, whose blocks meet on a count that starts at zero
             if (j) CK(cudaMemsetAsync(L.meet, 0, sizeof(unsigned int), s));
             CK(launch_train_tc64(t, o.steps, L.c12, L.meet, s));
         }
     } else {
         const uint32_t mb = *std::max_element(blocks.begin(), blocks.end());
-        for (uint32_t k = 0; k < o.steps; ++k)
+        // the samples' status arrives while the steps are launched; if every model is refused, no more are
+        if ((rc = ensure_pinned(w, count * sizeof(uint32_t), s))) return rc;
+        const uint32_t *he = reinterpret_cast<const uint32_t *>(w->pinned);
+        if (!w->arrived) CK(cudaEventCreateWithFlags(&w->arrived, cudaEventDisableTiming));
+        CK(cudaMemcpyAsync(w->pinned, L.err, count * sizeof(uint32_t), cudaMemcpyDeviceToHost, s));
+        CK(cudaEventRecord(w->arrived, s));
+        bool waiting = true;
+        for (uint32_t k = 0; k < o.steps; ++k) {
+            if (waiting) {
+                const cudaError_t q = cudaEventQuery(w->arrived);
+                if (q == cudaErrorNotReady) cudaGetLastError();  // not an error of the launches that follow
+                else CK(q);
+                waiting = q != cudaSuccess;
+                if (!waiting && std::all_of(he, he + count, [](uint32_t e) { return (e & ERR_NAN) != 0; })) break;
+            }
             CK(launch_train_step(pa, L.jobs, count, mb, h, Pp, (int)k, hc[k], hc[steps + k], s));
+        }
     }
     uint32_t te = 0;
     if (tc64) CK(cudaMemcpyAsync(&te, terr, sizeof(uint32_t), cudaMemcpyDeviceToHost, s));
     CK(cudaMemcpyAsync(host.data() + off_par, dev + off_par, back_end - off_par, cudaMemcpyDeviceToHost, s));
     CK(cudaStreamSynchronize(s));
     if (te & ERR_TIMEOUT) return NNSORT_E_TIMEOUT;
-    if (h_loss && steps) std::memcpy(h_loss, hp(L.loss), count * steps * sizeof(float));
     std::vector<float> up(P);
     for (uint32_t j = 0; j < count; ++j) {
         const float *pp = reinterpret_cast<const float *>(hp(L.params + j * Pp));
@@ -1875,6 +1892,7 @@ int nnsort_train_models(const void *const *d_keys, const uint64_t *ns, uint32_t 
         uint32_t err = 0;
         std::memcpy(&err, hp(L.err + j), 4);
         if (err & ERR_NAN) { rcs[j] = NNSORT_E_NAN_KEY; continue; }
+        if (h_loss && steps) std::memcpy(h_loss + j * steps, hp(L.loss + j * steps), steps * sizeof(float));
         rcs[j] = nnsort_model_create(&d, up.data(), &out[j]);
     }
     return NNSORT_OK;

@@ -251,6 +251,7 @@ struct TrainStepArgs {
     int loss; float delta;
     float lr, b1, b2, eps;
     const float *mask;    // nullable: +1/-1 sign a parameter must keep, 0 free
+    const uint32_t *refused;  // device word: not zero when the model's sample was refused
 };
 // One model of a training call (models of one architecture trained side by side): its sample, its
 // batch and its parameters. Sample arrays of all models are packed; `off` is the model's first entry.
@@ -260,7 +261,7 @@ struct TrainJob {
     uint64_t sseed, bseed;   // sample and mini-batch streams
     uint64_t B;              // samples per step
     float inv_n;             // 1 / B
-    uint32_t blocks;         // partial gradient rows of a step
+    uint32_t blocks;         // partial gradient rows of a step (0 on the device: the model is refused)
     float *params, *m, *v;   // padded layout
     const float *mask;       // nullable: signs to keep
     const float *x, *label;  // [S]
@@ -278,8 +279,8 @@ struct TrainHyper {
 // normalisers once sorted
 cudaError_t launch_sample_jobs(const TrainJob *jobs, uint32_t models, uint64_t max_S, int key_bytes, int dtype,
                                void *sample_keys, uint32_t *group, uint32_t *err, cudaStream_t s);
-cudaError_t launch_norm_xy(const TrainJob *jobs, uint32_t models, uint64_t max_S, int key_bytes, int dtype,
-                           int translate, const void *sorted_keys, Norm *norms, cudaStream_t s);
+cudaError_t launch_norm_xy(TrainJob *jobs, uint32_t models, uint64_t max_S, int key_bytes, int dtype, int translate,
+                           const void *sorted_keys, Norm *norms, const uint32_t *err, cudaStream_t s);
 // one Adam step of every job (per-step kernels), all steps of one-hidden-layer jobs in one launch
 // (k_train_cluster.cu)
 cudaError_t launch_train_step(const PadArch &a, const TrainJob *jobs, uint32_t models, uint32_t max_blocks,

@@ -110,7 +110,8 @@ __device__ __forceinline__ double key_value(uint64_t w, int dtype) {
     return __ull2double_rn(w);
 }
 template <typename W>
-__global__ void k_norm_xy(const TrainJob *jobs, int dtype, int translate, const W *sorted, Norm *norms) {
+__global__ void k_norm_xy(TrainJob *jobs, int dtype, int translate, const W *sorted, Norm *norms,
+                          const uint32_t *err) {
     __shared__ Norm sn;
     const TrainJob &J = jobs[blockIdx.y];
     const uint64_t S = J.S;
@@ -133,7 +134,10 @@ __global__ void k_norm_xy(const TrainJob *jobs, int dtype, int translate, const 
         q.lo_f = __double2float_rn(q.lo_val);
         q.scale_f = __double2float_rn(q.scale);
         sn = q;
-        if (blockIdx.x == 0) norms[blockIdx.y] = q;
+        if (blockIdx.x == 0) {
+            norms[blockIdx.y] = q;
+            if (err[blockIdx.y]) jobs[blockIdx.y].blocks = 0;  // a NaN key: the steps skip the model
+        }
     }
     __syncthreads();
     const Norm N = sn;
@@ -149,13 +153,13 @@ __global__ void k_norm_xy(const TrainJob *jobs, int dtype, int translate, const 
     }
 }
 
-cudaError_t launch_norm_xy(const TrainJob *jobs, uint32_t models, uint64_t max_S, int key_bytes, int dtype,
-                           int translate, const void *sorted_keys, Norm *norms, cudaStream_t s) {
+cudaError_t launch_norm_xy(TrainJob *jobs, uint32_t models, uint64_t max_S, int key_bytes, int dtype, int translate,
+                           const void *sorted_keys, Norm *norms, const uint32_t *err, cudaStream_t s) {
     const dim3 grid((unsigned)std::min<uint64_t>((max_S + 255) / 256, 4096), models);
     if (key_bytes == 4)
-        k_norm_xy<uint32_t><<<grid, 256, 0, s>>>(jobs, dtype, translate, reinterpret_cast<const uint32_t *>(sorted_keys), norms);
+        k_norm_xy<uint32_t><<<grid, 256, 0, s>>>(jobs, dtype, translate, reinterpret_cast<const uint32_t *>(sorted_keys), norms, err);
     else
-        k_norm_xy<uint64_t><<<grid, 256, 0, s>>>(jobs, dtype, translate, reinterpret_cast<const uint64_t *>(sorted_keys), norms);
+        k_norm_xy<uint64_t><<<grid, 256, 0, s>>>(jobs, dtype, translate, reinterpret_cast<const uint64_t *>(sorted_keys), norms, err);
     return nns_launched(cudaGetLastError());
 }
 
@@ -693,6 +697,7 @@ __global__ void __launch_bounds__(RD_WARPS * 32) k_reduce(ReduceArgs r) {
     const size_t nb = (r.P + 31) / 32;
     if (r.jobs) {
         const TrainJob &J = r.jobs[blockIdx.y];
+        if (J.blocks == 0) return;  // refused
         r.partials = J.partials; r.blocks = (int)J.blocks; r.loss_partials = J.loss_partials;
         r.loss_out = J.loss_out + r.step; r.loss_scale = J.inv_n;
         r.params = J.params; r.m = J.m; r.v = J.v; r.mask = J.mask;

@@ -43,6 +43,7 @@ __global__ void __launch_bounds__(TC1_THREADS) k_train_cluster(const TrainJob *j
     const uint32_t c = cl.block_rank();
     const int tid = threadIdx.x;
     const TrainJob J = jobs[blockIdx.y];
+    if (J.blocks == 0) return;  // refused (every block of the cluster)
     // the rows of the per-step kernel: `nrow` rows of `per` samples
     const uint32_t B = (uint32_t)J.B, nrow = J.blocks, per = (B + nrow - 1) / nrow;
     const uint32_t rows = c < nrow ? (nrow - c + TC1_CTAS - 1) / TC1_CTAS : 0u;

@@ -599,6 +599,7 @@ struct TrainTcArgs {
     float *loss_out;           // [steps]
     float loss_scale, lr, b1, b2, eps;
     int steps;
+    const uint32_t *refused;   // not zero: nothing to train
     unsigned int *count;       // arrivals at the grid meetings (zero before the launch)
 };
 constexpr int NGRP = (GP + 31) / 32;  // parameter groups
@@ -687,6 +688,7 @@ __device__ __forceinline__ void reduce_adam(const TrainTcArgs &a, int step, floa
 }
 
 __global__ void __launch_bounds__(GTHREADS, 1) k_train_tc64(TrainTcArgs a) {
+    if (*a.refused) return;  // (written before the launch: the same for every block)
     extern __shared__ __align__(1024) unsigned char sm[];
     __shared__ __align__(8) unsigned long long bars[2 * GNG];
     __shared__ uint32_t tmem_slot;
@@ -751,7 +753,7 @@ cudaError_t launch_train_tc64(const TrainStepArgs &t, uint32_t steps, const floa
     a.g.loss_partials = t.loss_partials; a.g.gx = nullptr;
     a.params = t.params; a.m = t.m; a.v = t.v; a.mask = t.mask; a.c12 = c12; a.loss_out = t.loss_out;
     a.loss_scale = 1.0f / (float)B; a.lr = t.lr; a.b1 = t.b1; a.b2 = t.b2; a.eps = t.eps;
-    a.steps = (int)steps; a.count = count;
+    a.steps = (int)steps; a.count = count; a.refused = t.refused;
     void *args[] = {&a};
     e = cudaLaunchCooperativeKernel((const void *)k_train_tc64, dim3((unsigned)blocks), dim3(GTHREADS), args,
                                     SMEM_BYTES, s);
