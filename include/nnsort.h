@@ -143,7 +143,8 @@ typedef struct {
                                  own (a row trace, or bucket_log2 of 13 and 14) */
 } nnsort_sort_opts;
 
-/* Per-array statistics (Sec. "Model Analysis", Eq. (sorting rate), Eq. (ratio)). */
+/* Per-array statistics (Sec. "Model Analysis", Eq. (sorting rate), Eq. (ratio)). A sort refused for its keys or
+ * positions reports what the iterations counted (a bad position counts as 0), and no polish or repairs. */
 typedef struct {
     uint32_t rounds;                           /* t: completed iterations */
     uint32_t eps;

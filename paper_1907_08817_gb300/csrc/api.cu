@@ -1083,6 +1083,28 @@ int run_sort(const std::vector<SegIn> &in, const nnsort_sort_opts *op, int dtype
     CK(cudaStreamSynchronize(s));
     uint32_t err = 0;
     std::memcpy(&err, hp + err_off, 4);
+    if (st && err && onepass) {
+        // a refused call's statistics: the conflict arrays' sizes and t, but no out-of-order counts or
+        // repairs, as the two-kernel form counts them (the one-pass kernels leave the call at the error)
+        SolveArgs sr = sa;
+        sr.rk = nullptr;
+        sr.order = nullptr;
+        sr.giant = nullptr;
+        CK(cudaMemsetAsync(L.stats, 0, sizeof(SegStats) * nseg, s));
+        if (P.N > POLISH_BIG) {
+            CK(cudaMemsetAsync(L.order_cnt, 0, (size_t)((unsigned char *)(L.giant_cnt + 4) - (unsigned char *)L.order_cnt), s));
+            sr.giant = L.giant;
+            sr.giant_min = POLISH_BIG;
+            sr.list_refused = 1;
+            gr.cap = (uint32_t)(P.N / POLISH_BIG + 1);
+            CK(launch_bucket_order(sr, POLISH_BIG, L.order, L.order_cnt, s));
+        }
+        CK(launch_rounds(sr, s));
+        if (sr.giant) CK(launch_giant_rounds(sr, gr, o.eps, sms, s));
+        CK(launch_finalize(sr, s));
+        CK(cudaMemcpyAsync(hp, L.stats, sizeof(SegStats) * nseg, cudaMemcpyDeviceToHost, s));
+        CK(cudaStreamSynchronize(s));
+    }
     if (st) {
         for (int i = 0; i < nseg; ++i) {
             SegStats d;

@@ -173,6 +173,7 @@ struct SolveArgs {
     int seam_cap;             // elements that a block of the on-chip seam repair holds
     const uint32_t *heavy_cnt;  // with rk: the order's first *heavy_cnt buckets exceed bucket_cap[0]
     uint32_t giant_min;       // buckets above this many elements are listed in giant
+    int list_refused;         // 1: also after an error (their rounds only; nothing is written back)
     const uint32_t *order;    // [NB] nullable: block i of k_rounds / k_polish takes bucket order[i]
     BigRange *giant;          // nullable: k_bucket_order lists buckets above POLISH_BIG here and
     uint32_t *giant_cnt;      //   k_rounds leaves them to launch_giant_rounds

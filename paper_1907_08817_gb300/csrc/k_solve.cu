@@ -84,7 +84,7 @@ __global__ void k_bucket_order(SolveArgs a, uint32_t heavy, uint32_t *order, uin
     if (nbk > heavy) order[atomicAdd(&cnt[0], 1u)] = b;
     else order[a.NB - 1 - atomicAdd(&cnt[1], 1u)] = b;
     // after an error (NaN keys, bad positions) no bucket is listed: the listed ones are written back
-    if (a.giant && nbk > a.giant_min && !*a.err) {
+    if (a.giant && nbk > a.giant_min && (a.list_refused || !*a.err)) {
         BigRange r;
         r.lo = a.bstart[b]; r.hi = a.bstart[b + 1];
         r.seg = (uint32_t)seg_of_bucket(a.segs, a.nseg, b); r.off = 0; r.b = b; r.pad = 0;
