@@ -1691,8 +1691,8 @@ __global__ void __launch_bounds__(T, TIER == 0 ? 1024 / T : TIER == 1 ? 2 : 1) k
 // by one block per bucket from the claim table, right after the round's claims.
 constexpr int GT = 256, GI = 16;  // threads of a grid-wide block, elements per lane and chunk
 
-// packed offsets of the listed buckets (one block)
-__global__ void __launch_bounds__(1024) k_giant_offsets(GiantRounds g) {
+// packed offsets of the listed buckets (one block); their count among the oversized ones
+__global__ void __launch_bounds__(1024) k_giant_offsets(SolveArgs a, GiantRounds g) {
     __shared__ uint32_t scratch[33];
     const uint32_t n = g.count[0];
     uint32_t base = 0;
@@ -1701,7 +1701,10 @@ __global__ void __launch_bounds__(1024) k_giant_offsets(GiantRounds g) {
         const uint32_t len = j < n ? (uint32_t)(g.list[j].hi - g.list[j].lo) : 0u;
         uint32_t tot;
         const uint32_t ex = block_excl_sum(len, scratch, &tot);
-        if (j < n) g.list[j].off = base + ex;
+        if (j < n) {
+            g.list[j].off = base + ex;
+            if (len > (uint32_t)a.polish_cap) atomicAdd(&a.stats[g.list[j].seg].oversized, 1u);
+        }
         base += tot;
     }
 }
@@ -1846,7 +1849,6 @@ __global__ void __launch_bounds__(SOLVE_THREADS) k_giant_runs(SolveArgs a, Giant
             a.bmax[(size_t)R.b * MAXR + r] = o;
         }
         if (tid == 0) {
-            if (r == 0 && nbk > (uint32_t)a.polish_cap) atomicAdd(&a.stats[R.seg].oversized, 1u);
             if (left) atomicAdd(&a.stats[R.seg].count_ge[r + 1], (unsigned long long)left);
             if (out) atomicAdd(&a.stats[R.seg].ooo[r], (unsigned long long)out);
             a.rend[(size_t)R.b * MAXR + r] = roff + in;
@@ -1865,7 +1867,7 @@ static cudaError_t giant_runs_go(const SolveArgs &a, const GiantRounds &g, int r
 cudaError_t launch_giant_buckets(const SolveArgs &a, const GiantRounds &g, int eps, int sms, cudaStream_t s) {
     const unsigned grid = (unsigned)sms * 4, rgrid = std::min<unsigned>(g.cap, 2u * (unsigned)sms);
     cudaError_t e;
-    k_giant_offsets<<<1, 1024, 0, s>>>(g);
+    k_giant_offsets<<<1, 1024, 0, s>>>(a, g);
     if ((e = nns_launched(cudaGetLastError())) != cudaSuccess) return e;
     k_giant_clear<<<grid, GT, 0, s>>>(a, g, eps);
     if ((e = nns_launched(cudaGetLastError())) != cudaSuccess) return e;

@@ -79,3 +79,16 @@ def test_crowded_buckets(kind, want, dtype, wlog, threads):
     order, _, ost, _ = orc.nnsort(keys, slots, L, 3, 0, None)
     np.testing.assert_array_equal(bits(from_dev(dk, keys)), bits(order))
     assert stats_core(st) == stats_core(ost)
+
+
+@pytest.mark.parametrize("eps", [0, 1, 3])
+@pytest.mark.parametrize("n,traced", [(5_000, False), (40_000, False), (140_000, False), (140_000, True)])
+def test_oversized_buckets_are_counted_without_rounds(eps, n, traced):
+    """Every key in one bucket, above the polish's capacity from 5,000 u64 keys on, whichever form sorts it."""
+    keys = np.random.RandomState(n).permutation(n).astype(np.uint64)
+    dk, kt = to_dev(keys)
+    ds = torch.zeros(n, dtype=torch.int32, device="cuda")
+    r = nns.sort(dk, None, None, eps=eps, tau=0, slots=ds, key_type=kt, bucket_log2=12, fate=traced)
+    st = r[0] if traced else r
+    assert st["oversized_buckets"] == 1
+    np.testing.assert_array_equal(from_dev(dk, keys), np.sort(keys))
