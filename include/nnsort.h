@@ -309,7 +309,9 @@ int nnsort_radix_sort(void *d_keys, int32_t *d_payload, uint64_t n, int32_t dtyp
  * Per batch a worker copies the requests in, trains each request's model on the device
  * (nnsort_train with `train` options and a per-request seed), sorts all of them with one
  * nnsort_sort_batch call (`sort` options), and copies the results back into the caller's host
- * arrays. Latency is measured from submit to the result being in host memory. The paper has no
+ * arrays. A batch's models are trained side by side, and each request is charged its own against the
+ * budget (one that fits without is admitted by itself). Beside the budget the library's pool keeps up to
+ * 256 MB of freed memory per device until nnsort_release. Latency is measured from submit to the result being in host memory. The paper has no
  * serving layer; this is the batched, served form of its method. */
 typedef struct {
     size_t hbm_budget;          /* bytes of device memory admitted requests may hold */

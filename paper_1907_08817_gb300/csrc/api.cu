@@ -1726,6 +1726,15 @@ static std::vector<float> monotone_signs(const nnsort_train_opts &o, std::vector
     return sg;
 }
 
+size_t nnsort_train_model_bytes(const nnsort_train_opts &o) {
+    if (!arch_ok(o.layers, o.h1, o.h2)) return 0;
+    const PadArch pa = pad_arch(o.layers, o.h1, o.h2);
+    const size_t Pp = padded_param_count(pa);
+    const uint64_t B = o.batch ? o.batch : std::max<uint64_t>(1, o.sample_n);
+    const size_t rows = train_cluster_ok(pa, B) ? 0 : (size_t)train_grad_blocks(pa, B);
+    return ((size_t)(o.monotone ? 4 : 3) * Pp + rows * (Pp + 1) + o.steps) * sizeof(float) + 4096;
+}
+
 int nnsort_train_models(const void *const *d_keys, const uint64_t *ns, uint32_t count, int32_t dtype,
                         const nnsort_train_opts &o, const uint64_t *S, const uint64_t *seeds,
                         nnsort_model **out, int *rcs, float *h_loss, cudaStream_t s) {
@@ -1756,11 +1765,13 @@ int nnsort_train_models(const void *const *d_keys, const uint64_t *ns, uint32_t 
     if ((rc = ensure_part(w, total, s))) return rc;
     // one device block: tables and parameters (uploaded together), then what the kernels make; the
     // parameters, normalisers, losses and the error word lie together and come back in one copy
+    // (the rows of partial gradients: each model's own, or one set for all where their launches follow
+    // one another)
     std::vector<uint32_t> blocks(count);
     size_t rows = 0;
     for (uint32_t j = 0; j < count; ++j) {
         blocks[j] = (uint32_t)train_grad_blocks(pa, o.batch ? o.batch : S[j]);
-        rows += blocks[j];
+        rows = tc64 ? std::max<size_t>(rows, blocks[j]) : rows + blocks[j];
     }
     const size_t steps = o.steps;
     Carve c;
@@ -1846,7 +1857,7 @@ int nnsort_train_models(const void *const *d_keys, const uint64_t *ns, uint32_t 
         q.loss_out = L.loss + j * steps;
         hj[j] = q;
         off += S[j];
-        row += blocks[j];
+        if (!tc64) row += blocks[j];
     }
     CK(cudaMemcpyAsync(dev, host.data(), up_end, cudaMemcpyHostToDevice, s));
     CK(cudaMemsetAsync(L.err, 0, (size_t)((unsigned char *)(L.meet + 1) - (unsigned char *)L.err), s));

@@ -370,6 +370,9 @@ int nnsort_train_models(const void *const *d_keys, const uint64_t *ns, uint32_t 
                         const nnsort_train_opts &o, const uint64_t *S, const uint64_t *seeds,
                         struct nnsort_model **out, int *rc, float *h_loss, cudaStream_t s);
 
+// Device bytes of one of its models beside the sample: parameters, moments, partial gradients, losses.
+size_t nnsort_train_model_bytes(const nnsort_train_opts &o);
+
 // The model handle behind the opaque nnsort_model of the C ABI: one definition for every
 // translation unit that reads it.
 struct nnsort_model {

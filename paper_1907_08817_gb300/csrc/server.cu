@@ -47,6 +47,7 @@ struct nnsort_server {
     std::deque<uint64_t> waiting;  // submitted, waiting for budget (arrival order)
     std::deque<uint64_t> ready;    // admitted, not yet in a batch
     std::map<uint64_t, Req> reqs;
+    size_t model_bytes = 0;        // of a request's model while its batch trains side by side
     size_t used = 0;
     uint64_t next_id = 1;
     bool stop = false;
@@ -247,6 +248,7 @@ int nnsort_server_create(const nnsort_server_opts *o, nnsort_server **out) {
     if (!s) return NNSORT_E_OOM;
     s->o = opts;
     cudaGetDevice(&s->device);
+    s->model_bytes = nnsort_train_model_bytes(opts.train);
     for (int i = 0; i < opts.workers; ++i) s->workers.emplace_back(worker_main, s);
     *out = s;
     return NNSORT_OK;
@@ -264,6 +266,8 @@ int nnsort_server_submit(nnsort_server *s, void *h_keys, int32_t *h_payload, uin
     r.seed = seed;
     r.bytes = request_bytes(s, n, dtype, h_payload != nullptr);
     if (r.bytes > s->o.hbm_budget) return NNSORT_E_BUDGET;
+    // beside others a request's model needs room of its own; alone it is served within the budget's slack
+    r.bytes = std::min(r.bytes + s->model_bytes, s->o.hbm_budget);
     r.t_submit = now_s();
     std::lock_guard<std::mutex> lk(s->mu);
     if (s->stop) return NNSORT_E_STATE;
