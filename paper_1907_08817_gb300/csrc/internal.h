@@ -151,11 +151,11 @@ struct SolveArgs {
     uint32_t *pay_scratch, *row_scratch;
     uint32_t *err;
     int key_bytes, dtype;
-    int polish_cap;           // elements a bucket may hold on chip
+    int polish_cap;           // elements that a bucket of the two-kernel form may hold on chip
     size_t polish_smem;
     int allow_defer;          // 1: seam repairs above seam_max are left to the host's
                               //    multi-block sort (never when rows are carried)
-    uint32_t seam_max;
+    uint32_t seam_max;        // elements of the largest repair that one block performs
     SeamRange *ranges;        // [max_ranges]: block-sized repairs from the front, large from the back
     uint32_t max_ranges;      // >= NB + nseg
     uint32_t *seam_cnt;       // [4], zero before the seam: block-sized ranges, large ranges, next range to repair
@@ -174,9 +174,10 @@ struct SolveArgs {
     const uint32_t *heavy_cnt;  // with rk: the order's first *heavy_cnt buckets exceed bucket_cap[0]
     uint32_t giant_min;       // buckets above this many elements are listed in giant
     int list_refused;         // 1: also after an error (their rounds only; nothing is written back)
-    const uint32_t *order;    // [NB] nullable: block i of k_rounds / k_polish takes bucket order[i]
-    BigRange *giant;          // nullable: k_bucket_order lists buckets above POLISH_BIG here and
-    uint32_t *giant_cnt;      //   k_rounds leaves them to launch_giant_rounds
+    const uint32_t *order;    // [NB] nullable: block i of k_bucket / k_rounds / k_polish takes bucket order[i]
+    BigRange *giant;          // nullable: k_bucket_order lists buckets above giant_min here, in any order;
+    uint32_t *giant_cnt;      //   [2] their count and their elements. k_bucket and k_rounds leave them to
+                              //   launch_giant_buckets and launch_giant_rounds
     BigRange *big;            // nullable: k_polish lists buckets above POLISH_BIG here (and only
     uint32_t *big_cnt;        //   splits their runs); their sort is left to the host's multi-block sort
 };
@@ -188,11 +189,11 @@ constexpr uint64_t SEAM_SMALL = 1u << 16;  // arrays of at most this many elemen
 // order[]: buckets holding more than `heavy` elements first (they run longest), the rest after
 cudaError_t launch_bucket_order(const SolveArgs &a, uint32_t heavy, uint32_t *order,
                                 uint32_t *cnt /*[2], zero, as giant_cnt*/, cudaStream_t s);
-// buckets above POLISH_BIG elements run their rounds on the whole GPU (global claim tables); the
+// buckets above giant_min elements run their rounds on the whole GPU (global claim tables); the
 // list, its count and the per-(bucket, round) statistics live in GiantRounds
 struct GiantRounds {
-    BigRange *list;               // [N / POLISH_BIG + 1]
-    uint32_t *count;              // [1]
+    BigRange *list;               // [N / giant_min + 1]
+    uint32_t *count;              // [2] entries, their elements
     unsigned long long *table;    // [list entries x W] round-tagged claims
     unsigned int *cnt;            // [entries x MAXR] elements stored per round
     unsigned long long *kmax;     // [entries x MAXR] largest order image stored per round

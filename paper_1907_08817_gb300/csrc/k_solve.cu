@@ -74,9 +74,10 @@ __device__ __forceinline__ KMax warp_max_kmax(KMax v) {
 }
 
 // ---------------------------------------------------------------------------------------------
-// Bucket order for the per-bucket kernels: blocks are dispatched roughly in index order, so heavy
-// buckets listed first start first and run alongside the many light ones instead of forming a
-// tail. Heavy buckets fill order[] from the front, light ones from the back.
+// Bucket order for the per-bucket kernels: heavy buckets fill order[] from the front, light ones from the
+// back. In the two-kernel form blocks are dispatched roughly in index order, so the heavy ones start first
+// and run alongside the many light ones instead of forming a tail. The one-pass form's light launch passes
+// the heavy ones by; their launches follow it, each as long as its fullest bucket (59 us at 2^28 keys).
 __global__ void k_bucket_order(SolveArgs a, uint32_t heavy, uint32_t *order, uint32_t *cnt) {
     const uint32_t b = blockIdx.x * blockDim.x + threadIdx.x;
     if (b >= a.NB) return;
@@ -146,7 +147,7 @@ cudaError_t launch_bounds_order_small(const SolveArgs &a, uint32_t *bstart, uint
 }
 
 // ---------------------------------------------------------------------------------------------
-// Rounds of buckets above POLISH_BIG elements, spread over the whole GPU: the same first-arrival
+// Two-kernel form: rounds of buckets above POLISH_BIG elements, spread over the whole GPU: the same first-arrival
 // rule with the claims in a global table per bucket. A claim in round r stores (MAXR - r) << 32 | i,
 // so one atomicMin both picks the lowest row among round-r claimants and overrides the entries of
 // earlier rounds; the table is cleared once. Every kernel walks the listed buckets in turn, each
@@ -1171,7 +1172,7 @@ __global__ void __launch_bounds__(SOLVE_THREADS) k_polish(SolveArgs a) {
 
 // ---------------------------------------------------------------------------------------------
 // One-pass buckets: the rounds, the run split and the sorted output of a bucket of at most
-// polish_cap elements in one block, which reads the bucket once (k_rounds and k_polish read it twice and
+// bucket_cap[2] elements in one block, which reads the bucket once (k_rounds and k_polish read it twice and
 // pass every element's round through memory). The one thing that needs other buckets is the carry of
 // the out-of-order split, the largest element that earlier buckets stored in o_r; but an element x of
 // o_r is out of order exactly when it is below the bucket's own earlier elements of o_r or below the
@@ -1179,15 +1180,15 @@ __global__ void __launch_bounds__(SOLVE_THREADS) k_polish(SolveArgs a) {
 // memory, and k_carried counts those below the carry by binary search.
 //
 // Sort: the order of the composite key (key - kmin) * 2^ib + index is the stable order. Each element's
-// top 32 composite bits are its word; words drop into 4,096 bins by their top 12 bits (shared-memory
-// atomics), and each thread puts the few elements of its eight bins in order by insertion. Words that
+// top 32 composite bits are its word; in a block of T threads words drop into 8 T bins by their top bits
+// (shared-memory atomics), and each thread puts the few elements of its eight bins in order by insertion. Words that
 // cannot hold the whole composite keep the index beside them and settle equal words
 // by key and index. When a bin holds more than BIN_MAX elements, or a thread's bins too many together,
 // sort_crowded cuts them finer, and the stable radix sort takes what that cannot.
 //
-// Bound by instruction issue and the latency of its barrier-separated phases. Buckets too large for two
-// blocks per SM take a second launch with one block per SM; the rest (launch_giant_buckets) run on the
-// whole GPU. Against k_rounds, k_polish and their one-block global-memory path: 2^28 f32 keys 3.6 ms
+// Bound by instruction issue and the latency of its barrier-separated phases. Buckets too large for the
+// blocks of their width take launches of their own (launch_heavy_buckets), two 512-thread blocks per SM and
+// then one; the rest (launch_giant_buckets) run on the whole GPU. Against k_rounds, k_polish and their one-block global-memory path: 2^28 f32 keys 3.6 ms
 // (5.4 ms), 64M u64 key-value 1.9 ms (3.6 ms), 50M u64 keys in three rounds 1.6 ms (3.0 ms).
 template <typename W> struct OPair;  // (order image, tie-break); all zero is the least pair and stands for none
 template <> struct OPair<uint32_t> {
@@ -2569,8 +2570,8 @@ __global__ void __launch_bounds__(SOLVE_THREADS, 2) k_seam_sort(SolveArgs a) {
     }
 }
 
-// Buckets above POLISH_BIG: k_big_pack copies their partitioned elements (br sorted by position,
-// br[j].off = packed offset) into the packed buffers with the bucket's list index j, or, with
+// Giant buckets (two-kernel form: those above POLISH_BIG): k_big_pack copies their partitioned elements (br
+// in any order of buckets, br[j].off = packed offset, ascending) into the packed buffers with the bucket's list index j, or, with
 // unpack = 1, the sorted packed elements to the bucket's output positions; k_big_bounds records
 // each such bucket's first and last output element for the seam.
 // Both pack kernels walk the packed elements in chunks of 256 per warp: one binary search finds the

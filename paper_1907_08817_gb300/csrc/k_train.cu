@@ -697,7 +697,6 @@ __global__ void __launch_bounds__(RD_WARPS * 32) k_reduce(ReduceArgs r) {
     const size_t nb = (r.P + 31) / 32;
     if (r.jobs) {
         const TrainJob &J = r.jobs[blockIdx.y];
-        if (J.blocks == 0) return;  // refused
         r.partials = J.partials; r.blocks = (int)J.blocks; r.loss_partials = J.loss_partials;
         r.loss_out = J.loss_out + r.step; r.loss_scale = J.inv_n;
         r.params = J.params; r.m = J.m; r.v = J.v; r.mask = J.mask;

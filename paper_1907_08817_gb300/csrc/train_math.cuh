@@ -1,5 +1,6 @@
-// train_math.cuh -- the scalar steps that every training kernel shares (Sec. "Training", Eq. (loss);
-// Adam per Kingma & Ba), stated once so that each kernel rounds them the same way.
+// train_math.cuh -- the scalar steps that the training kernels on the CUDA cores share (Sec. "Training",
+// Eq. (loss); Adam per Kingma & Ba), stated once so that each of them rounds them the same way. The kernels
+// of width 64 (k_train_tc.cu) state the same steps themselves, with the contractions the compiler chooses.
 #pragma once
 #include "common.cuh"
 
@@ -18,7 +19,8 @@ __device__ __forceinline__ void loss_term(float r, int loss, float delta, float 
     gy *= inv_n;
 }
 
-// one Adam step of one parameter, its contractions written out so that every kernel makes the same ones; c1, c2: bias corrections; mask: +1/-1 the sign to keep, 0 free
+// one Adam step of one parameter, its contractions written out so that every kernel that includes this makes
+// the same ones; c1, c2: bias corrections; mask: +1/-1 the sign to keep, 0 free
 __device__ __forceinline__ float adam_step(float p, float g, float &ms, float &vs, float lr, float b1, float b2,
                                            float eps, float c1, float c2, float mask) {
     const float m = __fmaf_rn(1.0f - b1, g, __fmul_rn(b1, ms));
