@@ -13,6 +13,14 @@ namespace nns {
 // counts kernels launched by the library (nnsort_launch_count)
 void note_launch(int kernels);
 
+// Allows a kernel `most` bytes of dynamic shared memory: the most that any launch of it takes, not this
+// launch's own share. The attribute is the function's, so a call that set what it needs itself could lower
+// it between another thread's setting and launch, which then fails.
+template <typename K> inline cudaError_t allow_smem(K kfn, size_t most) {
+    return cudaFuncSetAttribute(kfn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most);
+}
+constexpr size_t BLOCK_SMEM = 227 * 1024;  // of one block
+
 struct Seg;
 struct Norm;
 struct SegStats;

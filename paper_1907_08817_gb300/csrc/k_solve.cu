@@ -2699,7 +2699,7 @@ cudaError_t launch_seam_pack(const SeamRange *rg, uint32_t nr, const Seg *segs, 
 // ---------------------------------------------------------------------------------------------
 template <typename W> static cudaError_t rounds_go(const SolveArgs &a, cudaStream_t s) {
     const size_t smem = rounds_smem(a.wlog);
-    cudaError_t e = cudaFuncSetAttribute(k_rounds<W>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = allow_smem(k_rounds<W>, std::max(rounds_smem(12), rounds_smem(14)));
     if (e != cudaSuccess) return e;
     k_rounds<W><<<a.NB, RT, smem, s>>>(a);
     return nns_launched(cudaGetLastError());
@@ -2734,7 +2734,7 @@ template <typename W> static cudaError_t polish_go(const SolveArgs &a, cudaStrea
     const size_t smem = std::max(a.polish_smem, sizeof(PolishSmem) + 16 + ((size_t)4 << a.wlog));
     // the key's order image with its type fixed at compile time (IEEE float or unsigned)
     auto kfn = (a.dtype == NNSORT_F32 || a.dtype == NNSORT_F64) ? k_polish<W, true> : k_polish<W, false>;
-    cudaError_t e = cudaFuncSetAttribute(kfn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = allow_smem(kfn, BLOCK_SMEM);
     if (e != cudaSuccess) return e;
     kfn<<<a.NB, SOLVE_THREADS, smem, s>>>(a);
     return nns_launched(cudaGetLastError());
@@ -2769,12 +2769,12 @@ template <typename W> static cudaError_t seam_go(const SolveArgs &a, int sms, cu
         if ((e = nns_launched(cudaGetLastError())) != cudaSuccess) return e;
     }
     if (a.rk) {  // one-pass buckets
-        const size_t smem = bucket_fixed<W, SOLVE_THREADS>() + (size_t)a.seam_cap * bucket_per<W>(a.pay != nullptr);
+        const size_t per = bucket_per<W>(a.pay != nullptr), fixed = bucket_fixed<W, SOLVE_THREADS>();
+        const size_t smem = fixed + (size_t)a.seam_cap * per;
         const bool fl = a.dtype == NNSORT_F32 || a.dtype == NNSORT_F64;
         auto kfn = a.pay ? (fl ? k_seam_sort<W, true, true> : k_seam_sort<W, false, true>)
                          : (fl ? k_seam_sort<W, true, false> : k_seam_sort<W, false, false>);
-        if ((e = cudaFuncSetAttribute(kfn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess)
-            return e;
+        if ((e = allow_smem(kfn, fixed + (size_t)a.bucket_cap[2] * per)) != cudaSuccess) return e;
         kfn<<<std::min<unsigned>(a.max_ranges, 2u * (unsigned)sms), SOLVE_THREADS, smem, s>>>(a);
         return nns_launched(cudaGetLastError());
     }

@@ -330,16 +330,17 @@ __global__ void __launch_bounds__(T) k_train_block(TrainBlockArgs a) {
 
 template <typename W, int T>
 static cudaError_t tb_go(const TrainBlockArgs &a, int H, uint32_t blocks, cudaStream_t s) {
-    auto go = [&](auto kfn, size_t smem) -> cudaError_t {
-        cudaError_t e = cudaFuncSetAttribute(kfn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    constexpr uint32_t most = T == 128 ? 1024 : T == 512 ? 4096 : TB_MAX_S;  // the class's largest sample
+    auto go = [&](auto kfn, size_t smem, size_t top) -> cudaError_t {
+        cudaError_t e = allow_smem(kfn, top);
         if (e != cudaSuccess) return e;
         kfn<<<blocks, T, smem, s>>>(a);
         return nns_launched(cudaGetLastError());
     };
     switch (H) {
-    case 8: return go(k_train_block<W, 8, T>, tb_smem<8>(a.cap));
-    case 16: return go(k_train_block<W, 16, T>, tb_smem<16>(a.cap));
-    case 32: return go(k_train_block<W, 32, T>, tb_smem<32>(a.cap));
+    case 8: return go(k_train_block<W, 8, T>, tb_smem<8>(a.cap), tb_smem<8>(most));
+    case 16: return go(k_train_block<W, 16, T>, tb_smem<16>(a.cap), tb_smem<16>(most));
+    case 32: return go(k_train_block<W, 32, T>, tb_smem<32>(a.cap), tb_smem<32>(most));
     }
     return cudaErrorInvalidValue;
 }

@@ -155,11 +155,14 @@ template <int H>
 cudaError_t go(const TrainJob *jobs, uint32_t models, const TrainHyper &hp, uint64_t max_batch, bool probe,
                cudaStream_t s) {
     static_assert(3 * H + 2 <= TC1_THREADS, "a thread per sum");
-    const uint64_t nrow = (max_batch + TC1_ROW - 1) / TC1_ROW;
-    const uint32_t rcap = (uint32_t)((nrow + TC1_CTAS - 1) / TC1_CTAS), cap = rcap * TC1_ROW;
-    const size_t smem = (size_t)cap * 20 + (size_t)rcap * (3 * H + 2) * 4;
+    auto rows_of = [](uint64_t batch) {  // of a block
+        return (uint32_t)(((batch + TC1_ROW - 1) / TC1_ROW + TC1_CTAS - 1) / TC1_CTAS);
+    };
+    auto smem_of = [](uint32_t rows) { return (size_t)rows * TC1_ROW * 20 + (size_t)rows * (3 * H + 2) * 4; };
+    const uint32_t rcap = rows_of(max_batch), cap = rcap * TC1_ROW;
+    const size_t smem = smem_of(rcap);
     auto kfn = k_train_cluster<H>;
-    cudaError_t e = cudaFuncSetAttribute(kfn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = allow_smem(kfn, smem_of(rows_of(TC1_MAX_BATCH)));
     if (e == cudaSuccess) e = cudaFuncSetAttribute(kfn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
     if (e != cudaSuccess) return e;
     cudaLaunchConfig_t cfg{};

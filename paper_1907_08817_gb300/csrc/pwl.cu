@@ -316,8 +316,7 @@ cudaError_t launch_predict_pwl(const PredictArgs &p, int sms, cudaStream_t s) {
     if (grid == 0) return cudaSuccess;
     auto k4 = k_predict_pwl<uint32_t>;
     auto k8 = k_predict_pwl<uint64_t>;
-    cudaError_t e = cudaFuncSetAttribute(p.key_bytes == 4 ? k4 : k8,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = allow_smem(p.key_bytes == 4 ? k4 : k8, (size_t)pwl_max_segments(2, 64, 64) * 24);
     if (e != cudaSuccess) return e;
     if (p.key_bytes == 4) k4<<<grid, PRED_THREADS, smem, s>>>(p);
     else k8<<<grid, PRED_THREADS, smem, s>>>(p);
