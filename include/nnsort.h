@@ -230,7 +230,7 @@ int nnsort_sample_labels(const void *d_keys, uint64_t n, int32_t dtype, uint64_t
                          uint32_t *d_rows, cudaStream_t stream);
 /* Trains f on the device: sample + labels as above, parameters initialised from the seed, then
  * `steps` Adam steps on the mean loss, with the gradient from the library's backward kernels.
- * h_loss (nullable, `steps` floats) receives the loss before each step. Synchronous. */
+ * h_loss (nullable, `steps` floats) receives the loss before each step, if the training succeeds. Synchronous. */
 int nnsort_train(const void *d_keys, uint64_t n, int32_t dtype, const nnsort_train_opts *o,
                  nnsort_model **out, float *h_loss, cudaStream_t stream);
 /* Trains `count` models at once, model j on the device array d_keys[j] (host array of device
