@@ -586,6 +586,9 @@ __device__ Idx *cta_radix_sort(Idx *src, Idx *dst, uint32_t cnt, int keybits, Ke
     const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
     const unsigned lt = (1u << lane) - 1u;
     const int npass = keybits / 8;
+    // a call just before may still be reading the tables: its last digits, when they are constant, pass without
+    // a barrier, and a thread that then found them cleared would take those passes alone
+    __syncthreads();
     for (int i = tid; i < npass * 256; i += T) hist[i] = 0;
     for (int i = tid; i < (T / 32) * 256; i += T) wcnt[i] = 0;
     static_assert(T >= 256 || T == 128, "a thread per digit, or two");

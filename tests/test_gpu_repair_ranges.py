@@ -47,3 +47,26 @@ def test_ranges_around_a_blocks_capacity(dtype):
         few = [_sort(dtype, n, m) for m in (cap - 1, cap)]
         many = [_sort(dtype, n, m) for m in (cap + 1, cap + 1_000)]
         assert max(few) < min(many)
+
+
+@pytest.mark.parametrize("dtype", [np.float32, np.uint64])
+def test_many_ranges_with_rows(dtype):
+    """Hundreds of repairs with rows carried, each a sort by row and then by key over the same tables: the
+    output, with its payload and fates, is the stable sort run after run."""
+    n, rs = 3_000_001, np.random.RandomState(77)
+    rank = rs.permutation(n)
+    keys = (rank // 2).astype(dtype)  # pairs of equal keys, which the rows order
+    lim, _, _ = orc.nm_split(n)
+    slots = (rank * 5 // 4 + rs.randint(-1, 2, n)).astype(np.int64)
+    idx = rs.choice(n, 300, replace=False)
+    slots[idx] += rs.randint(-3000, 3000, 300)
+    slots = np.clip(slots, 0, lim - 1)
+    src, kt = to_dev(keys)
+    ds = torch.from_numpy(slots.astype(np.uint32).view(np.int32)).cuda()
+    order = torch.from_numpy(np.argsort(keys, kind="stable").astype(np.int32)).cuda()
+    want = src[order.long()]
+    for _ in range(24):
+        dk, pay = src.clone(), torch.arange(n, dtype=torch.int32, device="cuda")
+        st, _ = nns.sort(dk, pay, None, slots=ds, eps=3, tau=0, fate=True, key_type=kt, bucket_log2=9)
+        assert st["repair_ranges"] > 200
+        assert torch.equal(dk, want) and torch.equal(pay, order)
